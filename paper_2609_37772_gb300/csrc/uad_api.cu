@@ -35,7 +35,7 @@ struct LayerW {
   Lin wd;                // ADARMS [W][F]
   Lin wqc;               // DiT [Hq dh][W]
   Lin woc;               // DiT [W][Hq dh]
-  void* wkc = nullptr;   // DiT [Hq dh][Pw] (used once per observation)
+  void* wkc = nullptr;   // DiT [Hq dh][Pw] (once per observation; null when w_pkv holds it)
   void* wvc = nullptr;   // DiT [Hq dh][Pw]
   Lin w1;                // DiT [F][W]
   Lin w2;                // DiT [W][F]
@@ -90,6 +90,9 @@ struct uad_ctx {
   void* w_in = nullptr; float* b_in = nullptr;   // [W][D]
   void* w_out = nullptr; float* b_out = nullptr; // [D][W]
   Lin w_out_tc;                                  // the same padded to 128 rows, tiled (tensor cores)
+  Lin w_pkv;                                     // DiT on the tensor cores: prefix projections, rows
+                                                 // [layer][k, v][Hq dh], K = prefix_width
+  void* pre_tok = nullptr;                       // its input: one robot's prefix tokens [P][Pw] bf16
   void* w_mod = nullptr; float* b_mod = nullptr; // [rowlen][W], all layers' modulation + final
   // time-concatenating expert (UAD_KIND_CONCAT): input MLP; e(tau) W_it + b_it sits in the table
   void* w_it = nullptr; float* b_it = nullptr;   // [W][W] (table fill)
@@ -948,6 +951,14 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
     TRY(mklin(&c->w_out_tc, 128, W));
     if (c->w_out_tc.tiled) put("out_w", c->w_out_tc, 1, 0);
   }
+  // DiT prefix projections: all layers' K and V in one tensor-core weight
+  const bool pkv_tc = a.kind == UAD_KIND_DIT && a.n_layers > 0 && dt == BF16 && !c->force_simt && c->qd % 128 == 0 &&
+                      a.prefix_width % 64 == 0;
+  if (pkv_tc) {
+    TRY(mklin(&c->w_pkv, a.n_layers * 2 * c->qd, a.prefix_width));
+    TRY(dalloc(c, &c->pre_tok, (size_t)a.prefix_len * a.prefix_width * es));
+    TRY(make_tmap(c, c->pre_tok, a.prefix_width, a.prefix_len));
+  }
   for (int l = 0; l < a.n_layers; ++l) {
     const std::string p = "l" + std::to_string(l) + ".";
     LayerW& w = c->L[l];
@@ -964,8 +975,13 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
     } else {
       TRY(mklin(&w.wqc, c->qd, W)); put(p + "wqc", w.wqc, 1, 0);
       TRY(mklin(&w.woc, W, c->qd)); put(p + "woc", w.woc, 1, 0);
-      TRY(dalloc(c, &w.wkc, (size_t)c->qd * a.prefix_width * es)); lin(p + "wkc", w.wkc, 1, 0);
-      TRY(dalloc(c, &w.wvc, (size_t)c->qd * a.prefix_width * es)); lin(p + "wvc", w.wvc, 1, 0);
+      if (pkv_tc) {
+        put(p + "wkc", c->w_pkv, 1, (long long)(2 * l) * c->qd);
+        put(p + "wvc", c->w_pkv, 1, (long long)(2 * l + 1) * c->qd);
+      } else {
+        TRY(dalloc(c, &w.wkc, (size_t)c->qd * a.prefix_width * es)); lin(p + "wkc", w.wkc, 1, 0);
+        TRY(dalloc(c, &w.wvc, (size_t)c->qd * a.prefix_width * es)); lin(p + "wvc", w.wvc, 1, 0);
+      }
       TRY(mklin(&w.w1, F, W)); put(p + "w1", w.w1, 1, 0);
       TRY(mklin(&w.w2, W, F)); put(p + "w2", w.w2, 1, 0);
       TRY(vec(p + "b1", &w.b1)); TRY(vec(p + "b2", &w.b2));
@@ -1143,11 +1159,20 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
     const size_t n = (size_t)a.prefix_len * a.prefix_width;
     void *raw = nullptr, *tok = nullptr;
     if (cudaMalloc(&raw, n * ies) != cudaSuccess) return fail(c, UAD_ENOMEM, "prefix staging");
-    if (cudaMalloc(&tok, n * c->es) != cudaSuccess) { cudaFree(raw); return fail(c, UAD_ENOMEM, "prefix staging"); }
+    if (!c->pre_tok && cudaMalloc(&tok, n * c->es) != cudaSuccess) { cudaFree(raw); return fail(c, UAD_ENOMEM, "prefix staging"); }
     cudaMemcpyAsync(raw, k, n * ies, cudaMemcpyDefault, s);
-    launch_convert(raw, dtype, tok, a.dtype, (long long)n, s);
+    launch_convert(raw, dtype, c->pre_tok ? c->pre_tok : tok, a.dtype, (long long)n, s);
     const size_t per_layer = (size_t)a.prefix_len * c->qd;
-    for (int l = 0; l < a.n_layers; ++l) {
+    if (c->pre_tok) {
+      TcGemmArgs t;
+      t.w_tiled = c->w_pkv.w; t.M = a.prefix_len; t.N = c->w_pkv.N; t.K = a.prefix_width;
+      gemm_tc_prefix_plan(t.M, t.N, t.K, c->sms, &t);
+      t.epi = EPI_PREFIX_KV; t.out_dtype = BF16; t.err = c->dev_err;
+      const size_t base = (size_t)robot * a.n_layers * per_layer;
+      t.pkv = {static_cast<__nv_bfloat16*>(c->kpre) + base, static_cast<__nv_bfloat16*>(c->vpre) + base, c->qd};
+      launch_gemm_tc(&c->tmaps.at(c->pre_tok), t, s);
+    }
+    for (int l = 0; l < a.n_layers && !c->pre_tok; ++l) {
       for (int which = 0; which < 2; ++which) {
         GemmArgs g;
         g.A = tok; g.lda = a.prefix_width; g.a_dtype = a.dtype;
@@ -1159,10 +1184,14 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
         launch_gemm_simt(g, s);
       }
     }
+    int derr = 0;
+    if (c->pre_tok) cudaMemcpyAsync(&c->status_host->derr, c->dev_err, 4, cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaStreamSynchronize(s);
+    if (c->pre_tok && e == cudaSuccess && (derr = c->status_host->derr)) cudaMemset(c->dev_err, 0, 4);
     cudaFree(raw);
     cudaFree(tok);
     if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(c, UAD_ECUDA, "prefix projection failed");
+    if (derr) return fail(c, UAD_ECUDA, "a wait of the prefix projection timed out (code %d)", derr);
   }
   c->has_prefix[robot] = 1;
   return UAD_OK;

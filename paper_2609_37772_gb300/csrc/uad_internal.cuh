@@ -46,6 +46,14 @@ enum Epi {
   EPI_PARTIAL = 6,     // tensor cores: K split s writes its fp32 tile to plane s of out [splits][M][N]
   EPI_QKV_TC = 5,      // q/k rows pair-interleaved per head: RoPE, then scatter q -> Q, k -> K cache,
                        // v -> Vt cache (tensor-core attention layouts, see attn_tc.cu)
+  EPI_PREFIX_KV = 7,   // DiT prefix projections of every layer at once: rows [layer][k, v][width]
+                       // scatter to the K and V prefix caches (bf16)
+};
+
+// Where the DiT prefix projection (EPI_PREFIX_KV) writes: k, v [L][tokens][width] of one robot.
+struct PrefixKvOut {
+  __nv_bfloat16 *k = nullptr, *v = nullptr;
+  int width = 0;                     // Hq dh, a multiple of 128: a weight tile lies in one k or v
 };
 
 // Where the QKV projection epilogue (EPI_QKV_TC) writes, and the RoPE table it uses.
@@ -166,6 +174,7 @@ struct TcGemmArgs {
   void* out = nullptr; int ldo = 0; int out_dtype = BF16;
   const float* bias = nullptr;
   QkvTcOut qkv;                    // EPI_QKV_TC
+  PrefixKvOut pkv;                 // EPI_PREFIX_KV
   int n_store = 0;                 // EPI_STORE: > 0: rows n >= n_store are padding (not stored, no bias)
   float* acc = nullptr;            // split-K accumulator [M][N] fp32, zero between launches
   int* counters = nullptr;         // split-K arrival counters per output tile, zero between launches
@@ -184,6 +193,7 @@ int gemm_tc_splits(int M, int N, int K, int sms, int epi);
 int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form serves this projection
 // The tile plan of one projection (wide form, tokens per tile, K splits) into a.
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a);
+void gemm_tc_prefix_plan(int M, int N, int K, int sms, TcGemmArgs* a);   // EPI_PREFIX_KV: no K splits
 void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
 // element (k, n) of src [K][N] -> row n' * mult + off, column k of the tiled bf16 layout (K cols),
 // where n' = n, or with rope_dh > 0 the head-local pair interleave (d, d + dh/2) -> (2d, 2d + 1)

@@ -697,3 +697,18 @@ def test_prefix_given_in_bf16(name):
             assert res["evals"] == ref["evals"]
     finally:
         ex.close()
+
+
+@pytest.mark.parametrize("prefix,robots", [(1, 1), (64, 2), (65, 1), (129, 1), (257, 1)])
+def test_dit_prefix_projection_lengths(prefix, robots):
+    """The tensor-core prefix projection at the edges of its forms: one token, exactly one 64-token
+    tile (the last length of the narrow form), one token more, and one past a 128- and a 256-token
+    tile; the second robot's caches follow the first's."""
+    a = ARCHS["dit_small"].replace(name=f"dit_small_p{prefix}", prefix_len=prefix)
+    c = Case(a, B=robots, seed=51)
+    try:
+        noise = make_noise(a, batch=robots, seed=51)
+        bud = np.stack([group_budgets(16, [(0, 3, 2), (4, 15, 3)])] * robots)
+        check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL["bf16"])
+    finally:
+        c.close()
