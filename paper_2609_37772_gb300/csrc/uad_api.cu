@@ -110,6 +110,8 @@ struct uad_ctx {
   float* pos_code = nullptr;   // [H][W] (DiT)
 
   // prefix
+  unsigned char* stage = nullptr;         // copies of prefixes given in host memory, grown on demand
+  size_t stage_cap = 0;
   void *kpre = nullptr, *vpre = nullptr;  // ADARMS [B][L][P][Hkv dh]; DiT [B][L][P][Hq dh]
   float* few_ws = nullptr;                // few-query attention: partial rows of the key chunks
   unsigned* few_ctr = nullptr;            // and their arrival counts (zero between launches)
@@ -200,6 +202,53 @@ int dalloc_t(uad_ctx* c, T** p, size_t count, size_t elem = sizeof(T)) {
   int r = dalloc(c, &q, count * elem);
   *p = static_cast<T*>(q);
   return r;
+}
+
+// Work on stream s after what the legacy default stream holds now (a prefix computed there, or on
+// a stream that synchronises with it, needs no wait by the caller). Not while a stream that blocks
+// with it is being captured: the wait would end that capture.
+int after_default_stream(uad_ctx* c, cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(cudaStreamLegacy, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return UAD_OK;
+  }
+  CK(cudaEventRecord(c->ev_in, cudaStreamLegacy));
+  CK(cudaStreamWaitEvent(s, c->ev_in, 0));
+  return UAD_OK;
+}
+
+// Staging memory at byte `off` of a buffer of at least `total` bytes. Kept for later calls; a call
+// that grows it must not have used it yet (every call asks for its own total each time).
+int stage_at(uad_ctx* c, size_t off, size_t total, void** out) {
+  if (c->stage_cap < total) {
+    if (c->stage) cudaFree(c->stage);
+    c->stage = nullptr;
+    c->stage_cap = 0;
+    if (cudaMalloc((void**)&c->stage, total) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(c, UAD_ENOMEM, "prefix staging");
+    }
+    c->stage_cap = total;
+  }
+  *out = c->stage + off;
+  return UAD_OK;
+}
+
+// A 16-byte aligned address on this device of the caller's buffer p: p itself, or a copy at byte
+// `off` of the staging buffer (host memory, another device's, or an address that is not aligned).
+int on_device(uad_ctx* c, const void* p, size_t bytes, size_t off, size_t total, cudaStream_t s, const void** out) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+  else if (at.type == cudaMemoryTypeDevice && at.device == c->dev && reinterpret_cast<uintptr_t>(p) % 16 == 0) {
+    *out = p;
+    return UAD_OK;
+  }
+  void* q = nullptr;
+  const int rc = stage_at(c, off, total, &q);
+  if (rc) return rc;
+  *out = q;
+  return cudaMemcpyAsync(q, p, bytes, cudaMemcpyDefault, s) == cudaSuccess ? UAD_OK : UAD_ECUDA;
 }
 
 std::vector<Tensor> blob_layout(const uad_arch& a) {
@@ -1119,49 +1168,55 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
   if (dtype != UAD_DTYPE_F32 && dtype != UAD_DTYPE_BF16) return fail(c, UAD_EINVAL, "dtype");
   if (!k) return fail(c, UAD_EINVAL, "null prefix");
   if (c->in_flight) return fail(c, UAD_ESTATE, "a chunk is in flight");
+  if (a.kind != UAD_KIND_DIT && !v) return fail(c, UAD_EINVAL, "null prefix values");
+  if (a.kind == UAD_KIND_DIT && v) return fail(c, UAD_EINVAL, "DiT takes prefix tokens in k and NULL v");
   const int ies = dtype == UAD_DTYPE_BF16 ? 2 : 4;
   cudaStream_t s = c->worker;
-  if (a.kind != UAD_KIND_DIT && c->attn_tc) {
-    if (!v) return fail(c, UAD_EINVAL, "null prefix values");
+  int rc = after_default_stream(c, s);
+  if (rc) return rc;
+  if (a.kind != UAD_KIND_DIT) {
     const size_t n = (size_t)a.n_layers * a.prefix_len * c->kvd;
-    void *tk = nullptr, *tv = nullptr;
-    if (cudaMalloc(&tk, n * ies) != cudaSuccess) return fail(c, UAD_ENOMEM, "prefix staging");
-    if (cudaMalloc(&tv, n * ies) != cudaSuccess) { cudaFree(tk); return fail(c, UAD_ENOMEM, "prefix staging"); }
-    int rc = UAD_OK;
-    if (cudaMemcpyAsync(tk, k, n * ies, cudaMemcpyDefault, s) != cudaSuccess ||
-        cudaMemcpyAsync(tv, v, n * ies, cudaMemcpyDefault, s) != cudaSuccess)
-      rc = UAD_ECUDA;
-    else
-      launch_kv_prefix(tk, tv, dtype, c->at0, robot, s);
-    cudaError_t e = cudaStreamSynchronize(s);
-    cudaFree(tk);
-    cudaFree(tv);
-    if (rc != UAD_OK || e != cudaSuccess || cudaGetLastError() != cudaSuccess)
-      return fail(c, UAD_ECUDA, "prefix upload failed");
-  } else if (a.kind != UAD_KIND_DIT) {
-    if (!v) return fail(c, UAD_EINVAL, "null prefix values");
-    const size_t n = (size_t)a.n_layers * a.prefix_len * c->kvd;
-    void* tmp = nullptr;
-    if (cudaMalloc(&tmp, n * ies) != cudaSuccess) return fail(c, UAD_ENOMEM, "prefix staging");
-    int rc = UAD_OK;
-    for (int which = 0; which < 2 && rc == UAD_OK; ++which) {
-      const void* srcp = which ? v : k;
-      void* dst = static_cast<char*>(which ? c->vpre : c->kpre) + (size_t)robot * n * c->es;
-      if (cudaMemcpyAsync(tmp, srcp, n * ies, cudaMemcpyDefault, s) != cudaSuccess) rc = UAD_ECUDA;
-      else launch_convert(tmp, dtype, dst, a.dtype, (long long)n, s);
+    if (!c->attn_tc && dtype == a.dtype) {
+      // the caches keep the caller's layout
+      if (cudaMemcpyAsync(static_cast<char*>(c->kpre) + (size_t)robot * n * c->es, k, n * ies, cudaMemcpyDefault, s) != cudaSuccess ||
+          cudaMemcpyAsync(static_cast<char*>(c->vpre) + (size_t)robot * n * c->es, v, n * ies, cudaMemcpyDefault, s) != cudaSuccess)
+        rc = UAD_ECUDA;
+    } else {
+      const size_t half = (n * ies + 15) & ~(size_t)15;
+      const void *dk = nullptr, *dv = nullptr;
+      rc = on_device(c, k, n * ies, 0, 2 * half, s, &dk);
+      if (!rc) rc = on_device(c, v, n * ies, half, 2 * half, s, &dv);
+      if (!rc && c->attn_tc) launch_kv_prefix(dk, dv, dtype, c->at0, robot, s);
+      for (int which = 0; which < 2 && !rc && !c->attn_tc; ++which)
+        launch_convert(which ? dv : dk, dtype, static_cast<char*>(which ? c->vpre : c->kpre) + (size_t)robot * n * c->es,
+                       a.dtype, (long long)n, s);
     }
-    cudaError_t e = cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (rc == UAD_ENOMEM) return rc;
     if (rc != UAD_OK || e != cudaSuccess || cudaGetLastError() != cudaSuccess)
       return fail(c, UAD_ECUDA, "prefix upload failed");
   } else {
-    if (v) return fail(c, UAD_EINVAL, "DiT takes prefix tokens in k and NULL v");
     const size_t n = (size_t)a.prefix_len * a.prefix_width;
-    void *raw = nullptr, *tok = nullptr;
-    if (cudaMalloc(&raw, n * ies) != cudaSuccess) return fail(c, UAD_ENOMEM, "prefix staging");
-    if (!c->pre_tok && cudaMalloc(&tok, n * c->es) != cudaSuccess) { cudaFree(raw); return fail(c, UAD_ENOMEM, "prefix staging"); }
-    cudaMemcpyAsync(raw, k, n * ies, cudaMemcpyDefault, s);
-    launch_convert(raw, dtype, c->pre_tok ? c->pre_tok : tok, a.dtype, (long long)n, s);
+    const size_t half = (n * ies + 15) & ~(size_t)15;
+    const void* tok = c->pre_tok;
+    if (c->pre_tok && dtype == a.dtype) {
+      if (cudaMemcpyAsync(c->pre_tok, k, n * ies, cudaMemcpyDefault, s) != cudaSuccess) rc = UAD_ECUDA;
+    } else {
+      const void* raw = nullptr;
+      rc = on_device(c, k, n * ies, 0, half + (c->pre_tok ? 0 : n * c->es), s, &raw);
+      if (!rc && dtype == a.dtype) {
+        tok = raw;
+      } else if (!rc) {
+        void* dst = c->pre_tok;
+        if (!dst) rc = stage_at(c, half, half + n * c->es, &dst);
+        if (!rc) launch_convert(raw, dtype, dst, a.dtype, (long long)n, s);
+        tok = dst;
+      }
+    }
+    if (rc) {
+      cudaStreamSynchronize(s);
+      return rc == UAD_ENOMEM ? rc : fail(c, UAD_ECUDA, "prefix upload failed");
+    }
     const size_t per_layer = (size_t)a.prefix_len * c->qd;
     if (c->pre_tok) {
       TcGemmArgs t;
@@ -1188,8 +1243,6 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
     if (c->pre_tok) cudaMemcpyAsync(&c->status_host->derr, c->dev_err, 4, cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (c->pre_tok && e == cudaSuccess && (derr = c->status_host->derr)) cudaMemset(c->dev_err, 0, 4);
-    cudaFree(raw);
-    cudaFree(tok);
     if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(c, UAD_ECUDA, "prefix projection failed");
     if (derr) return fail(c, UAD_ECUDA, "a wait of the prefix projection timed out (code %d)", derr);
   }
@@ -1558,6 +1611,7 @@ void uad_destroy(uad_ctx* c) {
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   if (c->ev_done) cudaEventDestroy(c->ev_done);
   for (void* p : c->allocs) cudaFree(p);
+  if (c->stage) cudaFree(c->stage);
   if (c->plan_host) cudaFreeHost(c->plan_host);
   if (c->status_host) cudaFreeHost(c->status_host);
   if (c->host_rel) cudaFreeHost(c->host_rel);

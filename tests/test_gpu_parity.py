@@ -712,3 +712,35 @@ def test_dit_prefix_projection_lengths(prefix, robots):
         check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL["bf16"])
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("prefix", [1, 63, 64, 72, 129])
+def test_prefix_transposition_lengths(prefix):
+    """Prefix keys and values into the attention caches at the edges of the 64-position tiles and of
+    the runs of eight keys, from device memory read in place (16-byte aligned) and from an address
+    that is not aligned (copied first), in both element types."""
+    a = ARCHS["pi0_small"].replace(name=f"pi0_small_p{prefix}", prefix_len=prefix)
+    blob = make_weights(a, seed=52)
+    pre = make_prefix_kv(a, seed=52)
+    noise = make_noise(a, seed=52)
+    bud = group_budgets(a.chunk_len, [(0, 3, 2), (4, a.chunk_len - 1, 3)])
+    ref = denoise(build_model(a, blob, pre).velocity, noise[0], bud)
+    ex = uad.Expert(a, blob)
+
+    def placed(x, dtype, shift):
+        buf = torch.zeros(x.size + 8, dtype=dtype, device="cuda")
+        view = buf[shift:shift + x.size].view(x.shape)
+        view.copy_(torch.from_numpy(x))
+        return view
+
+    try:
+        for name, dtype, shift in (("f32", torch.float32, 0), ("f32", torch.float32, 1),
+                                   ("bf16", torch.bfloat16, 0), ("bf16", torch.bfloat16, 3)):
+            ex.set_prefix(0, *[placed(np.zeros_like(p), dtype, shift) for p in pre], dtype=name)   # nothing stays behind
+            ex.set_prefix(0, *[placed(p, dtype, shift) for p in pre], dtype=name)
+            ex.denoise(noise, bud[None])
+            res = ex.finish(timeout_us=TIMEOUT)
+            assert rel_err(res["final"][0], ref["final"]) <= TOL["bf16"], (name, shift)
+            assert rel_err(res["ghost"][0], ref["ghost"]) <= TOL["bf16"]
+    finally:
+        ex.close()
