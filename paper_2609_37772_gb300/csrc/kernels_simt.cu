@@ -1,5 +1,5 @@
-// CUDA-core kernels: fp32-FFMA GEMM (the fp32 mode and one-time table fills), adaptive
-// norms, attention over prefix + chunk, and the Euler / TR / release / GAC step epilogue.
+// CUDA-core kernels: projections with a tiny side, adaptive norms, attention for few queries, and
+// the Euler / TR / release / GAC step epilogue. (GEMM and general attention: ffma.cu.)
 #include "uad_internal.cuh"
 #include "euler.cuh"
 
@@ -50,85 +50,6 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// ------------------------------------------------------------------------------------------
-// GEMM: out[m][n] = epi(sum_k A[m][k] * Wt[n][k]); 64x64 tile, 4x4 outputs per thread, k in
-// ascending order (deterministic).
-// ------------------------------------------------------------------------------------------
-template <int AD, int WD>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs p) {
-  __shared__ float As[32][68];
-  __shared__ float Ws[32][68];
-  pdl_trigger();
-  pdl_wait();
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < p.K; k0 += 32) {
-    for (int e = tid; e < 64 * 32; e += 256) {
-      const int r = e >> 5, c = e & 31, k = k0 + c;
-      const int m = m0 + r, n = n0 + r;
-      As[c][r] = (m < p.M && k < p.K) ? ldf<AD>(p.A, (long long)m * p.lda + k) : 0.f;
-      Ws[c][r] = (n < p.N && k < p.K) ? ldf<WD>(p.W, (long long)n * p.K + k) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      float a[4], w[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = Ws[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= p.M) continue;
-    if (p.epi == EPI_GEGLU) {
-#pragma unroll
-      for (int jp = 0; jp < 2; ++jp) {
-        const int n = n0 + tx * 4 + 2 * jp;
-        if (n + 1 < p.N)
-          stf(p.out, (long long)m * p.ldo + n / 2, gelu_tanh(acc[i][2 * jp]) * acc[i][2 * jp + 1],
-              p.out_dtype);
-      }
-      continue;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= p.N) continue;
-      float r = acc[i][j] + (p.bias ? p.bias[n] : 0.f);
-      switch (p.epi) {
-        case EPI_STORE:
-          if (p.add_rows) r += p.add_rows[(long long)(m % p.add_mod) * p.N + n];
-          stf(p.out, (long long)m * p.ldo + n, r, p.out_dtype);
-          break;
-        case EPI_BIAS_SILU: stf(p.out, (long long)m * p.ldo + n, silu(r), p.out_dtype); break;
-        case EPI_BIAS_GELU: stf(p.out, (long long)m * p.ldo + n, gelu_tanh(r), p.out_dtype); break;
-        case EPI_RESID_GATE: {
-          const float gt = p.gate_tab ? p.gate_tab[(long long)p.tau_row[m] * p.gate_stride + n] : 1.f;
-          float* dst = p.resid + (long long)m * p.ldr + n;
-          *dst = fmaf(gt, r, *dst);
-          break;
-        }
-        default: break;
-      }
-    }
-  }
-}
-
 // Projections with a tiny side (action in: K = D; action out: N = D): one CTA per token row m,
 // the row staged in shared memory, then one warp per output (long K) or one thread per output
 // (short K). out[m][n] = sum_k A[m][k] Wt[n][k] + bias[n] (+ add_rows[m % add_mod][n]), fp32.
@@ -168,14 +89,6 @@ void launch_gemv_rows(const GemmArgs& a, cudaStream_t s) {
   else if (a.a_dtype == F32 && a.w_dtype == BF16) launch_k(gemv_rows_kernel<F32, BF16>, dim3(a.M), dim3(256), 0, s, a);
   else if (a.a_dtype == BF16 && a.w_dtype == BF16) launch_k(gemv_rows_kernel<BF16, BF16>, dim3(a.M), dim3(256), 0, s, a);
   else launch_k(gemv_rows_kernel<BF16, F32>, dim3(a.M), dim3(256), 0, s, a);
-}
-
-void launch_gemm_simt(const GemmArgs& a, cudaStream_t s) {
-  dim3 grid((a.N + 63) / 64, (a.M + 63) / 64);
-  if (a.a_dtype == F32 && a.w_dtype == F32) launch_k(gemm_simt_kernel<F32, F32>, grid, dim3(256), 0, s, a);
-  else if (a.a_dtype == F32 && a.w_dtype == BF16) launch_k(gemm_simt_kernel<F32, BF16>, grid, dim3(256), 0, s, a);
-  else if (a.a_dtype == BF16 && a.w_dtype == BF16) launch_k(gemm_simt_kernel<BF16, BF16>, grid, dim3(256), 0, s, a);
-  else launch_k(gemm_simt_kernel<BF16, F32>, grid, dim3(256), 0, s, a);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -460,13 +373,6 @@ void launch_norm(const NormArgs& a, cudaStream_t s) {
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Attention of chunk queries over [prefix keys ; chunk keys] with grouped KV heads,
-// online softmax in fp32. CTA = (16 queries, one query head, one robot); warp = 4 queries;
-// lane = one key of a 32-key block for the scores, 32-strided head dims for the output.
-// ------------------------------------------------------------------------------------------
-constexpr int AQ = 16, AKB = 32;
-
 __device__ __forceinline__ float rope_elem(const void* base, long long off, int d, int half,
                                            const float* cs, int dt) {
   const float x = ldf_rt(base, off + d, dt);
@@ -474,97 +380,6 @@ __device__ __forceinline__ float rope_elem(const void* base, long long off, int 
   const float c = cs[2 * j], s = cs[2 * j + 1];
   const float o = ldf_rt(base, off + (d < half ? d + half : d - half), dt);
   return d < half ? x * c - o * s : x * c + o * s;
-}
-
-template <int DPL>
-__global__ void __launch_bounds__(128) attn_kernel(AttnArgs p) {
-  extern __shared__ float sm[];
-  pdl_trigger();
-  pdl_wait();
-  const int dh = DPL * 32, half = dh / 2;
-  float* qs = sm;                   // [AQ][dh]
-  float* ks = qs + AQ * dh;         // [AKB][dh + 1]
-  float* vs = ks + AKB * (dh + 1);  // [AKB][dh]
-  float* ps = vs + AKB * dh;        // [AQ][AKB]
-  const int b = blockIdx.z, hq = blockIdx.y, i0 = blockIdx.x * AQ;
-  const int g = hq / (p.n_heads / p.n_kv_heads);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  for (int e = tid; e < AQ * dh; e += 128) {
-    const int qi = e / dh, d = e % dh, i = i0 + qi;
-    float val = 0.f;
-    if (i < p.H) {
-      const long long off = (long long)(b * p.H + i) * p.q_ld + hq * dh;
-      val = p.rope_cs ? rope_elem(p.q, off, d, half, p.rope_cs + (long long)i * dh, p.dtype)
-                      : ldf_rt(p.q, off + d, p.dtype);
-    }
-    qs[qi * dh + d] = val * p.scale;
-  }
-
-  float m_run[4], l_run[4], o[4][DPL];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    m_run[q] = -INFINITY;
-    l_run[q] = 0.f;
-#pragma unroll
-    for (int t = 0; t < DPL; ++t) o[q][t] = 0.f;
-  }
-  const int n_keys = p.P + (p.kc ? p.H : 0);
-  for (int j0 = 0; j0 < n_keys; j0 += AKB) {
-    __syncthreads();
-    for (int e = tid; e < AKB * dh; e += 128) {
-      const int jj = e / dh, d = e % dh, j = j0 + jj;
-      float kv = 0.f, vv = 0.f;
-      if (j < p.P) {
-        const long long off = b * p.kp_bstride + (long long)j * p.kp_ld + g * dh;
-        kv = ldf_rt(p.kp, off + d, p.dtype);
-        vv = ldf_rt(p.vp, off + d, p.dtype);
-      } else if (j < n_keys) {
-        const int i = j - p.P;
-        const long long off = (long long)(b * p.H + i) * p.kc_ld + g * dh;
-        kv = p.rope_cs ? rope_elem(p.kc, off, d, half, p.rope_cs + (long long)i * dh, p.dtype)
-                       : ldf_rt(p.kc, off + d, p.dtype);
-        vv = ldf_rt(p.vc, off + d, p.dtype);
-      }
-      ks[jj * (dh + 1) + d] = kv;
-      vs[jj * dh + d] = vv;
-    }
-    __syncthreads();
-    const bool valid = j0 + lane < n_keys;
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-      const int q = warp * 4 + qq;
-      float s = 0.f;
-      for (int d = 0; d < dh; ++d) s = fmaf(qs[q * dh + d], ks[lane * (dh + 1) + d], s);
-      s = valid ? s : -INFINITY;
-      const float m_new = fmaxf(m_run[qq], warp_max(s));
-      const float pe = valid ? expf(s - m_new) : 0.f;
-      const float alpha = m_run[qq] == -INFINITY ? 0.f : expf(m_run[qq] - m_new);
-      l_run[qq] = l_run[qq] * alpha + warp_sum(pe);
-      m_run[qq] = m_new;
-      ps[q * AKB + lane] = pe;
-#pragma unroll
-      for (int t = 0; t < DPL; ++t) o[qq][t] *= alpha;
-    }
-    __syncwarp();
-    for (int jj = 0; jj < AKB; ++jj) {
-#pragma unroll
-      for (int t = 0; t < DPL; ++t) {
-        const float vv = vs[jj * dh + lane + 32 * t];
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) o[qq][t] = fmaf(ps[(warp * 4 + qq) * AKB + jj], vv, o[qq][t]);
-      }
-    }
-  }
-#pragma unroll
-  for (int qq = 0; qq < 4; ++qq) {
-    const int i = i0 + warp * 4 + qq;
-    if (i >= p.H) continue;
-    const float inv = 1.f / l_run[qq];
-#pragma unroll
-    for (int t = 0; t < DPL; ++t)
-      stf(p.out, (long long)(b * p.H + i) * p.out_ld + hq * dh + lane + 32 * t, o[qq][t] * inv, p.dtype);
-  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -783,38 +598,13 @@ void launch_add_tau_silu(const float* x, const float* tab, int stride, int off, 
   launch_k(add_tau_silu_kernel, dim3(blocks), dim3(256), 0, s, x, tab, stride, off, tau_row, M, N, y, dt);
 }
 
-template <int DPL>
-static void launch_attn_dpl(const AttnArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-  launch_k(attn_kernel<DPL>, grid, dim3(128), smem, s, a);
-}
-
-size_t attention_smem_bytes(int dh) {
-  return sizeof(float) * (AQ * dh + AKB * (dh + 1) + AKB * dh + AQ * AKB);
-}
-
-void launch_attention_prepare(int dh) {
-  const int smem = (int)attention_smem_bytes(dh);
-  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (dh == 64) cudaFuncSetAttribute(attn_kernel<2>, at, smem);
-  if (dh == 128) cudaFuncSetAttribute(attn_kernel<4>, at, smem);
-  if (dh == 256) cudaFuncSetAttribute(attn_kernel<8>, at, smem);
-}
-
 void launch_attention(const AttnArgs& a, cudaStream_t s) {
-  const int dh = a.head_dim;
   if (attn_few_ok(a)) {
     const int n_keys = a.P + (a.kc ? a.H : 0);
     launch_k(attn_few_kernel, dim3(((a.H + kFewQ - 1) / kFewQ) * few_chunks(n_keys), a.n_heads, a.B), dim3(256), 0, s, a);
     return;
   }
-  const size_t smem = attention_smem_bytes(dh);
-  dim3 grid((a.H + AQ - 1) / AQ, a.n_heads, a.B);
-  switch (dh) {
-    case 64: launch_attn_dpl<2>(a, grid, smem, s); break;
-    case 128: launch_attn_dpl<4>(a, grid, smem, s); break;
-    case 256: launch_attn_dpl<8>(a, grid, smem, s); break;
-    default: break;  // rejected at init
-  }
+  launch_attn_rows(a, s);
 }
 
 // ------------------------------------------------------------------------------------------

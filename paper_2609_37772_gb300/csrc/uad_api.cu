@@ -342,19 +342,19 @@ int fill_times(uad_ctx* c, const std::vector<std::pair<int, int>>& fr, cudaStrea
   GemmArgs g;
   g.A = c->temb; g.lda = W; g.a_dtype = F32; g.W = c->t_w1; g.w_dtype = c->a.dtype;
   g.M = n; g.N = W; g.K = W; g.epi = EPI_BIAS_SILU; g.out = c->tc1; g.ldo = W; g.bias = c->t_b1;
-  launch_gemm_simt(g, s);
+  launch_gemm_ffma(g, s);
   g.A = c->tc1; g.W = c->t_w2; g.out = c->tc2; g.bias = c->t_b2;
-  launch_gemm_simt(g, s);
+  launch_gemm_ffma(g, s);
   g.A = c->tc2; g.W = c->w_mod; g.N = c->rowlen; g.epi = EPI_STORE; g.bias = c->b_mod;
   g.out = c->tab + (size_t)c->tab_rows * c->rowlen; g.ldo = c->rowlen;
-  launch_gemm_simt(g, s);
+  launch_gemm_ffma(g, s);
   if (c->a.kind == UAD_KIND_CONCAT) {
     // the time half of the input MLP: e(tau) W_it + b_it after the (constant) modulation
     GemmArgs t;
     t.A = c->temb; t.lda = W; t.a_dtype = F32; t.W = c->w_it; t.w_dtype = c->a.dtype;
     t.M = n; t.N = W; t.K = W; t.epi = EPI_STORE; t.bias = c->b_it;
     t.out = c->tab + (size_t)c->tab_rows * c->rowlen + concat_off(c); t.ldo = c->rowlen;
-    launch_gemm_simt(t, s);
+    launch_gemm_ffma(t, s);
   }
   CK(cudaGetLastError());
   for (int r = 0; r < n; ++r) c->tau_row[fr[r]] = c->tab_rows + r;
@@ -459,7 +459,7 @@ void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
     // action-in projection of a batch) goes to the tiled kernel, which reuses each weight tile
     // over 64 rows
     if (gemv_rows_ok(g) && (g.K > 64 || g.M <= 64)) launch_gemv_rows(g, s);
-    else launch_gemm_simt(g, s);
+    else launch_gemm_ffma(g, s);
     return;
   }
   TcGemmArgs t;
@@ -1149,8 +1149,8 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
   CK(cudaStreamCreateWithFlags(&c->worker, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&c->ev_done, cudaEventDisableTiming));
-  // attention kernels need more than 48 KB of dynamic shared memory: opt in once, here
-  launch_attention_prepare(a.head_dim);
+  // kernels with more than 48 KB of dynamic shared memory: opt in once, here
+  ffma_prepare(a.head_dim);
   launch_euler_prepare();
   CK(cudaDeviceSynchronize());
   CK(cudaGetLastError());
@@ -1236,7 +1236,7 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
         g.out = static_cast<char*>(which ? c->vpre : c->kpre) +
                 ((size_t)robot * a.n_layers * per_layer + (size_t)l * per_layer) * c->es;
         g.ldo = c->qd;
-        launch_gemm_simt(g, s);
+        launch_gemm_ffma(g, s);
       }
     }
     int derr = 0;

@@ -144,7 +144,6 @@ struct EulerArgs {
 
 // kernels_simt.cu
 constexpr int kGemvMaxK = 8192;
-void launch_gemm_simt(const GemmArgs& a, cudaStream_t s);
 bool gemv_rows_ok(const GemmArgs& a);                     // tiny-side projection (N or K <= 64)
 void launch_gemv_rows(const GemmArgs& a, cudaStream_t s);
 void launch_norm(const NormArgs& a, cudaStream_t s);   // applies the pending residual if part != null
@@ -156,14 +155,17 @@ void launch_begin(const float* noise, float* x, float* g, float* u, int n, int* 
 // dst[(n * mult + off) * K + k] = src[k * N + n]: transpose [K][N] -> rows of K, convert dtype
 void launch_relayout(const float* src, int K, int N, void* dst, int dtype, int mult, long long off,
                      cudaStream_t s);
-size_t attention_smem_bytes(int dh);
-void launch_attention_prepare(int dh);  // opt in to > 48 KB dynamic shared memory (call once)
 void launch_convert(const void* src, int src_dtype, void* dst, int dst_dtype, long long n, cudaStream_t s);
 void launch_so3_check(const float* w, int n, float* log_exp, float* log_comp, cudaStream_t s);
 // y[m][n] = SiLU(x[m][n] + tab[tau_row[m] * stride + off + n]) in dtype dt (the input MLP of the
 // time-concatenating expert: the table holds e(tau) W_it + b_it per flow time)
 void launch_add_tau_silu(const float* x, const float* tab, int stride, int off, const int* tau_row, int M, int N,
                          void* y, int dt, cudaStream_t s);
+
+// ffma.cu: CUDA-core GEMM and attention
+void launch_gemm_ffma(const GemmArgs& a, cudaStream_t s);
+void launch_attn_rows(const AttnArgs& a, cudaStream_t s);
+void ffma_prepare(int head_dim);   // opt in to > 48 KB dynamic shared memory on the current device
 
 // gemm_tc.cu: tcgen05 projection GEMM (bf16 operands, fp32 accumulation in TMEM)
 constexpr int kTcMaxStages = 4;        // <= ~97 KB of shared memory: two CTAs fit one SM

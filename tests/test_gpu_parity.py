@@ -744,3 +744,28 @@ def test_prefix_transposition_lengths(prefix):
             assert rel_err(res["ghost"][0], ref["ghost"]) <= TOL["bf16"]
     finally:
         ex.close()
+
+
+@pytest.mark.parametrize("dtype,dh,heads,kv,width,mlp,chunk,prefix,rope,robots", [
+    ("f32", 64, 4, 4, 96, 333, 5, 58, False, 1),       # 16-row tiles; K = 333 (scalar loads, two chunks), 63 keys
+    ("f32", 64, 4, 2, 288, 1030, 17, 47, True, 1),     # one row past a tile, 64 keys, chunk keys rotated in place
+    ("f32", 64, 4, 4, 256, 1024, 16, 49, False, 9),    # 32-row tiles, 65 keys
+    ("f32", 64, 2, 1, 160, 2112, 33, 0, True, 16),     # 64-row tiles with a ragged edge, no prefix
+    ("f32", 128, 2, 2, 64, 96, 3, 31, False, 1),       # 34 keys: one past a 32-key tile and one more
+    ("f32", 256, 3, 1, 128, 64, 9, 96, True, 2),
+    ("f32", 64, 4, 4, 64, 64, 40, 200, False, 16),     # two queries a warp
+    ("bf16", 128, 3, 3, 96, 328, 7, 40, False, 2),     # bf16 weights outside the tensor-core layout
+    ("bf16", 256, 1, 1, 160, 72, 20, 45, True, 3),
+])
+def test_cuda_core_gemm_and_attention_edges(dtype, dh, heads, kv, width, mlp, chunk, prefix, rope, robots):
+    """The CUDA-core GEMM at the edges of its three tiles (rows, columns and K) and the general
+    attention at the edges of its key tiles, in the types and head dims they serve."""
+    a = ARCHS["tiny"].replace(name="edges", dtype=dtype, n_layers=1, width=width, n_heads=heads, n_kv_heads=kv,
+                              head_dim=dh, mlp_dim=mlp, chunk_len=chunk, prefix_len=prefix, rope=rope)
+    c = Case(a, B=robots, seed=53)
+    try:
+        noise = make_noise(a, batch=robots, seed=53)
+        bud = np.stack([group_budgets(chunk, [(0, 1, 1), (2, chunk - 1, 2)])] * robots)
+        check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL[dtype])
+    finally:
+        c.close()
