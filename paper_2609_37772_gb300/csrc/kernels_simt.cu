@@ -50,9 +50,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Projections with a tiny side (action in: K = D; action out: N = D): one CTA per token row m,
-// the row staged in shared memory, then one warp per output (long K) or one thread per output
-// (short K). out[m][n] = sum_k A[m][k] Wt[n][k] + bias[n] (+ add_rows[m % add_mod][n]), fp32.
+// Projections with a tiny side (action in: K = D; action out: N = D), fp32 out:
+// out[m][n] = sum_k A[m][k] Wt[n][k] + bias[n] (+ add_rows[m % add_mod][n]). Long K: one CTA per token row,
+// the row staged in shared memory, one warp per output.
 template <int AD, int WD>
 __global__ void __launch_bounds__(256) gemv_rows_kernel(GemmArgs p) {
   __shared__ float a_s[kGemvMaxK];
@@ -63,20 +63,70 @@ __global__ void __launch_bounds__(256) gemv_rows_kernel(GemmArgs p) {
   __syncthreads();
   float* out = static_cast<float*>(p.out) + (long long)m * p.ldo;
   const float* add = p.add_rows ? p.add_rows + (long long)(m % p.add_mod) * p.N : nullptr;
-  if (p.K <= 64) {
-    for (int n = tid; n < p.N; n += 256) {
-      float acc = 0.f;
-      for (int k = 0; k < p.K; ++k) acc = fmaf(a_s[k], ldf<WD>(p.W, (long long)n * p.K + k), acc);
-      out[n] = acc + (p.bias ? p.bias[n] : 0.f) + (add ? add[n] : 0.f);
-    }
-  } else {
-    for (int n = warp; n < p.N; n += 8) {
-      float acc = 0.f;
+  for (int n = warp; n < p.N; n += 8) {
+    float acc = 0.f;
 #pragma unroll 8
-      for (int k = lane; k < p.K; k += 32) acc = fmaf(a_s[k], ldf<WD>(p.W, (long long)n * p.K + k), acc);
-      acc = warp_sum(acc);
-      if (lane == 0) out[n] = acc + (p.bias ? p.bias[n] : 0.f) + (add ? add[n] : 0.f);
+    for (int k = lane; k < p.K; k += 32) acc = fmaf(a_s[k], ldf<WD>(p.W, (long long)n * p.K + k), acc);
+    acc = warp_sum(acc);
+    if (lane == 0) out[n] = acc + (p.bias ? p.bias[n] : 0.f) + (add ? add[n] : 0.f);
+  }
+}
+
+// Short K (at most 64): a thread keeps the weights of one output in registers, read before the wait for
+// the kernel that writes A, and a CTA of 256 outputs walks `rows` token rows staged in shared memory.
+// Bound by the bytes out; one CTA a row re-read every weight for each row.
+template <int AD, int WD>
+__global__ void __launch_bounds__(256) short_k_kernel(GemmArgs p, int rows) {
+  constexpr int KM = 64, RM = 16;
+  __shared__ float a_s[RM * KM];
+  pdl_trigger();
+  const int n = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * rows, K = p.K;
+  const int cnt = p.M - m0 < rows ? p.M - m0 : rows;
+  float w[KM], b = 0.f;
+#pragma unroll
+  for (int k = 0; k < KM; ++k) w[k] = 0.f;
+  if (n < p.N) {
+    if (WD == BF16 && K % 8 == 0) {   // rows of W are 16-byte aligned then
+#pragma unroll
+      for (int k = 0; k < KM; k += 8) {
+        if (k >= K) break;
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.W) + (long long)n * K + k));
+        const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 f = __bfloat1622float2(v2[q]);
+          w[k + 2 * q] = f.x;
+          w[k + 2 * q + 1] = f.y;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        if (k >= K) break;
+        w[k] = ldf<WD>(p.W, (long long)n * K + k);
+      }
     }
+    if (p.bias) b = p.bias[n];
+  }
+  pdl_wait();
+  for (int e = threadIdx.x; e < cnt * KM; e += 256) {
+    const int r = e / KM, k = e % KM;
+    a_s[e] = k < K ? ldf<AD>(p.A, (long long)(m0 + r) * p.lda + k) : 0.f;
+  }
+  __syncthreads();
+  if (n >= p.N) return;
+  float* out = static_cast<float*>(p.out) + n;
+  const int k4 = (K + 3) / 4;
+  for (int r = 0; r < cnt; ++r) {
+    float acc = 0.f;
+#pragma unroll
+    for (int q = 0; q < KM / 4; ++q) {
+      if (q >= k4) break;
+      const float4 a = *reinterpret_cast<const float4*>(a_s + r * KM + 4 * q);
+      acc = fmaf(a.w, w[4 * q + 3], fmaf(a.z, w[4 * q + 2], fmaf(a.y, w[4 * q + 1], fmaf(a.x, w[4 * q], acc))));
+    }
+    const int m = m0 + r;
+    out[(long long)m * p.ldo] = acc + b + (p.add_rows ? p.add_rows[(long long)(m % p.add_mod) * p.N + n] : 0.f);
   }
 }
 
@@ -84,11 +134,21 @@ bool gemv_rows_ok(const GemmArgs& a) {
   return a.epi == EPI_STORE && a.out_dtype == F32 && a.K <= kGemvMaxK && (a.N <= 64 || a.K <= 64);
 }
 
+template <int AD, int WD>
+static void launch_gemv(const GemmArgs& a, cudaStream_t s) {
+  if (a.K > 64) {
+    launch_k(gemv_rows_kernel<AD, WD>, dim3(a.M), dim3(256), 0, s, a);
+    return;
+  }
+  const int cols = (a.N + 255) / 256, rows = a.M * cols >= 16 * 304 ? 16 : a.M * cols >= 4 * 304 ? 4 : 1;   // two CTAs an SM
+  launch_k(short_k_kernel<AD, WD>, dim3(cols, (a.M + rows - 1) / rows), dim3(256), 0, s, a, rows);
+}
+
 void launch_gemv_rows(const GemmArgs& a, cudaStream_t s) {
-  if (a.a_dtype == F32 && a.w_dtype == F32) launch_k(gemv_rows_kernel<F32, F32>, dim3(a.M), dim3(256), 0, s, a);
-  else if (a.a_dtype == F32 && a.w_dtype == BF16) launch_k(gemv_rows_kernel<F32, BF16>, dim3(a.M), dim3(256), 0, s, a);
-  else if (a.a_dtype == BF16 && a.w_dtype == BF16) launch_k(gemv_rows_kernel<BF16, BF16>, dim3(a.M), dim3(256), 0, s, a);
-  else launch_k(gemv_rows_kernel<BF16, F32>, dim3(a.M), dim3(256), 0, s, a);
+  if (a.a_dtype == F32 && a.w_dtype == F32) launch_gemv<F32, F32>(a, s);
+  else if (a.a_dtype == F32 && a.w_dtype == BF16) launch_gemv<F32, BF16>(a, s);
+  else if (a.a_dtype == BF16 && a.w_dtype == BF16) launch_gemv<BF16, BF16>(a, s);
+  else launch_gemv<BF16, F32>(a, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -373,209 +433,219 @@ void launch_norm(const NormArgs& a, cudaStream_t s) {
   }
 }
 
-__device__ __forceinline__ float rope_elem(const void* base, long long off, int d, int half,
-                                           const float* cs, int dt) {
-  const float x = ldf_rt(base, off + d, dt);
-  const int j = d < half ? d : d - half;
-  const float c = cs[2 * j], s = cs[2 * j + 1];
-  const float o = ldf_rt(base, off + (d < half ? d + half : d - half), dt);
-  return d < half ? x * c - o * s : x * c + o * s;
-}
-
 // ------------------------------------------------------------------------------------------
-// Attention for few queries (bf16 operands, head dim 64), split over 64-key chunks (split-KV):
-// CTA (query block of 16, key chunk, head, robot) computes the chunk's scores with 256 threads over
-// (query, 4 keys) pairs, its softmax partials (max, sum) and P V with threads over (query, 4 dims).
-// With one chunk the rows are written at once; otherwise each CTA leaves its partial rows in the
-// workspace and the last CTA of the (robot, head, query block) merges them by log-sum-exp and
-// resets the arrival count for the next launch. Used by the DiT head: self-attention over the
-// chunk's tokens and cross-attention over the projected prefix.
-constexpr int kFewDh = 64, kFewQ = 16, kFewKC = 64;
-constexpr int kFewPart = kFewDh + 4;     // partial row: O, max, sum, padding (16-byte rows)
-constexpr int kFewKPitch = kFewDh + 2;   // bf16 per key row: rows 33 words apart, no bank conflicts
+// Attention for few queries (bf16 operands, head dim 64): the DiT head's self-attention over the chunk
+// and cross-attention over the projected prefix. CTA = 16 queries of one head and robot and a share of
+// the 64-key tiles; the CTAs that share a query block form a cluster and its first CTA merges their
+// partial rows by log-sum-exp, received through distributed shared memory. Per tile: Q K^T on the tensor
+// cores (m16n8k16: the products of bf16 operands are exact, sums in fp32), warp = 8 keys, operands
+// straight from global memory; softmax in fp32; P V on the tensor cores with every fp32 probability
+// as the sum of three bf16 terms (24 bits: nothing is rounded away), warp = 8 head dims.
+// What bounds it is latency, half of it instruction fetch: a kernel whose code is not in the SM's
+// instruction cache runs at a dozen cycles an instruction. The prefix keys and values, which no
+// kernel of the loop writes, are loaded before the wait for the previous kernel, and a rehearsal pass
+// over them (its results dropped) brings the code in while the CTA would idle.
+constexpr int kFewDh = 64, kFewQ = 16, kFewKT = 64, kFewCluster = 8;
+constexpr int kFewPitch = kFewDh + 8;     // bf16 rows of V and P: ldmatrix without bank conflicts
+constexpr int kFewSPitch = kFewKT + 4;    // fp32 rows of scores and partial outputs
 
-__host__ __device__ inline int few_chunks(int n_keys) { return (n_keys + kFewKC - 1) / kFewKC; }
-
-__device__ __forceinline__ uint32_t pack_bf16_pair(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
+struct FewSmem {
+  __nv_bfloat16 v[kFewKT * kFewPitch];
+  __nv_bfloat16 p[3][kFewQ * kFewPitch];
+  float s[kFewQ * kFewSPitch];
+  float m[kFewQ], l[kFewQ], alpha[kFewQ];
+  float part[1];                          // [CTAs of the cluster][16][kFewSPitch]: O, then max and sum
+};
+static size_t few_smem_bytes(int c) { return sizeof(FewSmem) + (c > 1 ? (size_t)c * kFewQ * kFewSPitch * 4 : 0); }
+static int few_cluster(int n_keys) {
+  const int t = (n_keys + kFewKT - 1) / kFewKT;
+  return t < kFewCluster ? t : kFewCluster;
 }
 
-__global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p) {
-  __shared__ float qs[kFewQ][kFewDh];
-  __shared__ float ps[kFewQ][kFewKC];
-  __shared__ __align__(16) __nv_bfloat16 ks[kFewKC * kFewKPitch];
-  __shared__ __align__(16) __nv_bfloat16 vs[kFewKC * kFewDh];
-  __shared__ float ml[kFewQ][2];
-  __shared__ int last;
+__device__ __forceinline__ void ldsm4(uint32_t* r, const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t* r, const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, const uint32_t* b) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+__device__ __forceinline__ void st_dsm2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+
+__global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
+  extern __shared__ __align__(16) unsigned char few_raw[];
+  FewSmem& sm = *reinterpret_cast<FewSmem*>(few_raw);
   pdl_trigger();
-  pdl_wait();
-  constexpr int dh = kFewDh, half = dh / 2;
-  const int n_keys = p.P + (p.kc ? p.H : 0);
-  const int C = few_chunks(n_keys), qb = blockIdx.x / C, kc = blockIdx.x % C, key0 = kc * kFewKC;
-  const int nk = min(kFewKC, n_keys - key0);
-  const int b = blockIdx.z, hq = blockIdx.y, i0 = qb * kFewQ;
+  const int rank = blockIdx.x % C, i0 = blockIdx.x / C * kFewQ, hq = blockIdx.y, b = blockIdx.z;
   const int g = hq / (p.n_heads / p.n_kv_heads);
-  const int tid = threadIdx.x;
-  // the chunk's keys and values: 16-byte loads, all issued before any use
-  for (int e = tid; e < nk * (dh / 8); e += 256) {
-    const int j = key0 + e / (dh / 8), c8 = e % (dh / 8);
-    uint4 kv, vv;
-    if (j < p.P) {
-      const long long off = b * p.kp_bstride + (long long)j * p.kp_ld + g * dh + c8 * 8;
-      kv = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.kp) + off);
-      vv = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.vp) + off);
-    } else {
-      const long long off = (long long)(b * p.H + j - p.P) * p.kc_ld + g * dh + c8 * 8;
-      kv = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.kc) + off);
-      vv = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.vc) + off);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gr = lane >> 2, tc = 2 * (lane & 3);
+  const int n_keys = p.P + (p.kc ? p.H : 0), nt = (n_keys + kFewKT - 1) / kFewKT;
+  if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  const __nv_bfloat16* qrow = static_cast<const __nv_bfloat16*>(p.q) + (long long)(b * p.H + i0 + gr) * p.q_ld + hq * kFewDh + tc;
+  const bool q0 = i0 + gr < p.H, q1 = i0 + gr + 8 < p.H;
+  // key j's row of keys (or values) of this head; null past the end
+  const auto row_of = [&](const void* pre, const void* chunk, int j) -> const __nv_bfloat16* {
+    if (j < p.P) return static_cast<const __nv_bfloat16*>(pre) + b * p.kp_bstride + (long long)j * p.kp_ld + g * kFewDh;
+    if (j < n_keys) return static_cast<const __nv_bfloat16*>(chunk) + (long long)(b * p.H + j - p.P) * p.kc_ld + g * kFewDh;
+    return nullptr;
+  };
+  uint32_t kf[8];
+  const auto load_tile = [&](int t) {
+    const __nv_bfloat16* kr = row_of(p.kp, p.kc, t * kFewKT + 8 * warp + gr);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) kf[u] = kr ? __ldcg(reinterpret_cast<const unsigned*>(kr + 8 * u + tc)) : 0u;
+    const int j = tid >> 2, c = 16 * (tid & 3);   // a quarter of a value row each
+    const __nv_bfloat16* vr = row_of(p.vp, p.vc, t * kFewKT + j);
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    const uint4 v0 = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + c)) : zero;
+    const uint4 v1 = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + c + 8)) : zero;
+    *reinterpret_cast<uint4*>(sm.v + j * kFewPitch + c) = v0;
+    *reinterpret_cast<uint4*>(sm.v + j * kFewPitch + c + 8) = v1;
+  };
+  const bool early = (rank + 1) * kFewKT <= p.P;   // this CTA's first tile is prefix keys alone
+  if (early) load_tile(rank);
+
+  float o[4];
+  const int q = tid >> 4, kg = tid & 15;           // softmax: query q, keys 4 kg .. 4 kg + 3
+#pragma unroll 1
+  for (int pass = early ? 0 : 1; pass < 2; ++pass) {
+    if (pass) pdl_wait();
+    if (tid < kFewQ) {
+      sm.m[tid] = -INFINITY;
+      sm.l[tid] = 0.f;
     }
-    uint32_t* kd = reinterpret_cast<uint32_t*>(ks + (size_t)(j - key0) * kFewKPitch + c8 * 8);
-    kd[0] = kv.x;
-    kd[1] = kv.y;
-    kd[2] = kv.z;
-    kd[3] = kv.w;
-    *reinterpret_cast<uint4*>(vs + (size_t)(j - key0) * dh + c8 * 8) = vv;
-  }
-  for (int e = tid; e < kFewQ * dh; e += 256) {
-    const int qi = e / dh, d = e % dh, i = i0 + qi;
-    float val = 0.f;
-    if (i < p.H) {
-      const long long off = (long long)(b * p.H + i) * p.q_ld + hq * dh;
-      val = p.rope_cs ? rope_elem(p.q, off, d, half, p.rope_cs + (long long)i * dh, BF16)
-                      : ldf_rt(p.q, off + d, BF16);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[e] = 0.f;
+    uint32_t qf[4][4];
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        qf[ks][e] = (e & 1 ? q1 : q0) ? __ldcg(reinterpret_cast<const unsigned*>(qrow + (e & 1) * 8ll * p.q_ld + 16 * ks + 8 * (e >> 1))) : 0u;
+#pragma unroll 1
+    for (int t = rank; t < nt; t += C) {
+      if (pass && (t != rank || !early)) load_tile(t);
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) mma16816(c, qf[ks], kf + 2 * ks);
+      float* sr = sm.s + gr * kFewSPitch + 8 * warp + tc;
+      *reinterpret_cast<float2*>(sr) = make_float2(c[0] * p.scale, c[1] * p.scale);
+      *reinterpret_cast<float2*>(sr + 8 * kFewSPitch) = make_float2(c[2] * p.scale, c[3] * p.scale);
+      __syncthreads();
+      const float4 s4 = *reinterpret_cast<const float4*>(sm.s + q * kFewSPitch + 4 * kg);
+      float sc[4] = {s4.x, s4.y, s4.z, s4.w};
+      const float m_old = sm.m[q];
+      float mx = m_old, sum = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (t * kFewKT + 4 * kg + e >= n_keys) sc[e] = -INFINITY;   // keys past the end
+        mx = fmaxf(mx, sc[e]);
+      }
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+      float rest[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        rest[e] = t * kFewKT + 4 * kg + e < n_keys ? expf(sc[e] - mx) : 0.f;
+        sum += rest[e];
+      }
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {   // the probabilities' leading, middle and last 8 bits
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(rest[0], rest[1]), hi = __floats2bfloat162_rn(rest[2], rest[3]);
+        uint2 w;
+        w.x = *reinterpret_cast<const uint32_t*>(&lo);
+        w.y = *reinterpret_cast<const uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(sm.p[k] + q * kFewPitch + 4 * kg) = w;
+        rest[0] -= __low2float(lo);
+        rest[1] -= __high2float(lo);
+        rest[2] -= __low2float(hi);
+        rest[3] -= __high2float(hi);
+      }
+      if (kg == 0) {
+        const float a = m_old == -INFINITY ? 0.f : expf(m_old - mx);
+        sm.alpha[q] = a;
+        sm.m[q] = mx;
+        sm.l[q] = sm.l[q] * a + sum;
+      }
+      __syncthreads();
+      const float a0 = sm.alpha[gr], a1 = sm.alpha[gr + 8];
+      o[0] *= a0;
+      o[1] *= a0;
+      o[2] *= a1;
+      o[3] *= a1;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t vf[4];
+        ldsm4_t(vf, sm.v + (32 * half + lane) * kFewPitch + 8 * warp);
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            uint32_t pf[4];
+            ldsm4(pf, sm.p[k] + (lane & 15) * kFewPitch + 32 * half + 16 * k2 + 8 * (lane >> 4));
+            mma16816(o, pf, vf + 2 * k2);
+          }
+      }
+      if (!pass) break;
+      __syncthreads();   // the next tile's values, scores and probabilities overwrite this one's
     }
-    qs[qi][d] = val * p.scale;
   }
-  __syncthreads();
-  // chunk keys carry RoPE like the queries (prefix keys come rotated)
-  if (p.rope_cs && p.kc) {
-    for (int e = tid; e < nk * half; e += 256) {
-      const int jj = e / half, d = e % half, j = key0 + jj;
-      if (j < p.P) continue;
-      __nv_bfloat16* kr = ks + (size_t)jj * kFewKPitch;
-      const float* cs = p.rope_cs + (long long)(j - p.P) * dh;
-      const float x0 = __bfloat162float(kr[d]), x1 = __bfloat162float(kr[d + half]);
-      kr[d] = __float2bfloat16_rn(x0 * cs[2 * d] - x1 * cs[2 * d + 1]);
-      kr[d + half] = __float2bfloat16_rn(x1 * cs[2 * d] + x0 * cs[2 * d + 1]);
-    }
-    __syncthreads();
-  }
-  // scores: thread (query q, keys 4 kg .. 4 kg + 3); a 16-lane group shares q
-  const int q = tid >> 4, kg = tid & 15;
-  float sc[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) sc[e] = 0.f;
-#pragma unroll 4
-  for (int d2 = 0; d2 < dh / 2; ++d2) {
-    const float q0 = qs[q][2 * d2], q1 = qs[q][2 * d2 + 1];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 kf = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(ks + (size_t)(4 * kg + e) * kFewKPitch)[d2]);
-      sc[e] = fmaf(q0, kf.x, fmaf(q1, kf.y, sc[e]));
-    }
-  }
-  float mx = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    if (4 * kg + e >= nk) sc[e] = -INFINITY;   // keys past the end
-    mx = fmaxf(mx, sc[e]);
-  }
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  float sum = 0.f;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const float pe = expf(sc[e] - mx);
-    ps[q][4 * kg + e] = pe;
-    sum += pe;
-  }
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (kg == 0) {
-    ml[q][0] = mx;
-    ml[q][1] = sum;
-  }
-  __syncthreads();
-  // O = P V: thread (query q, dims 4 c .. 4 c + 3)
-  const int c = tid & 15;
-  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-  for (int j = 0; j < nk; ++j) {
-    const float pj = ps[q][j];
-    const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(vs + (size_t)j * dh + 4 * c);
-    const float2 v0 = __bfloat1622float2(v2[0]), v1 = __bfloat1622float2(v2[1]);
-    o.x = fmaf(pj, v0.x, o.x);
-    o.y = fmaf(pj, v0.y, o.y);
-    o.z = fmaf(pj, v1.x, o.z);
-    o.w = fmaf(pj, v1.y, o.w);
-  }
-  const int i = i0 + q;
-  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) + (long long)(b * p.H + i) * p.out_ld + hq * dh + 4 * c;
+
+  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) + (long long)(b * p.H + i0) * p.out_ld + hq * kFewDh;
   if (C == 1) {
-    if (i < p.H) {
-      const float inv = 1.f / ml[q][1];
-      uint2 pk;
-      pk.x = pack_bf16_pair(o.x * inv, o.y * inv);
-      pk.y = pack_bf16_pair(o.z * inv, o.w * inv);
-      *reinterpret_cast<uint2*>(dst) = pk;
-    }
+    const float l0 = 1.f / sm.l[gr], l1 = 1.f / sm.l[gr + 8];
+    if (q0) *reinterpret_cast<__nv_bfloat162*>(dst + (long long)gr * p.out_ld + 8 * warp + tc) = __floats2bfloat162_rn(o[0] * l0, o[1] * l0);
+    if (q1) *reinterpret_cast<__nv_bfloat162*>(dst + (long long)(gr + 8) * p.out_ld + 8 * warp + tc) = __floats2bfloat162_rn(o[2] * l1, o[3] * l1);
     return;
   }
-  // partial rows of this chunk: [group][chunk][q][kFewPart] (O, then max and sum)
-  const int QB = gridDim.x / C;
-  const size_t grp = ((size_t)b * p.n_heads + hq) * QB + qb;
-  float* part = p.split_ws + ((grp * C + kc) * kFewQ + q) * kFewPart;
-  *reinterpret_cast<float4*>(part + 4 * c) = o;
-  if (c == 0) {
-    part[dh] = ml[q][0];
-    part[dh + 1] = ml[q][1];
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const unsigned prev = atomicAdd(p.split_ctr + grp, 1u);
-    last = prev == (unsigned)C - 1u;
-    if (last) p.split_ctr[grp] = 0u;   // every chunk has arrived: reset for the next launch
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // merge the chunks by log-sum-exp
-  const float* base = p.split_ws + (grp * C * kFewQ + q) * kFewPart;
+  // partial rows to the cluster's first CTA, once it runs
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  uint32_t to;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(sm.part + rank * kFewQ * kFewSPitch)));
+  st_dsm2(to + (gr * kFewSPitch + 8 * warp + tc) * 4, o[0], o[1]);
+  st_dsm2(to + ((gr + 8) * kFewSPitch + 8 * warp + tc) * 4, o[2], o[3]);
+  if (tid < kFewQ) st_dsm2(to + (tid * kFewSPitch + kFewDh) * 4, sm.m[tid], sm.l[tid]);
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank != 0) return;
+  const float* base = sm.part + q * kFewSPitch;
   float M = -INFINITY;
-  for (int k = 0; k < C; ++k) M = fmaxf(M, __ldcg(base + (size_t)k * kFewQ * kFewPart + dh));
+  for (int k = 0; k < C; ++k) M = fmaxf(M, base[k * kFewQ * kFewSPitch + kFewDh]);
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float L = 0.f;
   for (int k = 0; k < C; ++k) {
-    const float* r = base + (size_t)k * kFewQ * kFewPart;
-    const float w = expf(__ldcg(r + dh) - M);
-    L = fmaf(w, __ldcg(r + dh + 1), L);
-    const float4 v = __ldcg(reinterpret_cast<const float4*>(r + 4 * c));
+    const float* r = base + k * kFewQ * kFewSPitch;
+    const float w = expf(r[kFewDh] - M);
+    L = fmaf(w, r[kFewDh + 1], L);
+    const float4 v = *reinterpret_cast<const float4*>(r + 4 * kg);
     acc.x = fmaf(w, v.x, acc.x);
     acc.y = fmaf(w, v.y, acc.y);
     acc.z = fmaf(w, v.z, acc.z);
     acc.w = fmaf(w, v.w, acc.w);
   }
-  if (i < p.H) {
+  if (i0 + q < p.H) {
     const float inv = 1.f / L;
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x * inv, acc.y * inv), hi = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
     uint2 pk;
-    pk.x = pack_bf16_pair(acc.x * inv, acc.y * inv);
-    pk.y = pack_bf16_pair(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2*>(dst) = pk;
+    pk.x = *reinterpret_cast<const uint32_t*>(&lo);
+    pk.y = *reinterpret_cast<const uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(dst + (long long)q * p.out_ld + 4 * kg) = pk;
   }
 }
 
-size_t attn_few_ws_floats(int B, int n_heads, int H, int n_keys) {
-  return (size_t)B * n_heads * ((H + kFewQ - 1) / kFewQ) * few_chunks(n_keys) * kFewQ * kFewPart;
-}
-size_t attn_few_ctr_count(int B, int n_heads, int H) { return (size_t)B * n_heads * ((H + kFewQ - 1) / kFewQ); }
-
-bool attn_few_ok(const AttnArgs& a) {
+// bf16, head dim 64, no rotation (rotated queries are fp32), 16-byte rows of keys and values.
+static bool attn_few_ok(const AttnArgs& a) {
   const int n_keys = a.P + (a.kc ? a.H : 0);
-  const bool aligned = a.kp_ld % 8 == 0 && a.kc_ld % 8 == 0 && a.q_ld % 8 == 0 && a.out_ld % 4 == 0;
-  return a.dtype == BF16 && a.head_dim == kFewDh && n_keys >= 1 && aligned && (a.kp_bstride % 8) == 0 &&
-         (a.n_heads * a.head_dim) % 8 == 0 && (few_chunks(n_keys) == 1 || (a.split_ws && a.split_ctr));
+  return a.dtype == BF16 && a.head_dim == kFewDh && !a.rope_cs && n_keys >= 1 && a.kp_ld % 8 == 0 && a.kc_ld % 8 == 0 &&
+         a.q_ld % 8 == 0 && a.out_ld % 4 == 0 && a.kp_bstride % 8 == 0;
 }
 
 __global__ void add_tau_silu_kernel(const float* __restrict__ x, const float* __restrict__ tab, int stride, int off,
@@ -598,10 +668,14 @@ void launch_add_tau_silu(const float* x, const float* tab, int stride, int off, 
   launch_k(add_tau_silu_kernel, dim3(blocks), dim3(256), 0, s, x, tab, stride, off, tau_row, M, N, y, dt);
 }
 
+void launch_attention_prepare() {
+  cudaFuncSetAttribute(attn_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)few_smem_bytes(kFewCluster));
+}
+
 void launch_attention(const AttnArgs& a, cudaStream_t s) {
   if (attn_few_ok(a)) {
-    const int n_keys = a.P + (a.kc ? a.H : 0);
-    launch_k(attn_few_kernel, dim3(((a.H + kFewQ - 1) / kFewQ) * few_chunks(n_keys), a.n_heads, a.B), dim3(256), 0, s, a);
+    const int C = few_cluster(a.P + (a.kc ? a.H : 0));
+    launch_cluster(attn_few_kernel, dim3((a.H + kFewQ - 1) / kFewQ * C, a.n_heads, a.B), dim3(256), few_smem_bytes(C), C, s, a, C);
     return;
   }
   launch_attn_rows(a, s);

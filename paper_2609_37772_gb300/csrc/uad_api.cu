@@ -113,8 +113,6 @@ struct uad_ctx {
   unsigned char* stage = nullptr;         // copies of prefixes given in host memory, grown on demand
   size_t stage_cap = 0;
   void *kpre = nullptr, *vpre = nullptr;  // ADARMS [B][L][P][Hkv dh]; DiT [B][L][P][Hq dh]
-  float* few_ws = nullptr;                // few-query attention: partial rows of the key chunks
-  unsigned* few_ctr = nullptr;            // and their arrival counts (zero between launches)
   std::vector<int> has_prefix;
 
   // activations / state
@@ -455,10 +453,7 @@ double gemm_bytes(const GemmArgs& g, int wes) {
 void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   g.W = w.w;
   if (!w.tiled) {
-    // row-at-a-time kernel for a long K (action out) or few rows; a short K over many rows (the
-    // action-in projection of a batch) goes to the tiled kernel, which reuses each weight tile
-    // over 64 rows
-    if (gemv_rows_ok(g) && (g.K > 64 || g.M <= 64)) launch_gemv_rows(g, s);
+    if (gemv_rows_ok(g)) launch_gemv_rows(g, s);
     else launch_gemm_ffma(g, s);
     return;
   }
@@ -726,7 +721,6 @@ void enqueue_chunk(uad_ctx* c, int B, int n_steps, bool step, cudaStream_t s) {
         at.vc = static_cast<const char*>(c->qkv) + (size_t)(c->qd + c->kvd) * c->es;
         at.kc_ld = c->qkvd;
         at.out = c->o; at.out_ld = c->qd; at.dtype = dt; at.scale = 1.f / std::sqrt((float)a.head_dim);
-        at.split_ws = c->few_ws; at.split_ctr = c->few_ctr;
         if (!dit) {
           at.kp = static_cast<const char*>(c->kpre) + (size_t)l * a.prefix_len * c->kvd * c->es;
           at.vp = static_cast<const char*>(c->vpre) + (size_t)l * a.prefix_len * c->kvd * c->es;
@@ -765,7 +759,6 @@ void enqueue_chunk(uad_ctx* c, int B, int n_steps, bool step, cudaStream_t s) {
           ac.vp = static_cast<const char*>(c->vpre) + (size_t)l * a.prefix_len * c->qd * c->es;
           ac.P = a.prefix_len; ac.kp_bstride = (long long)a.n_layers * a.prefix_len * c->qd; ac.kp_ld = c->qd;
           ac.out = c->o; ac.out_ld = c->qd; ac.dtype = dt; ac.scale = at.scale;
-          ac.split_ws = c->few_ws; ac.split_ctr = c->few_ctr;
           {
             const double by = c->es * ((double)B * ac.P * c->qd * 2 + 2.0 * M * c->qd);
             Mark mk(c, s, "cross_attn", by, 4.0 * M * a.n_heads * (double)ac.P * a.head_dim);
@@ -1077,15 +1070,6 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
   TRY(dalloc(c, &c->kpre, a.max_batch * per_robot_kv * es));
   TRY(dalloc(c, &c->vpre, a.max_batch * per_robot_kv * es));
   c->has_prefix.assign(a.max_batch, 0);
-  if (a.dtype == UAD_DTYPE_BF16 && a.head_dim == 64) {
-    // few-query attention split over key chunks (self-attention over the chunk, cross-attention
-    // over the prefix): partial rows and zeroed arrival counts
-    const int keys = std::max(a.chunk_len + (a.kind == UAD_KIND_DIT ? 0 : a.prefix_len), a.prefix_len);
-    TRY(dalloc_t(c, &c->few_ws, std::max<size_t>(1, attn_few_ws_floats(a.max_batch, a.n_heads, a.chunk_len, keys))));
-    const size_t nctr = std::max<size_t>(1, attn_few_ctr_count(a.max_batch, a.n_heads, a.chunk_len));
-    TRY(dalloc_t(c, &c->few_ctr, nctr));
-    CK(cudaMemset(c->few_ctr, 0, nctr * sizeof(unsigned)));
-  }
   const size_t M = c->mmax;
   TRY(dalloc_t(c, &c->h, M * W));
   TRY(dalloc(c, &c->y, M * W * es));
@@ -1150,6 +1134,7 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
   CK(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&c->ev_done, cudaEventDisableTiming));
   // kernels with more than 48 KB of dynamic shared memory: opt in once, here
+  launch_attention_prepare();
   ffma_prepare(a.head_dim);
   launch_euler_prepare();
   CK(cudaDeviceSynchronize());

@@ -36,6 +36,33 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
 }
 
+// The same for a grid of thread-block clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t s,
+                                  Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = cluster;
+    at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (pdl_enabled()) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
+}
+
 // GEMM epilogues (out[m][n] from acc = sum_k A[m][k] * Wt[n][k]).
 enum Epi {
   EPI_STORE = 0,       // out = acc (+ bias) (+ add_rows[m % add_mod][n])
@@ -104,14 +131,7 @@ struct AttnArgs {
   void* out = nullptr; int out_ld = 0;                   // out[(b*H + i) * out_ld + hq*dh + d]
   int dtype = F32;
   float scale = 1.f;
-  // few-query attention split over key chunks: partial rows and per-(robot, head, query block)
-  // arrival counts (zero between launches: the last CTA of a group resets its count)
-  float* split_ws = nullptr;
-  unsigned* split_ctr = nullptr;
 };
-// Workspace of the few-query attention split over key chunks, in floats and counters.
-size_t attn_few_ws_floats(int B, int n_heads, int H, int n_keys);
-size_t attn_few_ctr_count(int B, int n_heads, int H);
 
 // Per-step, per-token plan entry (built on the host).
 enum PlanFlag { PF_ACTIVE = 1, PF_GHOST = 2, PF_RELEASE = 4, PF_EARLY = 8, PF_FROZEN = 16,
@@ -148,6 +168,7 @@ bool gemv_rows_ok(const GemmArgs& a);                     // tiny-side projectio
 void launch_gemv_rows(const GemmArgs& a, cudaStream_t s);
 void launch_norm(const NormArgs& a, cudaStream_t s);   // applies the pending residual if part != null
 void launch_attention(const AttnArgs& a, cudaStream_t s);
+void launch_attention_prepare();   // opt in to > 48 KB dynamic shared memory on the current device
 void launch_euler(const EulerArgs& a, cudaStream_t s);
 void launch_euler_prepare();   // shared memory for H x D GAC terms (up to 256 x 64)
 void launch_begin(const float* noise, float* x, float* g, float* u, int n, int* nonfinite, int* evals,
