@@ -94,13 +94,10 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   } else if (threadIdx.x == 32) {
     if (mbar_wait(bar_qk, 0, p.err, 21)) {
       tc_fence_after();
-      const uint32_t q0 = su32(sQ), k0 = su32(sK);
+      const uint64_t qd = sw128_desc(su32(sQ)), kd = sw128_desc(su32(sK));
 #pragma unroll
       for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_bf16(tS, sw128_desc(q0 + c * (kQT * 128) + 32 * k), sw128_desc(k0 + c * (kKT * 128) + 32 * k),
-                   idesc_m128(kKT), (c | k) ? 1u : 0u);
+        mma_kblock(tS, qd + c * (kQT * 128 >> 4), kd + c * (kKT * 128 >> 4), idesc_m128(kKT), c ? 1u : 0u);
     }
     mma_commit(bar_s);
   }
@@ -155,13 +152,10 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   if (threadIdx.x == 32) {
     tc_fence_after();
     if (ok_s && mbar_wait(bar_v, 0, p.err, 23)) {
-      const uint32_t p0 = su32(sP), v0 = su32(sV);
+      const uint64_t pd = sw128_desc(su32(sP)), vd = sw128_desc(su32(sV));
 #pragma unroll
       for (int u = 0; u < kKT / 64; ++u)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_bf16(tO, sw128_desc(p0 + u * (kQT * 128) + 32 * k), sw128_desc(v0 + u * (DH * 128) + 32 * k),
-                   idesc_m128(DH), (u | k) ? 1u : 0u);
+        mma_kblock(tO, pd + u * (kQT * 128 >> 4), vd + u * (DH * 128 >> 4), idesc_m128(DH), u ? 1u : 0u);
     }
     mma_commit(bar_o);
   }
@@ -330,7 +324,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   } else if (threadIdx.x == 160) {
     // issuer: S(0); per chunk c: S(c + 1), then P V(c) once the softmax warps have written P(c)
     bool ok = mbar_wait(q_full, 0, p.err, 42);
-    const uint32_t q0 = su32(sQ), r0 = su32(sR);
+    const uint64_t qdesc = sw128_desc(su32(sQ)), rdesc = sw128_desc(su32(sR));
     const auto issue_s = [&](int c) {
       const int sb = c & 1;
       if (c >= 2) ok = mbar_wait(s_empty + sb, ((c >> 1) - 1) & 1, p.err, 44);
@@ -341,10 +335,8 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
         tc_fence_after();
 #pragma unroll
         for (int cc = 0; cc < NCP; ++cc)
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_bf16(tmem + sb * kKC2, sw128_desc(q0 + (j * NCP + cc) * (kQT * 128) + 32 * k),
-                     sw128_desc(r0 + t * SLOT + cc * (kKC2 * 128) + 32 * k), idesc_m128(kKC2), (j | cc | k) ? 1u : 0u);
+          mma_kblock(tmem + sb * kKC2, qdesc + (uint64_t)((j * NCP + cc) * (kQT * 128 >> 4)),
+                     rdesc + (uint64_t)(t * (SLOT >> 4) + cc * (kKC2 * 128 >> 4)), idesc_m128(kKC2), (j | cc) ? 1u : 0u);
         mma_commit(r_empty + t);
       }
       if (ok) mma_commit(s_full + sb);
@@ -361,7 +353,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
         tc_fence_after();
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          mma_bf16_ts(tO, tmem + sb * kKC2 + 8 * (4 * h + k), sw128_desc(r0 + t * SLOT + 32 * k), idesc_m128(DV),
+          mma_bf16_ts(tO, tmem + sb * kKC2 + 8 * (4 * h + k), rdesc + (uint64_t)(t * (SLOT >> 4) + 2 * k), idesc_m128(DV),
                       (ch | h | k) ? 1u : 0u);
         mma_commit(r_empty + t);
       }

@@ -461,6 +461,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
     if (lane == 0) {
       // ---- MMA issuer ----
       const uint32_t tmem = *tmem_slot;
+      const uint64_t adesc = sw128_desc(su32(sA)), bdesc = sw128_desc(su32(sB));
       int it = 0, j = 0;
       bool ok = true;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
@@ -477,10 +478,8 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
           const int st = it % STAGES, round = it / STAGES;
           if (!mbar_wait(full + st, round & 1, p.err, 64)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a0 = su32(sA + (size_t)st * kStageA), b0 = su32(sB + (size_t)st * kStageBw);
-#pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            ptx::mma_bf16(d, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), idesc, (kb > k0 || k > 0) ? 1u : 0u);
+          mma_kblock(d, adesc + (uint64_t)(st * (kStageA >> 4)), bdesc + (uint64_t)(st * (kStageBw >> 4)), idesc,
+                     kb > k0 ? 1u : 0u);
           mma_commit(empty + st);
         }
         if (ok) mma_commit(tfull + b);

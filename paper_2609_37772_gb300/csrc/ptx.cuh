@@ -51,7 +51,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err
   unsigned long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
     if (mbar_test(b, parity)) return true;
-    if ((it & 255) == 0) {
+    // not on the first turns: the error word is an L2 round trip away
+    if ((it & 63) == 63) {
       if (*reinterpret_cast<volatile int*>(err) != 0) return false;
       const unsigned long long t = gtime();
       if (t0 == 0) t0 = t;
@@ -145,6 +146,16 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a, uint64_t b, 
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
       ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(accum));
+}
+// The four K = 16 MMAs of a 64-wide k-block: a and b are the descriptors of its operands (128-byte rows;
+// a K step of 16 bf16 is two 16-byte units further). One addition per operand and MMA: building each
+// descriptor from its address made the issuing thread the limit (92, 107 and 170 cycles an MMA at N =
+// 64, 128 and 256; 56, 72 and 131 with the descriptors at hand).
+__device__ __forceinline__ void mma_kblock(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+  mma_bf16(d, a, b, idesc, accum);
+  mma_bf16(d, a + 2, b + 2, idesc, 1u);
+  mma_bf16(d, a + 4, b + 4, idesc, 1u);
+  mma_bf16(d, a + 6, b + 6, idesc, 1u);
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar)) : "memory");

@@ -671,6 +671,7 @@ __device__ __noinline__ void projection_step(const StepShared& __restrict__ sh, 
     ++st.a_uses;
     // the next weight tile's barrier is tested (without blocking) before the current tile's MMAs
     // are issued, so that the test's latency overlaps the issue
+    const uint64_t ring0 = sw128_desc(su32(S.ring)), act0 = sw128_desc(su32(S.X));
     bool ready = mbar_peek(S.full + st.slot, st.par);
     bool good = mbar_wait(S.a_full, st.apar, p.err, 42, p.wait_ns);
     for (int i = 0; i < nt && good; ++i) {
@@ -682,10 +683,7 @@ __device__ __noinline__ void projection_step(const StepShared& __restrict__ sh, 
       const int cur = st.slot;
       if (++st.slot == p.ring) { st.slot = 0; st.par ^= 1u; }
       ready = i + 1 < nt && mbar_peek(S.full + st.slot, st.par);
-      const uint32_t a0 = su32(S.ring + (size_t)cur * kSlot), b0 = su32(S.X + (size_t)i * kATile);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        mma_bf16(tmem, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), idesc_m128(64), (i | k) ? 1u : 0u);
+      mma_kblock(tmem, ring0 + (uint64_t)(cur * (kSlot >> 4)), act0 + (uint64_t)(i * (kATile >> 4)), idesc_m128(64), i ? 1u : 0u);
       mma_commit(S.empty + cur);
     }
     mma_commit(S.g_done);
@@ -803,22 +801,16 @@ __device__ __noinline__ void attention_step(const StepArgs& __restrict__ p, cons
       bool good = mbar_wait(S.q_full, st.ipar, p.err, 45, p.wait_ns);
       if (good) {
         tc_fence_after();
-        const uint32_t q0 = su32(sQ), k0 = su32(sK);
+        const uint64_t qd = sw128_desc(su32(sQ)), kd = sw128_desc(su32(sK));
 #pragma unroll
         for (int cc = 0; cc < NC; ++cc)
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_bf16(tmem, sw128_desc(q0 + cc * (kQT * 128) + 32 * k), sw128_desc(k0 + cc * (kKC * 128) + 32 * k),
-                     idesc_m128(kKC), (cc | k) ? 1u : 0u);
+          mma_kblock(tmem, qd + cc * (kQT * 128 >> 4), kd + cc * (kKC * 128 >> 4), idesc_m128(kKC), cc ? 1u : 0u);
       }
       mma_commit(S.s_full);
       good = good && mbar_wait(S.p_full, st.ipar, p.err, 46, p.wait_ns) && mbar_wait(S.v_full, st.ipar, p.err, 47, p.wait_ns);
       if (good) {
         tc_fence_after();
-        const uint32_t p0 = su32(sP), v0 = su32(sV);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_bf16(tmem + 256, sw128_desc(p0 + 32 * k), sw128_desc(v0 + 32 * k), idesc_m128(DH), k ? 1u : 0u);
+        mma_kblock(tmem + 256, sw128_desc(su32(sP)), sw128_desc(su32(sV)), idesc_m128(DH), 0u);
       }
       mma_commit(S.o_done);
     }
