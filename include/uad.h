@@ -248,11 +248,10 @@ int uad_tile_weight(const float* w, int32_t K, int32_t N, uint16_t* out);
  * the projection kernel of every velocity-network layer (Sec. 3, Eq. 1).
  * x: device bf16 [M][K]; w_tiled: device, the layout of uad_tile_weight; bias: device fp32 [N]
  * or NULL; out: device fp32 [M][N]. Needs N % 128 == 0, K % 64 == 0, M >= 1.
- * Split-K scratch (an fp32 [M][N] accumulator and per-tile counters) is allocated by the library
- * with cudaMalloc on the first call on each device and grown on demand; it is kept until exit.
- * Asynchronous on `stream` (a cudaStream_t, NULL = legacy stream). Calls on one device must not
- * overlap on the GPU, since they share that scratch. Returns UAD_OK, UAD_EINVAL, UAD_ENOMEM or
- * UAD_ECUDA. */
+ * An error word is allocated by the library with cudaMalloc on the first call on each device and kept
+ * until exit; K splits are combined on the chip, so calls on different streams may overlap.
+ * Asynchronous on `stream` (a cudaStream_t, NULL = legacy stream). Returns UAD_OK, UAD_EINVAL,
+ * UAD_ENOMEM or UAD_ECUDA. */
 int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out, int32_t M,
                int32_t N, int32_t K, void* stream);
 
@@ -262,19 +261,16 @@ int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out
  * time and synchronize the device, stalling the control loop), and a host framework whose
  * caching allocator already holds the GPU's memory cannot take a stray allocation. This entry
  * point computes exactly what uad_linear computes but allocates nothing: no cudaMalloc,
- * cudaFree or allocating library call. Its split-K scratch is a fixed array inside the
- * library's device image (about 4 MiB), held by every GPU that loads the library until exit.
+ * cudaFree or allocating library call. It needs no scratch beyond an error word inside the
+ * library's device image.
  *   - Limits: M * N <= UAD_LINEAR_STATIC_MAX_ELEMS and (N / 128) * ceil(M / 64) <=
  *     UAD_LINEAR_STATIC_MAX_TILES; larger calls return UAD_ETOOBIG and launch nothing.
- *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress,
+ *   - The first call on a device looks up that word's device address (cudaGetSymbolAddress,
  *     which may load the library's device code: with lazy module loading, the CUDA default,
- *     the driver reserves the array only then). Make one warm-up call per device during
+ *     the driver reserves its memory only then). Make one warm-up call per device during
  *     start-up, before any stream capture begins and before the control loop runs, so that
- *     the device code and its array are resident when "allocates nothing" matters.
- *   - Every call on a device shares the one array and it keeps the previous call's contents:
- *     each call clears the part it uses (asynchronously, on `stream`) before its kernel.
- *     Calls whose work overlaps on the GPU (different streams, or threads racing) corrupt
- *     each other's results; order them on one stream.
+ *     the device code is resident when "allocates nothing" matters.
+ *   - Every call clears the error word (asynchronously, on `stream`) before its kernel.
  * Arguments, layout and other errors are those of uad_linear. */
 #define UAD_ETOOBIG (-7)
 #define UAD_LINEAR_STATIC_MAX_ELEMS (1 << 20)

@@ -1,0 +1,350 @@
+// Few-token tensor-core projection: the K range of an output tile split over a thread-block cluster.
+//
+// out[m][n] = epi(sum_k X[m][k] * Wt[n][k]) for tiles of 128 weight rows x up to 64 tokens. With few
+// tokens a projection is a short chain of dependent steps (operands, MMAs, the sum over the K splits,
+// the epilogue), so the kernel keeps that sum out of global memory: the S CTAs of a cluster each
+// multiply their share of K into tensor memory, stage the fp32 tile in shared memory and send every
+// other CTA the token rows it owns with one bulk copy through distributed shared memory; each CTA adds
+// the S partial rows of its tokens in rank order (the result does not depend on timing) and applies
+// the epilogue to them. Weights are requested before the wait for the kernel that produces the
+// activations. Every wait is bounded; the cluster barriers are reached on every path.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include "uad_internal.cuh"
+#include "ptx.cuh"
+
+namespace uad {
+
+using namespace ptx;
+
+namespace {
+
+constexpr int kBM = 128, kBN = 64, kBK = 64;
+constexpr int kSlotA = kBM * kBK * 2;            // weights of a k-block: 16 KB
+constexpr int kSlotB = kBN * kBK * 2;            // activations: 8 KB
+constexpr int kSlot = kSlotA + kSlotB;
+constexpr int kConsWarps = 8, kCons = 32 * kConsWarps;
+constexpr int kThreads = kCons + 64;             // + producer warp, + MMA warp
+constexpr unsigned long long kWaitNs = 2000000000ull;
+
+__device__ __forceinline__ bool wait_bar(uint64_t* b, uint32_t parity, int* err, int code) {
+  return ptx::mbar_wait(b, parity, err, code, kWaitNs);
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Shared memory -> another CTA's shared memory; completes on that CTA's barrier.
+__device__ __forceinline__ void bulk_s2dsm(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(su32(src)), "r"(bytes), "r"(bar) : "memory");
+}
+
+__device__ __forceinline__ float gelu_tanh_f(float x) {
+  const float k0 = 0.7978845608028654f;
+  return 0.5f * x * (1.f + tanhf(k0 * (x + 0.044715f * x * x * x)));
+}
+__device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) { return make_uint2(pack_bf16(a, b), pack_bf16(c, d)); }
+
+// Where a CTA's shared memory goes: the ring of k-block slots, reused after the MMAs as the staged
+// tile T[token][128] and the partial rows received from the other CTAs, [rank][owned token][128].
+__host__ __device__ __forceinline__ size_t cl_body_bytes(int ring, int splits) {
+  const size_t pipe = (size_t)ring * kSlot, red = (size_t)(kBN + (splits > 1 ? kBN + splits : 0)) * kBM * 4;
+  return pipe > red ? pipe : red;
+}
+
+__global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int S = p.splits, rank = blockIdx.x, nt = blockIdx.y, mt = blockIdx.z;
+  const int KC = p.K / kBK, c0 = rank * KC / S, nkb = (rank + 1) * KC / S - c0;
+  const int m0 = mt * kBN, mcount = p.M - m0 < kBN ? p.M - m0 : kBN;
+  const int per = (mcount + S - 1) / S, t0 = rank * per;            // token rows this CTA finishes
+  const int cnt = mcount - t0 < 0 ? 0 : mcount - t0 < per ? mcount - t0 : per;
+  float* T = reinterpret_cast<float*>(smem);
+  float* recv = T + kBN * kBM;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + cl_body_bytes(ring, S));
+  uint64_t* empty = full + ring;
+  uint64_t* done = empty + ring;
+  uint64_t* got = done + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(got + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < ring; ++i) {
+      mbar_init(full + i, 1);
+      mbar_init(empty + i, 1);
+    }
+    mbar_init(done, 1);
+    mbar_init(got, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (S > 1 && cnt > 0) mbar_expect_tx(got, (uint32_t)((S - 1) * cnt * kBM * 4));
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(kBN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_trigger();
+
+  if (warp == kConsWarps) {
+    // ---- producer ----
+    if (lane == 0) {
+      const uint64_t pol = policy_evict_first();
+      const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + ((size_t)nt * KC + c0) * kSlotA;
+      const int first = nkb < ring ? nkb : ring;
+      for (int i = 0; i < first; ++i) {
+        mbar_expect_tx(full + i, kSlot);
+        bulk_g2s(smem + (size_t)i * kSlot, wt + (size_t)i * kSlotA, kSlotA, full + i, pol);
+      }
+      pdl_wait();
+      for (int i = 0; i < first; ++i) tma_2d(smem + (size_t)i * kSlot + kSlotA, &tmx, (c0 + i) * kBK, m0, full + i);
+      int issued = first;
+      for (int i = first; i < nkb; ++i, ++issued) {
+        const int st = i % ring;
+        if (!wait_bar(empty + st, (i / ring - 1) & 1, p.err, 71)) break;
+        mbar_expect_tx(full + st, kSlot);
+        bulk_g2s(smem + (size_t)st * kSlot, wt + (size_t)i * kSlotA, kSlotA, full + st, pol);
+        tma_2d(smem + (size_t)st * kSlot + kSlotA, &tmx, (c0 + i) * kBK, m0, full + st);
+      }
+      // no copies in flight into shared memory that is reused, or of a CTA that exits
+      for (int i = issued - ring > 0 ? issued - ring : 0; i < issued; ++i) wait_bar(full + i % ring, (i / ring) & 1, p.err, 72);
+    }
+    __syncwarp();
+    if (S > 1) {
+      cluster_arrive();
+      cluster_wait();
+    }
+  } else if (warp == kConsWarps + 1) {
+    // ---- MMA issuer ----
+    if (lane == 0) {
+      const uint32_t tmem = *tmem_slot;
+      const uint32_t idesc = idesc_m128((mcount + 15) / 16 * 16);
+      const uint64_t ring0 = sw128_desc(su32(smem));
+      for (int i = 0; i < nkb; ++i) {
+        const int st = i % ring;
+        if (!wait_bar(full + st, (i / ring) & 1, p.err, 73)) break;
+        tc_fence_after();
+        const uint64_t a = ring0 + (uint64_t)(st * (kSlot >> 4));
+        mma_kblock(tmem, a, a + (kSlotA >> 4), idesc, i ? 1u : 0u);
+        if (i + ring < nkb) mma_commit(empty + st);
+      }
+      mma_commit(done);
+    }
+    __syncwarp();
+    if (S > 1) {
+      cluster_arrive();
+      cluster_wait();
+    }
+  } else {
+    // ---- epilogue warps ----
+    // residual update: this warp's first tokens' gates and residual rows are requested before the
+    // MMAs are waited for
+    constexpr int U = 4;
+    const int n = nt * kBM + 4 * lane;   // this lane's four output features
+    const bool resid = p.epi == EPI_RESID_H;
+    const bool vec = reinterpret_cast<uintptr_t>(p.out) % 16 == 0 && p.ldo % 4 == 0;   // a caller's pointer may not be
+    float4 hv[U], gv[U], bias = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.bias) {
+      const int nb = p.n_store > 0 ? p.n_store : p.N;
+      if (n < nb) bias.x = __ldg(p.bias + n);
+      if (n + 1 < nb) bias.y = __ldg(p.bias + n + 1);
+      if (n + 2 < nb) bias.z = __ldg(p.bias + n + 2);
+      if (n + 3 < nb) bias.w = __ldg(p.bias + n + 3);
+    }
+    const auto load_gates = [&](int t) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tt = t + kConsWarps * u;
+        gv[u] = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (tt < cnt && p.gate_tab)
+          gv[u] = __ldg(reinterpret_cast<const float4*>(p.gate_tab + (size_t)__ldg(p.tau_row + m0 + t0 + tt) * p.gate_stride + n));
+      }
+    };
+    const auto load_h = [&](int t) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tt = t + kConsWarps * u;
+        if (tt < cnt) hv[u] = __ldcg(reinterpret_cast<const float4*>(p.resid + (size_t)(m0 + t0 + tt) * p.N + n));
+      }
+    };
+    if (resid) load_gates(warp);
+    const int row = (warp & 3) * 32 + lane;
+    pdl_wait();
+    if (resid) load_h(warp);
+    const bool ok = wait_bar(done, 0, p.err, 74);
+    tc_fence_after();
+    const uint32_t tm = tmem_base_after_wait(tmem_slot) + ((uint32_t)((warp & 3) * 32) << 16);
+    __syncwarp();
+    for (int q = 16 * (warp >> 2); q < mcount; q += 32) {   // warps 4-7 take the odd 16-token slices
+      float v[16];
+      tmem_ld16(tm + q, v);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) T[(q + e) * kBM + row] = v[e];
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    named_sync(1, kCons);
+    if (S > 1) {
+      // every CTA's MMAs are done (its ring may be written) and its barrier is set up
+      cluster_arrive();
+      cluster_wait();
+      if (threadIdx.x < S && (int)threadIdx.x != rank) {
+        const int r = threadIdx.x, first = r * per, rc = mcount - first < per ? mcount - first : per;
+        if (rc > 0)
+          bulk_s2dsm(mapa(su32(recv + (size_t)rank * per * kBM), r), T + (size_t)first * kBM, (uint32_t)(rc * kBM * 4),
+                     mapa(su32(got), r));
+      }
+    }
+    const bool all = S == 1 || cnt == 0 || wait_bar(got, 0, p.err, 75);
+    if (ok && all) {
+      for (int t = warp; t < cnt; t += kConsWarps * U) {
+        if (resid && t != warp) {
+          load_gates(t);
+          load_h(t);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int tt = t + kConsWarps * u;
+          if (tt >= cnt) break;
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int r = 0; r < S; ++r) {
+            const float* src = r == rank ? T + (size_t)(t0 + tt) * kBM : recv + ((size_t)r * per + tt) * kBM;
+            const float4 q = *reinterpret_cast<const float4*>(src + 4 * lane);
+            v.x += q.x;
+            v.y += q.y;
+            v.z += q.z;
+            v.w += q.w;
+          }
+          const int m = m0 + t0 + tt;
+          v.x += bias.x;
+          v.y += bias.y;
+          v.z += bias.z;
+          v.w += bias.w;
+          switch (p.epi) {
+            case EPI_RESID_H: {
+              float4 h = hv[u];
+              h.x = fmaf(gv[u].x, v.x, h.x);
+              h.y = fmaf(gv[u].y, v.y, h.y);
+              h.z = fmaf(gv[u].z, v.z, h.z);
+              h.w = fmaf(gv[u].w, v.w, h.w);
+              *reinterpret_cast<float4*>(p.resid + (size_t)m * p.N + n) = h;
+              break;
+            }
+            case EPI_GEGLU: {
+              // rows 2i (gate) and 2i + 1 (up) give output i
+              const size_t off = (size_t)m * p.ldo + n / 2;
+              const uint32_t pk = pack_bf16(gelu_tanh_approx(v.x) * v.y, gelu_tanh_approx(v.z) * v.w);
+              if (p.out_dtype == BF16)
+                *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(p.out) + off) = pk;
+              else
+                *reinterpret_cast<float2*>(static_cast<float*>(p.out) + off) = make_float2(gelu_tanh_f(v.x) * v.y, gelu_tanh_f(v.z) * v.w);
+              break;
+            }
+            case EPI_QKV_TC: {
+              const QkvTcOut& o = p.qkv;
+              const int b = m / o.H, i = m - b * o.H;
+              if (nt * kBM < o.qd + o.kvd) {
+                // q or k: two RoPE pairs (rows 2j, 2j + 1 of a head hold dims j and j + dh/2)
+                const bool isq = nt * kBM < o.qd;
+                const int sn = isq ? n : n - o.qd, h = sn / o.dh, r = sn % o.dh, half = o.dh / 2;
+                __nv_bfloat16* dst = isq ? o.q + (((size_t)b * o.Hkv * o.G + h) * o.H + i) * o.dh
+                                         : o.kcache + ((((size_t)b * o.L + o.layer) * o.Hkv + h) * o.NK + o.P + i) * o.dh;
+                if (o.rope) {
+                  const float4 cs = __ldg(reinterpret_cast<const float4*>(o.rope + (size_t)i * o.dh + r));
+                  const int d = r >> 1;
+                  const uint32_t w0 = pack_bf16(v.x * cs.x - v.y * cs.y, v.z * cs.z - v.w * cs.w);
+                  const uint32_t w1 = pack_bf16(v.y * cs.x + v.x * cs.y, v.w * cs.z + v.z * cs.w);
+                  *reinterpret_cast<uint32_t*>(dst + d) = w0;
+                  *reinterpret_cast<uint32_t*>(dst + d + half) = w1;
+                } else {
+                  *reinterpret_cast<uint2*>(dst + r) = pack4(v.x, v.y, v.z, v.w);
+                }
+              } else {
+                const int sn = n - o.qd - o.kvd, g = sn / o.dh, d = sn % o.dh;   // four dims of one head
+                __nv_bfloat16* dst = o.vtcache + ((((size_t)b * o.L + o.layer) * o.Hkv + g) * o.dh + d) * o.NKp + o.P + i;
+                dst[0] = __float2bfloat16_rn(v.x);
+                dst[o.NKp] = __float2bfloat16_rn(v.y);
+                dst[2 * (size_t)o.NKp] = __float2bfloat16_rn(v.z);
+                dst[3 * (size_t)o.NKp] = __float2bfloat16_rn(v.w);
+              }
+              break;
+            }
+            case EPI_PREFIX_KV: {
+              const int w = p.pkv.width, part = nt * kBM / w;   // part = 2 layer + (0 k, 1 v)
+              *reinterpret_cast<uint2*>(((part & 1) ? p.pkv.v : p.pkv.k) + ((size_t)(part >> 1) * p.M + m) * w + (n - part * w)) =
+                  pack4(v.x, v.y, v.z, v.w);
+              break;
+            }
+            default: {
+              if (p.epi == EPI_BIAS_GELU) v = make_float4(gelu_tanh_f(v.x), gelu_tanh_f(v.y), gelu_tanh_f(v.z), gelu_tanh_f(v.w));
+              const size_t off = (size_t)m * p.ldo + n;
+              const int ns = p.n_store > 0 ? p.n_store : p.N;   // a narrow projection's padding rows are not stored
+              if (!vec || n + 3 >= ns) {
+                const float e[4] = {v.x, v.y, v.z, v.w};
+                for (int k = 0; k < 4 && n + k < ns; ++k) {
+                  if (p.out_dtype == BF16) static_cast<__nv_bfloat16*>(p.out)[off + k] = __float2bfloat16_rn(e[k]);
+                  else static_cast<float*>(p.out)[off + k] = e[k];
+                }
+              } else if (p.out_dtype == BF16) {
+                *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.out) + off) = pack4(v.x, v.y, v.z, v.w);
+              } else {
+                *reinterpret_cast<float4*>(static_cast<float*>(p.out) + off) = v;
+              }
+              break;
+            }
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  // a CTA leaves once every CTA has received its rows: until then its own are still being read
+  if (S > 1) {
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kBN));
+  }
+}
+
+}  // namespace
+
+// K splits (= CTAs of a cluster) of a projection, at most eight: as many as keep the grid near one
+// and a half CTAs an SM, so that the next kernel's CTAs find room beside them and fetch their first
+// weights early (two CTAs an SM: DiT head, MLP up in two waves, 894 -> 993 us per evaluation).
+int gemm_cl_splits(int M, int N, int K, int sms) {
+  const int tiles = (N / kBM) * ((M + kBN - 1) / kBN), KC = K / kBK;
+  int s = (3 * sms + tiles) / (2 * tiles);
+  s = s < 1 ? 1 : s > kClMaxSplits ? kClMaxSplits : s;
+  return s < KC ? s : KC;
+}
+
+// The cluster form serves every projection of one 64-token tile, and with more tokens those with so
+// few tiles that the SMs need K splits; a projection with more tiles takes one CTA a tile (narrow form,
+// gemm_tc.cu), whose epilogue it shares with nobody.
+bool gemm_cl_serves(int M, int N, int sms) {
+  return M <= kBN || 2 * (N / kBM) * ((M + kBN - 1) / kBN) <= sms;
+}
+
+static size_t gemm_cl_smem_bytes(int ring, int splits) { return 1024 + cl_body_bytes(ring, splits) + (2 * ring + 2) * 8 + 16; }
+
+void gemm_cl_prepare() {
+  cudaFuncSetAttribute(gemm_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_cl_smem_bytes(kTcMaxStages, kClMaxSplits));
+}
+
+void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
+  const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, ring = per < kTcMaxStages ? per : kTcMaxStages;
+  launch_cluster(gemm_cl_kernel, dim3(a.splits, a.N / kBM, (a.M + kBN - 1) / kBN), dim3(kThreads),
+                 gemm_cl_smem_bytes(ring, a.splits), a.splits, s, *tmx, a, ring);
+}
+
+}  // namespace uad

@@ -8,11 +8,7 @@
 // swizzle and zero fill past the last row. One thread issues tcgen05.mma, one thread feeds
 // the TMA ring, four warps drain TMEM with tcgen05.ld.
 //
-// Split-K: CTAs sharing an output tile each own a K range; they add their partial tile into
-// an fp32 accumulator in L2 (red.global.add) and the last one to arrive (per-tile counter)
-// applies the epilogue, then clears the accumulator and counter for the next launch. The
-// residual projections instead write each split's tile to a plane of its own (EPI_PARTIAL):
-// the norm that follows sums the planes in a fixed order as part of the residual update.
+// Projections with so few tiles that the SMs need K splits take the cluster form (gemm_cl.cu).
 // Many tokens (a batch of robots) take the persistent wide form instead: one CTA per SM walks
 // units of up to 256 tokens x 128 weight rows with two tensor-memory accumulators, so that the
 // epilogue of one unit overlaps the main loop of the next.
@@ -46,13 +42,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err
   return ptx::mbar_wait(b, parity, err, code, kWaitNs);
 }
 
-// Instruction descriptor, kind::f16: bf16 x bf16 -> fp32, both K-major, M = 128, N = 64.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) |
-                            ((uint32_t)(kBM >> 4) << 24);
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t accum) {
-  ptx::mma_bf16(d, a, b, kIdesc, accum);
-}
-
 __device__ __forceinline__ float gelu_tanh_f(float x) {
   const float k0 = 0.7978845608028654f;
   return 0.5f * x * (1.f + tanhf(k0 * (x + 0.044715f * x * x * x)));
@@ -72,10 +61,9 @@ __device__ __forceinline__ void store_out(void* out, long long i, float v, int d
 }
 
 
-// Shared-memory plan: [pipeline stages, at least 32 KB (reused as the split-K staging tile)]
-// [mbarriers, TMEM slot, flag].
-__host__ __device__ __forceinline__ int tc_stages(int nch, int epi) {
-  (void)epi;
+// Shared-memory plan of the narrow form: [pipeline stages, at least 32 KB (reused as the staged tile)]
+// [mbarriers, TMEM slot].
+__host__ __device__ __forceinline__ int tc_stages(int nch) {
   return nch < kTcMaxStages ? nch : kTcMaxStages;
 }
 __host__ __device__ __forceinline__ size_t tc_pipe_bytes(int stages) {
@@ -205,29 +193,17 @@ __device__ __forceinline__ void tile_epilogue(const TcGemmArgs& p, const float* 
   }
 }
 
-// Optional phase timestamps (TcGemmArgs::trace): slot i of this CTA's 16.
-#define TC_TRACE(i)                                                                                  \
-  do {                                                                                               \
-    if (p.trace)                                                                                     \
-      p.trace[((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 16 + (i)] = gtime(); \
-  } while (0)
-
 __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p) {
   extern __shared__ uint8_t smem_raw[];
-  if (threadIdx.x == 0) TC_TRACE(0);
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int t = blockIdx.x, mt = blockIdx.y, s = blockIdx.z;
-  const int KC = p.K / kBK;
-  const int c0 = s * KC / p.splits, c1 = (s + 1) * KC / p.splits, nch = c1 - c0;
-  const int stages = tc_stages(nch, p.epi);
-  const bool partial = p.epi == EPI_PARTIAL;
+  const int t = blockIdx.x, mt = blockIdx.y, nch = p.K / kBK;
+  const int stages = tc_stages(nch);
   uint8_t* sA = smem;
   uint8_t* sB = smem + (size_t)stages * kStageA;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + tc_pipe_bytes(stages));
   uint64_t* empty = full + kTcMaxStages;
   uint64_t* done = empty + kTcMaxStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-  int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = mt * kBN;
   const int mcount = p.M - m0 < kBN ? p.M - m0 : kBN;
@@ -248,7 +224,6 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  if (threadIdx.x == 0) TC_TRACE(1);
 
   pdl_trigger();
   if (threadIdx.x == 0) {
@@ -256,23 +231,21 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     //      Weights are constant: the first ring's worth is requested before waiting for the
     //      kernel that produces the activations. ----
     const uint64_t pol = policy_evict_first();
-    const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + ((size_t)t * KC + c0) * kStageA;
+    const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + (size_t)t * nch * kStageA;
     const int first = nch < stages ? nch : stages;
     for (int i = 0; i < first; ++i) {
       mbar_expect_tx(full + i, kStageA + kStageB);
       bulk_g2s(sA + (size_t)i * kStageA, wt + (size_t)i * kStageA, kStageA, full + i, pol);
     }
-    TC_TRACE(2);
     pdl_wait();
-    TC_TRACE(3);
-    for (int i = 0; i < first; ++i) tma_2d(sB + (size_t)i * kStageB, &tmx, (c0 + i) * kBK, mt * kBN, full + i);
+    for (int i = 0; i < first; ++i) tma_2d(sB + (size_t)i * kStageB, &tmx, i * kBK, mt * kBN, full + i);
     int issued = first;
     for (int i = first; i < nch; ++i) {
       const int st = i % stages, round = i / stages;
       if (!mbar_wait(empty + st, (round - 1) & 1, p.err, 11)) break;
       mbar_expect_tx(full + st, kStageA + kStageB);
       bulk_g2s(sA + (size_t)st * kStageA, wt + (size_t)i * kStageA, kStageA, full + st, pol);
-      tma_2d(sB + (size_t)st * kStageB, &tmx, (c0 + i) * kBK, mt * kBN, full + st);
+      tma_2d(sB + (size_t)st * kStageB, &tmx, i * kBK, mt * kBN, full + st);
       ++issued;
     }
     // do not leave copies in flight into shared memory of an exiting CTA
@@ -280,20 +253,17 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
       mbar_wait(full + i % stages, (i / stages) & 1, p.err, 12);
   } else if (threadIdx.x == 32) {
     // ---- MMA issuer ----
+    const uint64_t adesc = sw128_desc(su32(sA)), bdesc = sw128_desc(su32(sB));
     bool ok = true;
     for (int i = 0; i < nch && ok; ++i) {
       const int st = i % stages, round = i / stages;
       ok = mbar_wait(full + st, round & 1, p.err, 13);
       if (!ok) break;
-      if (i == 0) TC_TRACE(4);
       tc_fence_after();
-      const uint32_t a0 = su32(sA + (size_t)st * kStageA), b0 = su32(sB + (size_t)st * kStageB);
-#pragma unroll
-      for (int k = 0; k < kBK / 16; ++k)
-        mma_bf16(tmem, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), (i > 0 || k > 0) ? 1u : 0u);
+      mma_kblock(tmem, adesc + (uint64_t)(st * (kStageA >> 4)), bdesc + (uint64_t)(st * (kStageB >> 4)), idesc_m128(kBN),
+                 i > 0 ? 1u : 0u);
       mma_commit(empty + st);
     }
-    TC_TRACE(5);
     mma_commit(done);
   }
   __syncwarp();
@@ -301,14 +271,12 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   // ---- epilogue: TMEM -> registers, one weight row (output feature) per thread ----
   pdl_wait();
   const bool ok = mbar_wait(done, 0, p.err, 14);
-  if (threadIdx.x == 64) TC_TRACE(6);
   tc_fence_after();
   const int row = warp * 32 + lane;
   const int n = t * kBM + row;
   float v[kBN];
   __syncwarp();
   tmem_ld64(tmem + ((uint32_t)(warp * 32) << 16), v);
-  bool have = ok && nch > 0;
   // Stage the accumulator tile in shared memory, T[token j][row]: the epilogues below are
   // compact loops over it (neighbouring rows -- GeGLU and RoPE partners -- are one column
   // apart), which keeps the kernel's code small.
@@ -316,66 +284,9 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
 #pragma unroll
   for (int j = 0; j < kBN; ++j) T[j * kBM + row] = v[j];
   __syncthreads();
-  if (threadIdx.x == 0) TC_TRACE(7);
-  if (p.splits > 1 && !partial) {
-    // add the partial tile into the L2 accumulator with 16-byte reds; the last CTA of the tile
-    // reads the sum back (independent 16-byte loads) and clears it for the next launch
-    float* acc = p.acc + (size_t)m0 * p.N + t * kBM;
-    if (have) {
-      for (int idx = threadIdx.x; idx < mcount * (kBM / 4); idx += 128) {
-        const int j = idx / (kBM / 4), c4 = idx % (kBM / 4);
-        red_add_v4(acc + (size_t)j * p.N + c4 * 4, *reinterpret_cast<const float4*>(T + j * kBM + c4 * 4));
-      }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      TC_TRACE(8);
-      const int prev = atomicAdd(p.counters + mt * gridDim.x + t, 1);
-      *last_flag = prev == p.splits - 1;
-      TC_TRACE(9);
-    }
-    __syncthreads();
-    const bool last = *last_flag;
-    have = have && last;
-    if (last) {
-      __threadfence();
-      float4 q[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int idx = threadIdx.x + u * 128;
-        if (idx < mcount * (kBM / 4))
-          q[u] = __ldcg(reinterpret_cast<const float4*>(acc + (size_t)(idx / (kBM / 4)) * p.N + (idx % (kBM / 4)) * 4));
-      }
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int idx = threadIdx.x + u * 128;
-        if (idx < mcount * (kBM / 4)) {
-          const int j = idx / (kBM / 4), c4 = idx % (kBM / 4);
-          __stcg(reinterpret_cast<float4*>(acc + (size_t)j * p.N + c4 * 4), make_float4(0.f, 0.f, 0.f, 0.f));
-          *reinterpret_cast<float4*>(T + j * kBM + c4 * 4) = q[u];
-        }
-      }
-      if (threadIdx.x == 0) p.counters[mt * gridDim.x + t] = 0;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && last) TC_TRACE(10);
-  }
-  if (partial) {
-    // plane s of [splits][M][N]: whole rows of the tile as 16-byte stores
-    if (have) {
-      float* dst = static_cast<float*>(p.out) + (size_t)s * p.M * p.N + (size_t)m0 * p.N + t * kBM;
-      for (int idx = threadIdx.x; idx < mcount * (kBM / 4); idx += 128) {
-        const int j = idx / (kBM / 4), c4 = idx % (kBM / 4);
-        *reinterpret_cast<float4*>(dst + (size_t)j * p.N + c4 * 4) = *reinterpret_cast<const float4*>(T + j * kBM + c4 * 4);
-      }
-    }
-  } else if (have) {
-    tile_epilogue(p, T, kBM, m0, mcount, n, row, lane);
-  }
+  if (ok) tile_epilogue(p, T, kBM, m0, mcount, n, row, lane);
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) TC_TRACE(11);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kBN));
 }
 
@@ -600,9 +511,7 @@ int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows) {
   return r == CUDA_SUCCESS ? 0 : (int)r;
 }
 
-size_t gemm_tc_smem_bytes(int stages, int epi, int M) {
-  (void)epi;
-  (void)M;
+static size_t gemm_tc_smem_bytes(int stages) {
   return 1024 + tc_pipe_bytes(stages) + (2 * kTcMaxStages + 1) * 8 + 16;
 }
 
@@ -618,17 +527,18 @@ void gemm_tc_prepare() {
   static bool done = false;
   if (done) return;
   done = true;
+  gemm_cl_prepare();
   cudaFuncSetAttribute(gemm_tc_pers_kernel<256, kPersStages256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)gemm_tc_pers_smem_bytes(256));
   cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)gemm_tc_pers_smem_bytes(128));
   cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)gemm_tc_smem_bytes(kTcMaxStages, EPI_STORE, kBN));
+                       (int)gemm_tc_smem_bytes(kTcMaxStages));
 }
 
 // Wide tiles (MMA N up to 256 tokens) run the tensor cores near their rate (N = 64 runs at a
 // third of it) and cut L2 re-reads of the weights: 1 = the persistent wide form, 0 = narrow
-// 128 x 64 tiles with K splits. Wide from 512 tokens, or while 256-token tiles fill 60% of the
+// 128 x 64 tiles or the cluster form. Wide from 512 tokens, or while 256-token tiles fill 60% of the
 // SMs or 128-token tiles fill half of them (measured on the pi0-like projections from 200 to 3200
 // tokens: with fewer than 256 tokens the narrow tiles win; at 800 tokens the wide form with K
 // split planes wins for the 1024-row o and down projections too).
@@ -679,31 +589,11 @@ void gemm_tc_pers_plan(int M, int N, int K, int sms, int epi, int* tn, int* spli
   }
 }
 
-// K splits per output tile: one CTA per SM. Partial-plane epilogues (the consumer sums the
-// planes), and any epilogue when all tokens fit one 64-token tile, take more splits, up to two
-// CTAs per SM, so that every CTA holds its whole K range in flight (one HBM round trip). Where the
-// kernel reduces several token tiles in L2 extra splits cost more than they save (measured:
-// pi0-like qkv at 200 tokens 19.6 -> 20.2 us per layer; DiT qkv and MLP up at 16 tokens gain,
-// 1.134 -> 1.103 ms per evaluation).
-int gemm_tc_splits(int M, int N, int K, int sms, int epi) {
-  const int tiles = (N / kBM) * ((M + kBN - 1) / kBN);
-  const int KC = K / kBK;
-  const int cap = kTcMaxStages;
-  int s = sms / tiles;
-  if (s < 1) s = 1;
-  if ((epi == EPI_PARTIAL || M <= kBN) && (KC + s - 1) / s > cap) {
-    const int need = (KC + cap - 1) / cap;
-    const int most = 2 * sms / tiles;
-    s = need < most ? need : (most > s ? most : s);
-  }
-  if (s > KC) s = KC;
-  return s;
-}
-
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
   a->wide = gemm_tc_use_wide(M, N, sms);
   a->tn = 0;
   a->splits = 1;
+  a->cl = 0;
   if (a->wide) {
     // the plan search walks every unit: remember its answers
     thread_local std::map<std::array<int, 5>, std::pair<int, int>> memo;
@@ -716,8 +606,9 @@ void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
     }
     a->tn = it->second.first;
     a->splits = it->second.second;
-  } else {
-    a->splits = gemm_tc_splits(M, N, K, sms, epi);
+  } else if (epi == EPI_RESID_H || gemm_cl_serves(M, N, sms)) {
+    a->cl = 1;
+    a->splits = gemm_cl_splits(M, N, K, sms);
   }
 }
 
@@ -727,6 +618,7 @@ void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
 // for all of them (300 tokens x 49152 rows x 2048, one observation bound: 8.43 ms on the CUDA cores, 0.20 ms here).
 void gemm_tc_prefix_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
   a->wide = M > kBN;
+  a->cl = !a->wide;
   a->splits = 1;
   a->tn = 0;
   if (a->wide) gemm_tc_pers_plan(M, N, K, sms, EPI_PREFIX_KV, &a->tn, &a->splits);
@@ -747,10 +639,12 @@ void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s)
                *tmx, a);
     return;
   }
-  const int KC = a.K / kBK;
-  const int per = (KC + a.splits - 1) / a.splits;
-  dim3 grid(a.N / kBM, (a.M + kBN - 1) / kBN, a.splits);
-  launch_k(gemm_tc_kernel, grid, dim3(128), gemm_tc_smem_bytes(tc_stages(per, a.epi), a.epi, a.M), s, *tmx, a);
+  if (a.cl) {
+    launch_gemm_cl(tmx, a, s);
+    return;
+  }
+  launch_k(gemm_tc_kernel, dim3(a.N / kBM, (a.M + kBN - 1) / kBN), dim3(128), gemm_tc_smem_bytes(tc_stages(a.K / kBK)), s,
+           *tmx, a);
 }
 
 void launch_relayout_tiled(const float* src, int K, int N, void* dst, int mult, long long off, int rope_dh,

@@ -12,18 +12,9 @@ namespace {
 
 constexpr int kTileN = 128, kTileK = 64;
 
-// Split-K scratch of uad_linear, allocated by the library on first use on each device and
-// grown on demand: fp32 accumulator [M][N] and per-tile arrival counters, both all-zero
-// between launches (the last CTA of every tile clears its part).
-struct Scratch {
-  float* acc = nullptr;
-  size_t acc_floats = 0;
-  int* counters = nullptr;
-  int n_counters = 0;
-  int* err = nullptr;
-};
+// The kernels' error word on each device, allocated on first use.
 std::mutex g_mu;
-std::vector<Scratch> g_scratch;
+std::vector<int*> g_err;
 
 uint16_t f32_to_bf16_rne(float f) {
   uint32_t u;
@@ -43,10 +34,10 @@ int check_linear_args(const void* x, const void* w, const float* out, int32_t M,
 
 namespace uad {
 
-// Shared by uad_linear and its caller-scratch variants: launch the projection kernel with
-// out[M][N] = x[M][K] w^T (+ bias), fp32 output, the given split-K scratch.
-int launch_linear(const void* x, const void* w_tiled, const float* bias, float* out, int M, int N, int K,
-                  float* acc, int* counters, int* err, cudaStream_t s) {
+// Shared by uad_linear and its static variant: launch the projection kernel with
+// out[M][N] = x[M][K] w^T (+ bias), fp32 output.
+int launch_linear(const void* x, const void* w_tiled, const float* bias, float* out, int M, int N, int K, int* err,
+                  cudaStream_t s) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return UAD_ECUDA;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -56,7 +47,7 @@ int launch_linear(const void* x, const void* w_tiled, const float* bias, float* 
   a.w_tiled = w_tiled; a.M = M; a.N = N; a.K = K;
   gemm_tc_plan(M, N, K, sms, EPI_STORE, &a);   // the tile selection of the velocity network's projections
   a.epi = EPI_STORE; a.out = out; a.ldo = N; a.out_dtype = F32; a.bias = bias;
-  a.acc = acc; a.counters = counters; a.err = err;
+  a.err = err;
   gemm_tc_prepare();
   launch_gemm_tc(&tm, a, s);
   return cudaGetLastError() == cudaSuccess ? UAD_OK : UAD_ECUDA;
@@ -88,32 +79,17 @@ int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return UAD_ECUDA;
   std::lock_guard<std::mutex> lk(g_mu);
-  if ((int)g_scratch.size() <= dev) g_scratch.resize(dev + 1);
-  Scratch& sc = g_scratch[dev];
-  const size_t need = (size_t)((M + 63) / 64) * 64 * N;
-  const int tiles = linear_tiles(M, N);
-  if (sc.acc_floats < need) {
-    if (sc.acc) cudaFree(sc.acc);
-    sc.acc = nullptr;
-    sc.acc_floats = 0;
-    if (cudaMalloc(&sc.acc, need * 4) != cudaSuccess) return UAD_ENOMEM;
-    if (cudaMemset(sc.acc, 0, need * 4) != cudaSuccess) return UAD_ECUDA;
-    sc.acc_floats = need;
+  if ((int)g_err.size() <= dev) g_err.resize(dev + 1, nullptr);
+  if (!g_err[dev]) {
+    int* e = nullptr;
+    if (cudaMalloc(&e, 4) != cudaSuccess) return UAD_ENOMEM;
+    if (cudaMemset(e, 0, 4) != cudaSuccess) {
+      cudaFree(e);
+      return UAD_ECUDA;
+    }
+    g_err[dev] = e;
   }
-  if (sc.n_counters < tiles) {
-    if (sc.counters) cudaFree(sc.counters);
-    sc.counters = nullptr;
-    sc.n_counters = 0;
-    if (cudaMalloc(&sc.counters, (size_t)tiles * 4) != cudaSuccess) return UAD_ENOMEM;
-    if (cudaMemset(sc.counters, 0, (size_t)tiles * 4) != cudaSuccess) return UAD_ECUDA;
-    sc.n_counters = tiles;
-  }
-  if (!sc.err) {
-    if (cudaMalloc(&sc.err, 4) != cudaSuccess) return UAD_ENOMEM;
-    if (cudaMemset(sc.err, 0, 4) != cudaSuccess) return UAD_ECUDA;
-  }
-  return launch_linear(x, w_tiled, bias, out, M, N, K, sc.acc, sc.counters, sc.err,
-                       static_cast<cudaStream_t>(stream));
+  return launch_linear(x, w_tiled, bias, out, M, N, K, g_err[dev], static_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"

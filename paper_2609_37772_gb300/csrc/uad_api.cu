@@ -63,14 +63,12 @@ struct uad_ctx {
   bool use_graphs = true;
   bool force_simt = false;     // UAD_GEMM=simt: CUDA-core GEMMs only (debugging)
 
-  // tensor-core GEMM: TMA descriptors of the activation buffers, split-K workspace
+  // tensor-core GEMM: TMA descriptors of the activation buffers
   std::map<const void*, CUtensorMap> tmaps;
   // tensor-core attention (bf16 joint-attention experts): query matrix, K and Vt caches
   bool attn_tc = false;
   AttnTcArgs at0;                 // shapes and buffers; batch / layer set per launch
   AttnTcMaps atmaps;
-  float* tc_acc = nullptr;
-  int* tc_counters = nullptr;
   int* dev_err = nullptr;
   float* part = nullptr;          // K-split partial planes of the residual projections
   // persistent evaluation kernel (adaRMS, bf16, B * H <= 64): one launch per step
@@ -431,8 +429,10 @@ struct Mark {
   }
 };
 
-// Partial planes a residual projection [M][W] x [W][K]^T writes on the tensor cores.
+// Partial planes a residual projection [M][W] x [W][K]^T writes on the tensor cores (none with few
+// tokens, where it updates the residual stream itself).
 size_t residual_planes(const uad_ctx* c, int M, int K) {
+  if (!gemm_tc_use_wide(M, c->a.width, c->sms)) return 0;
   TcGemmArgs t;
   gemm_tc_plan(M, c->a.width, K, c->sms, EPI_PARTIAL, &t);
   return (size_t)t.splits;
@@ -461,7 +461,7 @@ void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   t.w_tiled = w.w; t.M = g.M; t.N = g.N; t.K = g.K;
   gemm_tc_plan(g.M, g.N, g.K, c->sms, g.epi, &t);
   t.epi = g.epi; t.out = g.out; t.ldo = g.ldo; t.out_dtype = g.out_dtype; t.bias = g.bias;
-  t.qkv = g.qkv; t.n_store = g.n_store; t.acc = c->tc_acc; t.counters = c->tc_counters; t.err = c->dev_err;
+  t.qkv = g.qkv; t.n_store = g.n_store; t.err = c->dev_err;
   launch_gemm_tc(&c->tmaps.at(g.A), t, s);
 }
 
@@ -484,6 +484,17 @@ struct PendingResid {
 void resid_gemm(uad_ctx* c, const Lin& w, GemmArgs g, int gate_off, const float* bias, PendingResid* pend,
                 const char* name, cudaStream_t s) {
   const double flops = 2.0 * g.M * g.N * g.K;
+  if (w.tiled && !gemm_tc_use_wide(g.M, g.N, c->sms)) {
+    TcGemmArgs t;
+    t.w_tiled = w.w; t.M = g.M; t.N = g.N; t.K = g.K; t.epi = EPI_RESID_H; t.ldo = g.N;
+    gemm_tc_plan(g.M, g.N, g.K, c->sms, t.epi, &t);
+    t.bias = bias; t.resid = c->h; t.err = c->dev_err; t.tau_row = g.tau_row;
+    if (gate_off >= 0) { t.gate_tab = c->tab + gate_off; t.gate_stride = c->rowlen; }
+    g.epi = EPI_RESID_GATE;
+    Mark mk(c, s, name, gemm_bytes(g, c->es), flops);
+    launch_gemm_tc(&c->tmaps.at(g.A), t, s);
+    return;
+  }
   if (w.tiled) {
     g.epi = EPI_PARTIAL; g.out = c->part; g.ldo = g.N; g.out_dtype = F32;
     pend->part = c->part;
@@ -1105,9 +1116,6 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
     TRY(make_tmap(c, c->y, W, (int)M));
     TRY(make_tmap(c, c->o, c->qd, (int)M));
     TRY(make_tmap(c, c->act, F, (int)M));
-    const size_t maxN = std::max({(size_t)c->qkvd, (size_t)2 * F, (size_t)W});
-    TRY(dalloc_t(c, &c->tc_acc, M * maxN));
-    TRY(dalloc_t(c, &c->tc_counters, 1 << 16));
     size_t part = 0;
     for (int b = 1; b <= a.max_batch; ++b)
       part = std::max({part, residual_planes(c, b * H, c->qd) * (size_t)b * H * W,

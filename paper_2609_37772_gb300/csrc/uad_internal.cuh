@@ -75,6 +75,7 @@ enum Epi {
                        // v -> Vt cache (tensor-core attention layouts, see attn_tc.cu)
   EPI_PREFIX_KV = 7,   // DiT prefix projections of every layer at once: rows [layer][k, v][width]
                        // scatter to the K and V prefix caches (bf16)
+  EPI_RESID_H = 8,     // tensor cores, few tokens: resid[m][n] += gate(m, n) * (acc + bias) in place
 };
 
 // Where the DiT prefix projection (EPI_PREFIX_KV) writes: k, v [L][tokens][width] of one robot.
@@ -198,24 +199,29 @@ struct TcGemmArgs {
   const float* bias = nullptr;
   QkvTcOut qkv;                    // EPI_QKV_TC
   PrefixKvOut pkv;                 // EPI_PREFIX_KV
+  float* resid = nullptr;          // EPI_RESID_H: residual stream [M][N]
+  const float* gate_tab = nullptr; int gate_stride = 0;   //   gate(m, n) = gate_tab[tau_row[m] * stride + n]; 1 if null
+  const int* tau_row = nullptr;
   int n_store = 0;                 // EPI_STORE: > 0: rows n >= n_store are padding (not stored, no bias)
-  float* acc = nullptr;            // split-K accumulator [M][N] fp32, zero between launches
-  int* counters = nullptr;         // split-K arrival counters per output tile, zero between launches
   int* err = nullptr;              // set to a nonzero code if a bounded wait gave up
   int wide = 0;                    // 1: the persistent wide form (one CTA per SM walking units of
                                    // tn tokens x 128 weight rows x a K range), 0: narrow split-K tiles
+  int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)
   int tn = 0;                      // persistent form: tokens per tile (256, 192 or 128)
-  unsigned long long* trace = nullptr;  // optional: 16 global-timer stamps per CTA (phase times)
 };
-size_t gemm_tc_smem_bytes(int stages, int epi, int M);
 // 2-D TMA descriptor of a bf16 activation matrix [rows][K] (64 x 64 boxes, 128-byte swizzle,
 // zero fill past the last row). 0 on success.
 int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows);
 void gemm_tc_prepare();
-int gemm_tc_splits(int M, int N, int K, int sms, int epi);
 int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form serves this projection
 // The tile plan of one projection (wide form, tokens per tile, K splits) into a.
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a);
+// gemm_cl.cu: the few-token form (K splits over a cluster), at most kClMaxSplits splits
+constexpr int kClMaxSplits = 8;
+int gemm_cl_splits(int M, int N, int K, int sms);
+bool gemm_cl_serves(int M, int N, int sms);
+void gemm_cl_prepare();
+void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
 void gemm_tc_prefix_plan(int M, int N, int K, int sms, TcGemmArgs* a);   // EPI_PREFIX_KV: no K splits
 void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
 // element (k, n) of src [K][N] -> row n' * mult + off, column k of the tiled bf16 layout (K cols),
