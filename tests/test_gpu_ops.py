@@ -60,6 +60,43 @@ def test_linear_wide_tiles_match_reference(M, N, K):
     assert np.abs(out - ref).max() <= 1e-5 * np.abs(ref).max()
 
 
+# The cluster form (K splits exchanged between CTAs) where a share is ragged or empty, and the long-K shapes
+# of many rows that it takes over from the wide form:
+#   (1, 128, 512): one token row for eight CTAs; (9, 256, 640): two rows each for five CTAs, ten k-blocks over eight;
+#   (63, 128, 4096): seven CTAs with eight rows, one with seven; (65, 256, 1024): a second tile of one row;
+#   (637, 1024, 2048), (1200, 512, 2112): two and three splits of ragged last tiles
+@pytest.mark.parametrize("M,N,K", [(1, 128, 512), (9, 256, 640), (63, 128, 4096), (65, 256, 1024), (637, 1024, 2048),
+                                   (1200, 512, 2112)])
+def test_linear_cluster_shares_match_reference(M, N, K):
+    rng = np.random.default_rng(M + N + K)
+    x = rng.normal(size=(M, K)).astype(np.float32)
+    w = (rng.normal(size=(K, N)) * 0.02).astype(np.float32)
+    rc, out = run_linear(x, w, None)
+    assert rc == 0
+    ref = reference(x, w, None)
+    assert np.abs(out - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 256, 512), (200, 8192, 128), (530, 2560, 128)])
+def test_linear_takes_outputs_and_biases_at_any_float_address(M, N, K):
+    """out and bias one float past a 16-byte boundary, on the cluster, narrow and wide forms: stores and
+    loads fall back to single floats, and nothing around the output is written."""
+    rng = np.random.default_rng(M + N + K)
+    x = torch.from_numpy(rng.normal(size=(M, K)).astype(np.float32)).to(torch.bfloat16).cuda()
+    w = (rng.normal(size=(K, N)) * 0.02).astype(np.float32)
+    wd = torch.from_numpy(uad.tile_weight(w).view(np.int16)).cuda()
+    room = torch.full((M * N + 8,), float("nan"), device="cuda")
+    bias = torch.from_numpy(rng.normal(size=N + 1).astype(np.float32)).cuda()
+    rc = uad.uad_linear(x.data_ptr(), wd.data_ptr(), bias[1:].data_ptr(), room[1:].data_ptr(), M, N, K,
+                        torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert rc == 0
+    got = room.cpu().numpy()
+    ref = x.float().cpu().numpy().astype(np.float64) @ round_to_bf16(w).astype(np.float64) + bias[1:].cpu().numpy()
+    assert np.abs(got[1:1 + M * N].reshape(M, N) - ref).max() <= 1e-5 * np.abs(ref).max()
+    assert np.isnan(got[0]) and np.isnan(got[1 + M * N:]).all()
+
+
 def test_linear_rejects_bad_shapes():
     assert uad.uad_linear(1, 1, None, 1, 50, 100, 64, None) == uad.UAD_EINVAL
     assert uad.uad_linear(1, 1, None, 1, 0, 128, 64, None) == uad.UAD_EINVAL
