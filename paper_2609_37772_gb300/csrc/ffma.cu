@@ -114,7 +114,31 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
     }
   };
   for (int c = 0; c < ST && c < nch; ++c) load_w(c);
+  // residual update: this thread's first outputs' gates before the wait, their residual values right after
+  // it, so that neither is fetched at the end
+  constexpr int EP = T::BM * T::BN / 256 < 4 ? T::BM * T::BN / 256 : 4;
+  float gate[EP], res[EP];
+  const auto out_of = [&](int u, int& m, int& n) {
+    const int e = tid + 256 * u;
+    m = m0 + e / T::BN;
+    n = n0 + e % T::BN;
+    return m < p.M && n < p.N;
+  };
+  if (p.epi == EPI_RESID_GATE) {
+#pragma unroll
+    for (int u = 0; u < EP; ++u) {
+      int m, n;
+      gate[u] = out_of(u, m, n) && p.gate_tab ? p.gate_tab[(long long)p.tau_row[m] * p.gate_stride + n] : 1.f;
+    }
+  }
   pdl_wait();
+  if (p.epi == EPI_RESID_GATE) {
+#pragma unroll
+    for (int u = 0; u < EP; ++u) {
+      int m, n;
+      res[u] = out_of(u, m, n) ? p.resid[(long long)m * p.ldr + n] : 0.f;
+    }
+  }
 #pragma unroll 1
   for (int c = 0; c < ST; ++c) {
     if (c < nch) load_a(c);
@@ -181,7 +205,14 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
     }
     return;
   }
-  for (int e = tid; e < T::BM * T::BN; e += 256) {
+  if (p.epi == EPI_RESID_GATE) {
+#pragma unroll
+    for (int u = 0; u < EP; ++u) {
+      int m, n;
+      if (out_of(u, m, n)) p.resid[(long long)m * p.ldr + n] = fmaf(gate[u], total(m - m0, n - n0) + (p.bias ? p.bias[n] : 0.f), res[u]);
+    }
+  }
+  for (int e = tid + (p.epi == EPI_RESID_GATE ? 256 * EP : 0); e < T::BM * T::BN; e += 256) {
     const int ml = e / T::BN, nl = e % T::BN, m = m0 + ml, n = n0 + nl;
     if (m >= p.M || n >= p.N) continue;
     float r = total(ml, nl) + (p.bias ? p.bias[n] : 0.f);

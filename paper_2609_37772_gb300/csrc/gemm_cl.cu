@@ -174,7 +174,18 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         if (tt < cnt) hv[u] = __ldcg(reinterpret_cast<const float4*>(p.resid + (size_t)(m0 + t0 + tt) * p.N + n));
       }
     };
+    // RoPE: likewise the (cos, sin) of this warp's first tokens (constant), kept where the residual rows would be
+    const bool qk = p.epi == EPI_QKV_TC && p.qkv.rope && nt * kBM < p.qkv.qd + p.qkv.kvd;
+    const auto load_cs = [&](int t) {
+      const int sn = n < p.qkv.qd ? n : n - p.qkv.qd, r = sn % p.qkv.dh;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tt = t + kConsWarps * u;
+        if (tt < cnt) hv[u] = __ldg(reinterpret_cast<const float4*>(p.qkv.rope + (size_t)((m0 + t0 + tt) % p.qkv.H) * p.qkv.dh + r));
+      }
+    };
     if (resid) load_gates(warp);
+    if (qk) load_cs(warp);
     const int row = (warp & 3) * 32 + lane;
     pdl_wait();
     if (resid) load_h(warp);
@@ -208,6 +219,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
           load_gates(t);
           load_h(t);
         }
+        if (qk && t != warp) load_cs(t);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int tt = t + kConsWarps * u;
@@ -256,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
                 __nv_bfloat16* dst = isq ? o.q + (((size_t)b * o.Hkv * o.G + h) * o.H + i) * o.dh
                                          : o.kcache + ((((size_t)b * o.L + o.layer) * o.Hkv + h) * o.NK + o.P + i) * o.dh;
                 if (o.rope) {
-                  const float4 cs = __ldg(reinterpret_cast<const float4*>(o.rope + (size_t)i * o.dh + r));
+                  const float4 cs = hv[u];
                   const int d = r >> 1;
                   const uint32_t w0 = pack_bf16(v.x * cs.x - v.y * cs.y, v.z * cs.z - v.w * cs.w);
                   const uint32_t w1 = pack_bf16(v.y * cs.x + v.x * cs.y, v.w * cs.z + v.z * cs.w);

@@ -186,21 +186,22 @@ __global__ void __launch_bounds__(256) norm_kernel(NormArgs p) {
 template <int NV>
 __global__ void __launch_bounds__(256) norm_reg_kernel(NormArgs p) {
   pdl_trigger();
-  pdl_wait();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= p.M) return;
   const float4* r4 = reinterpret_cast<const float4*>(p.h + (long long)row * p.ldh);
   const float* mod = p.tab ? p.tab + (long long)p.tau_row[row] * p.stride : nullptr;
   float4 x[NV], sc[NV], sh[NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) x[i] = r4[i * 32 + lane];
-  if (mod) {
+  if (mod) {   // the time table, which no kernel of the step loop writes, before the wait
+
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       sc[i] = __ldg(reinterpret_cast<const float4*>(mod + p.scale_off) + i * 32 + lane);
       sh[i] = __ldg(reinterpret_cast<const float4*>(mod + p.shift_off) + i * 32 + lane);
     }
   }
+  pdl_wait();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) x[i] = r4[i * 32 + lane];
   float mean = 0.f;
   if (p.layer_norm) {
     float t = 0.f;
@@ -256,7 +257,6 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 __global__ void __launch_bounds__(1024) resid_norm_kernel(NormArgs p) {
   __shared__ float red[32];
   pdl_trigger();
-  pdl_wait();
   const int row = blockIdx.x, c4 = threadIdx.x;
   const bool on = c4 * 4 < p.W;
   const int tr = p.tau_row[row];
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(1024) resid_norm_kernel(NormArgs p) {
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float4* h4 = reinterpret_cast<float4*>(p.h + (long long)row * p.ldh) + c4;
   if (on) {
-    x = *h4;
+    // the time table and the bias, which no kernel of the step loop writes, before the wait
     const float* mod = p.tab ? p.tab + (long long)tr * p.stride : nullptr;
     if (mod) {
       sc = __ldg(reinterpret_cast<const float4*>(mod + p.scale_off) + c4);
@@ -272,6 +272,10 @@ __global__ void __launch_bounds__(1024) resid_norm_kernel(NormArgs p) {
     }
     if (p.rgate_tab) gt = __ldg(reinterpret_cast<const float4*>(p.rgate_tab + (long long)tr * p.stride + p.rgate_off) + c4);
     if (p.rbias) bs = __ldg(reinterpret_cast<const float4*>(p.rbias) + c4);
+  }
+  pdl_wait();
+  if (on) {
+    x = *h4;
     const long long plane4 = (long long)p.M * p.W / 4;
     const float4* pp = reinterpret_cast<const float4*>(p.part + (long long)row * p.W) + c4;
     int i = 0;
@@ -327,7 +331,6 @@ __global__ void __launch_bounds__(1024) resid_norm_kernel(NormArgs p) {
 template <int NV>
 __global__ void __launch_bounds__(128) resid_norm_reg_kernel(NormArgs p) {
   pdl_trigger();
-  pdl_wait();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= p.M) return;
   const int tr = p.tau_row[row];
@@ -336,15 +339,16 @@ __global__ void __launch_bounds__(128) resid_norm_reg_kernel(NormArgs p) {
   const long long plane4 = (long long)p.M * p.W / 4;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f), one = make_float4(1.f, 1.f, 1.f, 1.f);
   float4 x[NV], acc[NV], gt[NV];
+  const float* mod = p.tab ? p.tab + (long long)tr * p.stride : nullptr;
+  const float4* g4 = p.rgate_tab ? reinterpret_cast<const float4*>(p.rgate_tab + (long long)tr * p.stride + p.rgate_off) : nullptr;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) gt[i] = g4 ? __ldg(g4 + i * 32 + lane) : one;
+  pdl_wait();
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     x[i] = h4[i * 32 + lane];
     acc[i] = p.n_part > 0 ? __ldcg(pp + i * 32 + lane) : zero;
   }
-  const float* mod = p.tab ? p.tab + (long long)tr * p.stride : nullptr;
-  const float4* g4 = p.rgate_tab ? reinterpret_cast<const float4*>(p.rgate_tab + (long long)tr * p.stride + p.rgate_off) : nullptr;
-#pragma unroll
-  for (int i = 0; i < NV; ++i) gt[i] = g4 ? __ldg(g4 + i * 32 + lane) : one;
   for (int sp = 1; sp < p.n_part; ++sp) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
