@@ -42,14 +42,17 @@ __device__ __forceinline__ float ex2_fast(float x) { return ptx::ex2_approx(x); 
 __host__ __device__ __forceinline__ size_t attn_q_bytes(int dh) { return (size_t)dh * kQT * 2; }
 __host__ __device__ __forceinline__ size_t attn_p_extra(int dh) { return attn_q_bytes(dh) >= 32768 ? 0 : 32768; }
 
-template <int DH>
+// DV = head dims of O per CTA: DH, or a half or a quarter of it while the grid stays within the SMs (each CTA
+// computes S and P in full, and P V and its partial rows for its dims only): the loads of V, the readout of O
+// and the partial rows written shrink with it, the scores are computed by CTAs that would be idle.
+template <int DH, int DV>
 __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tq,
                                                          const __grid_constant__ CUtensorMap tk,
                                                          const __grid_constant__ CUtensorMap tv, AttnTcArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   constexpr int NC = DH / 64;
-  constexpr uint32_t QB = DH * kQT * 2, KB = DH * kKT * 2, VB = DH * kKT * 2;
+  constexpr uint32_t QB = DH * kQT * 2, KB = DH * kKT * 2, VB = DV * kKT * 2, VBLK = DV * 128;
   uint8_t* sQ = smem;
   uint8_t* sK = sQ + QB;
   uint8_t* sV = sK + KB;
@@ -58,7 +61,8 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   uint64_t *bar_qk = bars, *bar_v = bars + 1, *bar_s = bars + 2, *bar_o = bars + 3;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
 
-  const int qt = blockIdx.x, kc = blockIdx.y, bg = blockIdx.z;   // bg = b * Hkv + g
+  constexpr int SP = DH / DV;
+  const int qt = blockIdx.x / SP, d0 = blockIdx.x % SP * DV, kc = blockIdx.y, bg = blockIdx.z;   // bg = b * Hkv + g
   const int b = bg / p.n_kv_heads, g = bg % p.n_kv_heads;
   const int kvz = (b * p.n_layers + p.layer) * p.n_kv_heads + g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -78,19 +82,22 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   // S occupies columns [0, 128); O = P V reuses columns [0, DH) once every thread has read S
   const uint32_t tS = tmem, tO = tmem;
   pdl_trigger();
-  pdl_wait();
 
   if (threadIdx.x == 0) {
+    // a chunk of prefix keys alone, which no kernel of the step loop writes, is loaded before the wait for the
+    // kernel that writes Q and the chunk's keys
     const uint64_t pol = policy_evict_last();
+    const bool early = (kc + 1) * kKT <= p.prefix;
+    if (!early) pdl_wait();
     mbar_expect_tx(bar_qk, QB + KB);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      tma_3d(sQ + c * (kQT * 128), &tq, c * 64, qt * kQT, bg, bar_qk, pol);
-      tma_3d(sK + c * (kKT * 128), &tk, c * 64, kc * kKT, kvz, bar_qk, pol);
-    }
+    for (int c = 0; c < NC; ++c) tma_3d(sK + c * (kKT * 128), &tk, c * 64, kc * kKT, kvz, bar_qk, pol);
     mbar_expect_tx(bar_v, VB);
 #pragma unroll
-    for (int u = 0; u < kKT / 64; ++u) tma_3d(sV + u * (DH * 128), &tv, kc * kKT + u * 64, 0, kvz, bar_v, pol);
+    for (int u = 0; u < kKT / 64; ++u) tma_3d(sV + u * VBLK, &tv, kc * kKT + u * 64, d0, kvz, bar_v, pol);
+    if (early) pdl_wait();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) tma_3d(sQ + c * (kQT * 128), &tq, c * 64, qt * kQT, bg, bar_qk, pol);
   } else if (threadIdx.x == 32) {
     if (mbar_wait(bar_qk, 0, p.err, 21)) {
       tc_fence_after();
@@ -104,6 +111,7 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   __syncwarp();
 
   // ---- softmax over this key chunk: one query row per thread ----
+  pdl_wait();
   const bool ok_s = mbar_wait(bar_s, 0, p.err, 22);
   tc_fence_after();
   const int row = warp * 32 + lane;
@@ -155,7 +163,7 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
       const uint64_t pd = sw128_desc(su32(sP)), vd = sw128_desc(su32(sV));
 #pragma unroll
       for (int u = 0; u < kKT / 64; ++u)
-        mma_kblock(tO, pd + u * (kQT * 128 >> 4), vd + u * (DH * 128 >> 4), idesc_m128(DH), u ? 1u : 0u);
+        mma_kblock(tO, pd + u * (kQT * 128 >> 4), vd + u * (VBLK >> 4), idesc_m128(DV), u ? 1u : 0u);
     }
     mma_commit(bar_o);
   }
@@ -168,11 +176,11 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   //      conflicts) and written with one 1-KB bulk copy per row ----
   const int qrow = qt * kQT + row;
   const size_t prow_idx = ((size_t)bg * gridDim.y + kc) * p.r_pad + qrow;
-  constexpr uint32_t pitch = DH * 4 + 16;
+  constexpr uint32_t pitch = DV * 4 + 16;
   uint8_t* srow = smem + (size_t)row * pitch;
   __syncwarp();
 #pragma unroll
-  for (int cc = 0; cc < DH / 32; ++cc) {
+  for (int cc = 0; cc < DV / 32; ++cc) {
     tmem_ld32(tO + lane_base + cc * 32, sv);
 #pragma unroll
     for (int i = 0; i < 32; i += 4)
@@ -180,10 +188,12 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (ok_o && qrow < p.rows) {
-    bulk_s2g(p.part_o + prow_idx * DH, srow, DH * 4);
+    bulk_s2g(p.part_o + prow_idx * DH + d0, srow, DV * 4);
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    p.part_ml[prow_idx * 2] = mx;
-    p.part_ml[prow_idx * 2 + 1] = l;
+    if (d0 == 0) {
+      p.part_ml[prow_idx * 2] = mx;
+      p.part_ml[prow_idx * 2 + 1] = l;
+    }
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
   tc_fence_before();
@@ -280,7 +290,6 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   const uint32_t tmem = *tmem_slot;
   const uint32_t tO = tmem + 2 * kKC2;
   pdl_trigger();
-  pdl_wait();
 
   // Ring entries in the order the MMAs read them: K of chunk 0, then per chunk c the K of chunk
   // c + 1 (S runs a chunk ahead of P V) and the Vt of chunk c.
@@ -288,38 +297,36 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   const auto v_entry = [&](int c, int h) { return KP + c * PPC + (c + 1 < nck ? KP : 0) + h; };
 
   if (threadIdx.x == 128) {
-    // producer: ring entry e into slot e % kSlots2 once entry e - kSlots2 has been read
+    // producer: ring entry e into slot e % kSlots2 once entry e - kSlots2 has been read. The first entries that
+    // hold prefix keys alone, which no kernel of the step loop writes, are requested before the wait for the
+    // kernel that writes Q and the chunk's keys
     const uint64_t pol = policy_evict_last();
-    mbar_expect_tx(q_full, QB);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) tma_3d(sQ + c * (kQT * 128), &tq, c * 64, qt * kQT, bg, q_full, pol);
-    int e = 0;
-    bool ok = true;
-    const auto slot = [&](int& t) {
-      t = e % kSlots2;
-      const int u = e / kSlots2;
-      ++e;
-      return u == 0 || mbar_wait(r_empty + t, (u - 1) & 1, p.err, 41);
-    };
-    const auto load_k = [&](int c) {
-      for (int j = 0; j < KP && ok; ++j) {
-        int t;
-        if (!(ok = slot(t))) break;
+    const int total = KP + (nck - 1) * PPC + 2;
+    const auto load = [&](int e) {
+      const int t = e % kSlots2, f = e - KP, c = e < KP ? -1 : f / PPC < nck - 1 ? f / PPC : nck - 1;
+      const int r = e < KP ? e : f - c * PPC;                        // place in the group of chunk c
+      const bool k = e < KP || (c + 1 < nck && r < KP);
+      if (k) {
         mbar_expect_tx(r_full + t, PB);
 #pragma unroll
         for (int cc = 0; cc < NCP; ++cc)
-          tma_3d(sR + t * SLOT + cc * (kKC2 * 128), &tk, (j * NCP + cc) * 64, c * kKC2, kvz, r_full + t, pol);
-      }
-    };
-    load_k(0);
-    for (int c = 0; c < nck && ok; ++c) {
-      if (c + 1 < nck) load_k(c + 1);
-      for (int h = 0; h < 2 && ok; ++h) {
-        int t;
-        if (!(ok = slot(t))) break;
+          tma_3d(sR + t * SLOT + cc * (kKC2 * 128), &tk, (r * NCP + cc) * 64, (c + 1) * kKC2, kvz, r_full + t, pol);
+      } else {
+        const int h = c + 1 < nck ? r - KP : r;
         mbar_expect_tx(r_full + t, VBLK);
         tma_3d(sR + t * SLOT, &tv, c * kKC2 + h * 64, d0, kvz, r_full + t, pol);
       }
+    };
+    int e = 0;
+    if (2 * kKC2 <= p.prefix)   // the ring's first entries: K of chunks 0 and 1, Vt of chunk 0
+      for (; e < kSlots2 && e < total; ++e) load(e);
+    pdl_wait();
+    mbar_expect_tx(q_full, QB);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) tma_3d(sQ + c * (kQT * 128), &tq, c * 64, qt * kQT, bg, q_full, pol);
+    for (; e < total; ++e) {
+      if (e >= kSlots2 && !mbar_wait(r_empty + e % kSlots2, (e / kSlots2 - 1) & 1, p.err, 41)) break;
+      load(e);
     }
   } else if (threadIdx.x == 160) {
     // issuer: S(0); per chunk c: S(c + 1), then P V(c) once the softmax warps have written P(c)
@@ -370,6 +377,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   }
 
   // ---- softmax warps: one query row per thread ----
+  pdl_wait();
   const int row = warp * 32 + lane;
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
   const float c2s = p.scale_log2;
@@ -616,7 +624,10 @@ int attn_tc_prepare(AttnTcMaps* maps, const AttnTcArgs& a, int batch_max) {
   // 128-key K chunks through `k` and Vt in 64-key boxes
   if (tmap3(&maps->k2, a.kcache, dh, NK, (uint64_t)batch_max * a.n_layers * a.n_kv_heads, (uint64_t)dh * 2,
             NK * dh * 2, 64, 64)) return -1;
-  // Vt boxes of half the head dims for the one-pass kernel's split form
+  // Vt boxes of half the head dims (the kernels' split forms) and of a quarter
+  maps->vt4 = maps->vt;
+  if (dh == 256 && tmap3(&maps->vt4, a.vtcache, NK, dh, (uint64_t)batch_max * a.n_layers * a.n_kv_heads, NKp * 2,
+                         (uint64_t)dh * NKp * 2, 64, (uint32_t)dh / 4)) return -1;
   if (dh >= 128) {
     if (tmap3(&maps->vt2, a.vtcache, NK, dh, (uint64_t)batch_max * a.n_layers * a.n_kv_heads, NKp * 2,
               (uint64_t)dh * NKp * 2, 64, (uint32_t)dh / 2)) return -1;
@@ -634,9 +645,17 @@ int attn_tc_prepare(AttnTcMaps* maps, const AttnTcArgs& a, int batch_max) {
     cudaFuncSetAttribute(attn_tc2_kernel<256, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2);
   }
   const int smem = (int)attn_tc_smem_bytes(dh);
-  if (dh == 64) cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (dh == 128) cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (dh == 256) cudaFuncSetAttribute(attn_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (dh == 64) cudaFuncSetAttribute(attn_tc_kernel<64, 64>, at, smem);
+  if (dh == 128) {
+    cudaFuncSetAttribute(attn_tc_kernel<128, 128>, at, smem);
+    cudaFuncSetAttribute(attn_tc_kernel<128, 64>, at, smem);
+  }
+  if (dh == 256) {
+    cudaFuncSetAttribute(attn_tc_kernel<256, 256>, at, smem);
+    cudaFuncSetAttribute(attn_tc_kernel<256, 128>, at, smem);
+    cudaFuncSetAttribute(attn_tc_kernel<256, 64>, at, smem);
+  }
   return 0;
 }
 
@@ -664,11 +683,27 @@ void launch_attn_tc(const AttnTcMaps& maps, const AttnTcArgs& a, cudaStream_t s)
     }
     return;
   }
-  dim3 grid((a.rows + kQT - 1) / kQT, attn_tc_chunks(a.n_keys), a.batch * a.n_kv_heads);
+  const int qt = (a.rows + kQT - 1) / kQT, kc = attn_tc_chunks(a.n_keys), bg = a.batch * a.n_kv_heads;
+  int sp = 1;
+  {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    while (a.head_dim / (2 * sp) >= 64 && 2 * sp * qt * kc * bg <= sms) sp *= 2;
+  }
+  const dim3 grid(qt * sp, kc, bg);
   const size_t smem = attn_tc_smem_bytes(a.head_dim);
-  if (a.head_dim == 64) launch_k(attn_tc_kernel<64>, grid, dim3(128), smem, s, maps.q, maps.k, maps.vt, a);
-  if (a.head_dim == 128) launch_k(attn_tc_kernel<128>, grid, dim3(128), smem, s, maps.q, maps.k, maps.vt, a);
-  if (a.head_dim == 256) launch_k(attn_tc_kernel<256>, grid, dim3(128), smem, s, maps.q, maps.k, maps.vt, a);
+  const CUtensorMap& vt = sp == 1 ? maps.vt : sp == 2 ? maps.vt2 : maps.vt4;
+  if (a.head_dim == 64) launch_k(attn_tc_kernel<64, 64>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+  if (a.head_dim == 128) {
+    if (sp == 1) launch_k(attn_tc_kernel<128, 128>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+    else launch_k(attn_tc_kernel<128, 64>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+  }
+  if (a.head_dim == 256) {
+    if (sp == 1) launch_k(attn_tc_kernel<256, 256>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+    else if (sp == 2) launch_k(attn_tc_kernel<256, 128>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+    else launch_k(attn_tc_kernel<256, 64>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
+  }
   launch_k(attn_combine_kernel, dim3(a.rows, a.batch * a.n_kv_heads), dim3(a.head_dim / 2), 0, s, a,
            attn_tc_chunks(a.n_keys));
 }

@@ -243,8 +243,8 @@ struct AttnTcArgs {
   int* err = nullptr;
 };
 // k: 128-key boxes; k2: 64-key boxes (step kernel); vt: 64-key Vt boxes of all head dims; vt2: of
-// half of them (the one-pass kernel's split form)
-struct AttnTcMaps { CUtensorMap q, k, vt, k2, vt2; };
+// half of them, vt4: of a quarter (the split forms)
+struct AttnTcMaps { CUtensorMap q, k, vt, k2, vt2, vt4; };
 size_t attn_tc_smem_bytes(int dh);
 int attn_tc_prepare(AttnTcMaps* maps, const AttnTcArgs& a, int batch_max);  // 0 on success
 int attn_tc_chunks(int n_keys);
