@@ -6,7 +6,9 @@
 // multiply their share of K into tensor memory, stage the fp32 tile in shared memory and send every
 // other CTA the token rows it owns with one bulk copy through distributed shared memory; each CTA adds
 // the S partial rows of its tokens in rank order (the result does not depend on timing) and applies
-// the epilogue to them. Weights are requested before the wait for the kernel that produces the
+// the epilogue to them. The receive area lies apart from the operand ring, so that rows arrive while other
+// CTAs' MMAs still run (aliased on the ring: DiT head 916 us per evaluation, apart 840; four robots 1246 and
+// 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. Weights are requested before the wait for the kernel that produces the
 // activations. Every wait is bounded; the cluster barriers are reached on every path.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -50,11 +52,15 @@ __device__ __forceinline__ float gelu_tanh_f(float x) {
 }
 __device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) { return make_uint2(pack_bf16(a, b), pack_bf16(c, d)); }
 
-// Where a CTA's shared memory goes: the ring of k-block slots, reused after the MMAs as the staged
-// tile T[token][128] and the partial rows received from the other CTAs, [rank][owned token][128].
-__host__ __device__ __forceinline__ size_t cl_body_bytes(int ring, int splits) {
-  const size_t pipe = (size_t)ring * kSlot, red = (size_t)(kBN + (splits > 1 ? kBN + splits : 0)) * kBM * 4;
-  return pipe > red ? pipe : red;
+// Where a CTA's shared memory goes: the ring of k-block slots, reused after the MMAs as the staged tile
+// T[token][128]; then the partial rows received from the other CTAs, [rank][owned token][128], apart from
+// the ring, so that they may arrive while this CTA's MMAs still run. `rows`: tokens of the largest tile.
+__host__ __device__ __forceinline__ size_t cl_ring_bytes(int ring, int rows) {
+  const size_t pipe = (size_t)ring * kSlot, tile = (size_t)((rows + 15) / 16 * 16) * kBM * 4;
+  return pipe > tile ? pipe : tile;
+}
+__host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits) {
+  return splits > 1 ? (size_t)((rows + splits - 1) / splits) * splits * kBM * 4 : 0;
 }
 
 __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
@@ -66,8 +72,9 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   const int per = (mcount + S - 1) / S, t0 = rank * per;            // token rows this CTA finishes
   const int cnt = mcount - t0 < 0 ? 0 : mcount - t0 < per ? mcount - t0 : per;
   float* T = reinterpret_cast<float*>(smem);
-  float* recv = T + kBN * kBM;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + cl_body_bytes(ring, S));
+  const int rows = p.M < kBN ? p.M : kBN;
+  float* recv = reinterpret_cast<float*>(smem + cl_ring_bytes(ring, rows));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + cl_ring_bytes(ring, rows) + cl_recv_bytes(rows, S));
   uint64_t* empty = full + ring;
   uint64_t* done = empty + ring;
   uint64_t* got = done + 1;
@@ -91,6 +98,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (S > 1) cluster_arrive();   // this CTA's barriers are set up and its receive area is free
   pdl_trigger();
 
   if (warp == kConsWarps) {
@@ -117,10 +125,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       for (int i = issued - ring > 0 ? issued - ring : 0; i < issued; ++i) wait_bar(full + i % ring, (i / ring) & 1, p.err, 72);
     }
     __syncwarp();
-    if (S > 1) {
-      cluster_arrive();
-      cluster_wait();
-    }
+    if (S > 1) cluster_wait();
   } else if (warp == kConsWarps + 1) {
     // ---- MMA issuer ----
     if (lane == 0) {
@@ -138,10 +143,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       mma_commit(done);
     }
     __syncwarp();
-    if (S > 1) {
-      cluster_arrive();
-      cluster_wait();
-    }
+    if (S > 1) cluster_wait();
   } else {
     // ---- epilogue warps ----
     // residual update: this warp's first tokens' gates and residual rows are requested before the
@@ -202,9 +204,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     named_sync(1, kCons);
     if (S > 1) {
-      // every CTA's MMAs are done (its ring may be written) and its barrier is set up
-      cluster_arrive();
-      cluster_wait();
+      cluster_wait();   // every CTA has started
       if (threadIdx.x < S && (int)threadIdx.x != rank) {
         const int r = threadIdx.x, first = r * per, rc = mcount - first < per ? mcount - first : per;
         if (rc > 0)
@@ -330,12 +330,17 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
 
 }  // namespace
 
-// K splits (= CTAs of a cluster) of a projection, at most eight: as many as keep the grid near one
-// and a half CTAs an SM, so that the next kernel's CTAs find room beside them and fetch their first
-// weights early (two CTAs an SM: DiT head, MLP up in two waves, 894 -> 993 us per evaluation).
+// K splits (= CTAs of a cluster), at most eight: as many as keep the grid near one and a half CTAs an SM, so
+// that the next kernel's CTAs find room beside them and fetch their first weights early; with up to 32 tokens,
+// where a CTA's work is shorter than its start, one CTA an SM unless a split would sum more than 768 products
+// (the tensor cores' accumulation truncates, so the error grows with the run). Per evaluation, 1 / 1.5 / 1.75
+// CTAs an SM: DiT head 805 / 838 / 887 us, its four robots 1227 / 1212 / 1321, pi0-like one robot 717 / 706 /
+// 706, four robots 957 / 900 / 897.
 int gemm_cl_splits(int M, int N, int K, int sms) {
   const int tiles = (N / kBM) * ((M + kBN - 1) / kBN), KC = K / kBK;
-  int s = (3 * sms + tiles) / (2 * tiles);
+  const int one = (sms + tiles / 2) / tiles, half = (3 * sms + tiles) / (2 * tiles);
+  int s = M <= 32 ? one : half;
+  while (s < half && K > 768 * s) ++s;
   s = s < 1 ? 1 : s > kClMaxSplits ? kClMaxSplits : s;
   return s < KC ? s : KC;
 }
@@ -347,16 +352,21 @@ bool gemm_cl_serves(int M, int N, int sms) {
   return M <= kBN || 2 * (N / kBM) * ((M + kBN - 1) / kBN) <= sms;
 }
 
-static size_t gemm_cl_smem_bytes(int ring, int splits) { return 1024 + cl_body_bytes(ring, splits) + (2 * ring + 2) * 8 + 16; }
+static size_t gemm_cl_smem_bytes(int ring, int rows, int splits) {
+  return 1024 + cl_ring_bytes(ring, rows) + cl_recv_bytes(rows, splits) + (2 * ring + 2) * 8 + 16;
+}
+constexpr size_t kClSmem = 112 * 1024;   // two CTAs fit an SM
 
 void gemm_cl_prepare() {
-  cudaFuncSetAttribute(gemm_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_cl_smem_bytes(kTcMaxStages, kClMaxSplits));
+  cudaFuncSetAttribute(gemm_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
 }
 
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
-  const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, ring = per < kTcMaxStages ? per : kTcMaxStages;
+  const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, rows = a.M < kBN ? a.M : kBN;
+  int ring = per < kTcMaxStages ? per : kTcMaxStages;
+  while (gemm_cl_smem_bytes(ring, rows, a.splits) > kClSmem) --ring;   // three slots at least
   launch_cluster(gemm_cl_kernel, dim3(a.splits, a.N / kBM, (a.M + kBN - 1) / kBN), dim3(kThreads),
-                 gemm_cl_smem_bytes(ring, a.splits), a.splits, s, *tmx, a, ring);
+                 gemm_cl_smem_bytes(ring, rows, a.splits), a.splits, s, *tmx, a, ring);
 }
 
 }  // namespace uad
