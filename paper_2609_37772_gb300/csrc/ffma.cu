@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
 #pragma unroll
     for (int u = 0; u < EP; ++u) {
       int m, n;
-      gate[u] = out_of(u, m, n) && p.gate_tab ? p.gate_tab[(long long)p.tau_row[m] * p.gate_stride + n] : 1.f;
+      gate[u] = out_of(u, m, n) && p.gate_tab ? p.gate_tab[(long long)__ldcg(p.tau_row + m) * p.gate_stride + n] : 1.f;
     }
   }
   pdl_wait();
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
       case EPI_BIAS_SILU: store_as(p.out, (long long)m * p.ldo + n, silu(r), p.out_dtype); break;
       case EPI_BIAS_GELU: store_as(p.out, (long long)m * p.ldo + n, gelu_tanh_f(r), p.out_dtype); break;
       case EPI_RESID_GATE: {
-        const float gt = p.gate_tab ? p.gate_tab[(long long)p.tau_row[m] * p.gate_stride + n] : 1.f;
+        const float gt = p.gate_tab ? p.gate_tab[(long long)__ldcg(p.tau_row + m) * p.gate_stride + n] : 1.f;
         float* dst = p.resid + (long long)m * p.ldr + n;
         *dst = fmaf(gt, r, *dst);
         break;

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         const int tt = t + kConsWarps * u;
         gv[u] = make_float4(1.f, 1.f, 1.f, 1.f);
         if (tt < cnt && p.gate_tab)
-          gv[u] = __ldg(reinterpret_cast<const float4*>(p.gate_tab + (size_t)__ldg(p.tau_row + m0 + t0 + tt) * p.gate_stride + n));
+          gv[u] = __ldg(reinterpret_cast<const float4*>(p.gate_tab + (size_t)__ldcg(p.tau_row + m0 + t0 + tt) * p.gate_stride + n));
       }
     };
     const auto load_h = [&](int t) {

@@ -79,7 +79,6 @@ template <int AD, int WD>
 __global__ void __launch_bounds__(256) short_k_kernel(GemmArgs p, int rows) {
   constexpr int KM = 64, RM = 16;
   __shared__ float a_s[RM * KM];
-  pdl_trigger();
   const int n = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * rows, K = p.K;
   const int cnt = p.M - m0 < rows ? p.M - m0 : rows;
   float w[KM], b = 0.f;
@@ -109,6 +108,9 @@ __global__ void __launch_bounds__(256) short_k_kernel(GemmArgs p, int rows) {
     if (p.bias) b = p.bias[n];
   }
   pdl_wait();
+  // not before the wait: this is a step's first kernel, and the ones after it read what the step epilogue wrote
+  // before their own waits
+  pdl_trigger();
   for (int e = threadIdx.x; e < cnt * KM; e += 256) {
     const int r = e / KM, k = e % KM;
     a_s[e] = k < K ? ldf<AD>(p.A, (long long)(m0 + r) * p.lda + k) : 0.f;
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(256) norm_kernel(NormArgs p) {
     ss = fmaf(d, d, ss);
   }
   const float rstd = 1.f / sqrtf(warp_sum(ss) / p.W + 1e-6f);
-  const float* mod = p.tab ? p.tab + (long long)p.tau_row[row] * p.stride : nullptr;
+  const float* mod = p.tab ? p.tab + (long long)__ldcg(p.tau_row + row) * p.stride : nullptr;
   for (int c = lane; c < p.W; c += 32) {
     float y = (r[c] - mean) * rstd;
     if (mod) y = fmaf(y, 1.f + mod[p.scale_off + c], mod[p.shift_off + c]);
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(256) norm_reg_kernel(NormArgs p) {
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= p.M) return;
   const float4* r4 = reinterpret_cast<const float4*>(p.h + (long long)row * p.ldh);
-  const float* mod = p.tab ? p.tab + (long long)p.tau_row[row] * p.stride : nullptr;
+  const float* mod = p.tab ? p.tab + (long long)__ldcg(p.tau_row + row) * p.stride : nullptr;
   float4 x[NV], sc[NV], sh[NV];
   if (mod) {   // the time table, which no kernel of the step loop writes, before the wait
 
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(1024) resid_norm_kernel(NormArgs p) {
   pdl_trigger();
   const int row = blockIdx.x, c4 = threadIdx.x;
   const bool on = c4 * 4 < p.W;
-  const int tr = p.tau_row[row];
+  const int tr = __ldcg(p.tau_row + row);
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f), sc = x, sh = x, gt = make_float4(1.f, 1.f, 1.f, 1.f), bs = x;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float4* h4 = reinterpret_cast<float4*>(p.h + (long long)row * p.ldh) + c4;
@@ -333,7 +335,7 @@ __global__ void __launch_bounds__(128) resid_norm_reg_kernel(NormArgs p) {
   pdl_trigger();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (row >= p.M) return;
-  const int tr = p.tau_row[row];
+  const int tr = __ldcg(p.tau_row + row);
   float4* h4 = reinterpret_cast<float4*>(p.h + (long long)row * p.ldh);
   const float4* pp = reinterpret_cast<const float4*>(p.part + (long long)row * p.W);
   const long long plane4 = (long long)p.M * p.W / 4;
@@ -659,7 +661,7 @@ __global__ void add_tau_silu_kernel(const float* __restrict__ x, const float* __
   const long long total = (long long)M * N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(e / N), n = (int)(e % N);
-    const float v = x[e] + tab[(size_t)tau_row[m] * stride + off + n];
+    const float v = x[e] + tab[(size_t)__ldcg(tau_row + m) * stride + off + n];
     stf(y, e, v / (1.f + expf(-v)), dt);
   }
 }
@@ -699,7 +701,16 @@ __global__ void __launch_bounds__(256) euler_kernel(EulerArgs p) {
   __shared__ float Cr[9];   // SO(3) correction of the tail (rotation dimensions)
   extern __shared__ float ediff[];   // [H][D]
   const EulerSmem sm{ediff, E_s, Cr, &s_rel};
-  euler_robot(p, blockIdx.x, threadIdx.x, blockDim.x, sm, CtaSync());
+  const int b = blockIdx.x, k = p.cur_k[b];
+  EulerArgs q = p;
+  q.k = k;
+  q.plan = p.plan + (size_t)(k - 1) * p.B * p.H;
+  euler_robot(q, b, threadIdx.x, blockDim.x, sm, CtaSync());
+  // the next step's number and modulation rows. The action-in projection, which follows, lets the kernels after
+  // it start only once it has waited for this one, so they may read the rows before their own waits
+  if (threadIdx.x == 0) p.cur_k[b] = k + 1;
+  if (k < p.n_steps)
+    for (int i = threadIdx.x; i < p.H; i += blockDim.x) p.cur_tau[b * p.H + i] = p.tau[((size_t)k * p.B + b) * p.H + i];
 }
 
 void launch_euler_prepare() {
@@ -711,8 +722,7 @@ void launch_euler(const EulerArgs& a, cudaStream_t s) {
 }
 
 __global__ void begin_kernel(const float* noise, float* x, float* g, float* u, int n, int* nonfinite,
-                             int* evals, unsigned long long* stamps) {
-  pdl_trigger();
+                             int* evals, unsigned long long* stamps, int* cur_k, int B, int* cur_tau, const int* tau, int M) {
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) {
@@ -720,6 +730,8 @@ __global__ void begin_kernel(const float* noise, float* x, float* g, float* u, i
     *evals = 0;
     stamps[0] = global_ns();
   }
+  if (i < B) cur_k[i] = 1;
+  if (i < M) cur_tau[i] = tau[i];
   if (i < n) {
     const float v = noise[i];
     x[i] = v;
@@ -729,8 +741,9 @@ __global__ void begin_kernel(const float* noise, float* x, float* g, float* u, i
 }
 
 void launch_begin(const float* noise, float* x, float* g, float* u, int n, int* nonfinite, int* evals,
-                  unsigned long long* stamps, cudaStream_t s) {
-  launch_k(begin_kernel, dim3((n + 255) / 256), dim3(256), 0, s, noise, x, g, u, n, nonfinite, evals, stamps);
+                  unsigned long long* stamps, int* cur_k, int B, int* cur_tau, const int* tau, int M, cudaStream_t s) {
+  launch_k(begin_kernel, dim3((n + 255) / 256), dim3(256), 0, s, noise, x, g, u, n, nonfinite, evals, stamps, cur_k, B, cur_tau,
+           tau, M);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -121,6 +121,7 @@ struct uad_ctx {
   int* nonfinite = nullptr;
   int* evals = nullptr;
   unsigned long long* stamps = nullptr;
+  int *cur_k = nullptr, *cur_tau = nullptr;   // the running step's number per robot and modulation row per token
 
   // the finished chunk's status words, copied back in one batch of asynchronous copies (pinned)
   struct ChunkStatus { int derr, nonfinite, evals, pad; unsigned long long stamps[kFlagStride]; };
@@ -144,7 +145,9 @@ struct uad_ctx {
 
   cudaStream_t worker = nullptr;
   cudaEvent_t ev_in = nullptr, ev_done = nullptr;
-  std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;   // (robots, N*, persistent kernel)
+  // (robots, N*, persistent kernel): the whole chunk on the persistent kernel, else as many steps as
+  // graph_steps allows, launched until N* are done
+  std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
 
   // in-flight chunk
   bool in_flight = false;
@@ -629,8 +632,17 @@ bool chunk_uses_step(const uad_ctx* c, int B, int max_shift) {
   return step_path(c, B) && max_shift <= kStepMaxShift && B * c->a.chunk_len + max_shift <= kStepMaxRows;
 }
 
-// Enqueue every kernel of one chunk (begin + n_steps evaluations) for B robots.
-void enqueue_chunk(uad_ctx* c, int B, int n_steps, bool step, cudaStream_t s) {
+// Enqueue a chunk's first kernel, which sets up the state and step 1.
+void enqueue_begin(uad_ctx* c, int B, int n_steps, cudaStream_t s) {
+  const int H = c->a.chunk_len, D = c->a.action_dim, M = B * H;
+  const int* tau = reinterpret_cast<const int*>(c->plan_dev + plan_layout(n_steps, B, H, D).tau);
+  Mark mk(c, s, "begin", 12.0 * M * D, 0);
+  launch_begin(c->noise, c->x, c->g, c->u, M * D, c->nonfinite, c->evals, c->stamps, c->cur_k, B, c->cur_tau, tau, M, s);
+}
+
+// Enqueue `count` evaluations and step epilogues of a chunk of n_steps for B robots: all n_steps of them on the
+// persistent kernel; any number on the per-operation kernels, whose steps are alike (the device counts them).
+void enqueue_steps(uad_ctx* c, int B, int n_steps, int count, bool step, cudaStream_t s) {
   const uad_arch& a = c->a;
   const int H = a.chunk_len, D = a.action_dim, W = a.width, M = B * H, F = a.mlp_dim;
   const int dt = a.dtype;
@@ -640,7 +652,6 @@ void enqueue_chunk(uad_ctx* c, int B, int n_steps, bool step, cudaStream_t s) {
   const int W6 = 6 * W;
   const bool dit = a.kind == UAD_KIND_DIT;
 
-  { Mark mk(c, s, "begin", 12.0 * M * D, 0); launch_begin(c->noise, c->x, c->g, c->u, M * D, c->nonfinite, c->evals, c->stamps, s); }
   if (step) {
     // the persistent kernel's accumulators are zero between uses; clearing them per chunk keeps
     // a chunk that ended in an error from leaking into the next one
@@ -652,12 +663,13 @@ void enqueue_chunk(uad_ctx* c, int B, int n_steps, bool step, cudaStream_t s) {
     cudaMemsetAsync(p.acc_d, 0, R * W * 4, s);
   }
   PendingResid pend;
-  for (int k = 1; k <= n_steps; ++k) {
-    const int* tr = tau + (size_t)(k - 1) * M;
+  for (int k = 1; k <= count; ++k) {
+    const int* tr = step ? tau + (size_t)(k - 1) * M : c->cur_tau;
     // step epilogue (Euler, TR, release, GAC): its own kernel, or the persistent kernel's end
     EulerArgs ea;
     ea.B = B; ea.H = H; ea.D = D; ea.k = k;
-    ea.plan = plan + (size_t)(k - 1) * M;
+    ea.plan = step ? plan + (size_t)(k - 1) * M : plan;
+    if (!step) { ea.cur_k = c->cur_k; ea.cur_tau = c->cur_tau; ea.tau = tau; ea.n_steps = n_steps; }
     ea.gstep = reinterpret_cast<const float*>(c->plan_dev + PL.gstep);
     ea.last_step = reinterpret_cast<const int*>(c->plan_dev + PL.last);
     ea.tail_count = reinterpret_cast<const int*>(c->plan_dev + PL.tailc);
@@ -833,6 +845,17 @@ int launches_per_step(const uad_ctx* c, int B) {
     attn = attn_tc_use_two_pass(t) ? 1 : 2;
   }
   return (6 + attn) * a.n_layers + 4 + (a.kind == UAD_KIND_CONCAT ? 4 : 0);
+}
+
+// Steps in a graph of the per-operation kernels: the most that divide the chunk's and stay near 256 launches.
+// Building a graph takes about 2 us a launch (pi0-like, 10 steps: 3 ms, more than a third of the chunk) and a
+// control loop pays it whenever a new batch or step count comes up; launching one per step costs the GPU a gap
+// of a few us, which short steps would feel.
+int graph_steps(const uad_ctx* c, int B, int n_steps) {
+  int g = 1;
+  for (int d = 1; d <= n_steps; ++d)
+    if (n_steps % d == 0 && d * launches_per_step(c, B) <= 256) g = d;
+  return g;
 }
 
 }  // namespace
@@ -1128,6 +1151,8 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
   TRY(dalloc_t(c, &c->nonfinite, 1));
   TRY(dalloc_t(c, &c->evals, 1));
   TRY(dalloc_t(c, &c->stamps, kFlagStride));
+  TRY(dalloc_t(c, &c->cur_k, (size_t)a.max_batch));
+  TRY(dalloc_t(c, &c->cur_tau, M));
   c->plan_bytes_cap = plan_layout(kMaxSteps, a.max_batch, H, D).total;
   TRY(dalloc(c, (void**)&c->plan_dev, c->plan_bytes_cap));
   CK(cudaHostAlloc((void**)&c->plan_host, c->plan_bytes_cap, cudaHostAllocDefault));
@@ -1362,11 +1387,12 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
   CK(cudaMemcpyAsync(c->noise, noise, (size_t)M * D * 4, cudaMemcpyDefault, s));
   if (c->use_graphs && !profile) {
     const auto key = std::make_tuple(B, steps, use_step ? 1 : 0);
+    const int per = use_step ? steps : graph_steps(c, B, steps);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
       cudaGraph_t g = nullptr;
       CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-      enqueue_chunk(c, B, steps, use_step, s);
+      enqueue_steps(c, B, steps, per, use_step, s);
       cudaError_t e = cudaStreamEndCapture(s, &g);
       if (e != cudaSuccess) return fail(c, UAD_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
       cudaGraphExec_t ex = nullptr;
@@ -1375,7 +1401,8 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
       if (e != cudaSuccess) return fail(c, UAD_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
       it = c->graphs.emplace(key, ex).first;
     }
-    CK(cudaGraphLaunch(it->second, s));
+    enqueue_begin(c, B, steps, s);
+    for (int k = 0; k < steps; k += per) CK(cudaGraphLaunch(it->second, s));
   } else if (profile) {
     // capture with an event-record node around every kernel, so that the event times are
     // GPU timestamps between graph nodes (no host launch gaps)
@@ -1393,7 +1420,8 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
     }
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    enqueue_chunk(c, B, steps, use_step, s);
+    enqueue_begin(c, B, steps, s);
+    enqueue_steps(c, B, steps, steps, use_step, s);
     cudaError_t e = cudaStreamEndCapture(s, &g);
     c->prof_on = false;
     if (e != cudaSuccess) return fail(c, UAD_ECUDA, "profile capture failed: %s", cudaGetErrorString(e));
@@ -1405,7 +1433,8 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
     cudaGraphExecDestroy(ex);
     if (e != cudaSuccess) return fail(c, UAD_ECUDA, "profile launch failed: %s", cudaGetErrorString(e));
   } else {
-    enqueue_chunk(c, B, steps, use_step, s);
+    enqueue_begin(c, B, steps, s);
+    enqueue_steps(c, B, steps, steps, use_step, s);
     CK(cudaGetLastError());
   }
   CK(cudaEventRecord(c->ev_done, s));

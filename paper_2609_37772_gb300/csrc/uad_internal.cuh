@@ -161,6 +161,13 @@ struct EulerArgs {
   int* nonfinite = nullptr;
   int* evals = nullptr;                  // velocity evaluations consumed this chunk
   unsigned long long* stamps = nullptr;  // [UAD_MAX_STEPS + 1], [0] = start
+  // per-operation path: the step is counted on the device, so that every step is the same sequence of launches;
+  // k and plan then come from cur_k (plan: the first step's), and the kernel sets up the next step
+  int* cur_k = nullptr;                  // [B] the step that runs
+  int* cur_tau = nullptr;                // [B][H] its modulation rows: kernels read them before their waits, from L2 (__ldcg;
+                                         // an SM's L1 may still hold the previous step's)
+  const int* tau = nullptr;              // [n_steps][B][H] every step's
+  int n_steps = 0;
 };
 
 // kernels_simt.cu
@@ -172,8 +179,10 @@ void launch_attention(const AttnArgs& a, cudaStream_t s);
 void launch_attention_prepare();   // opt in to > 48 KB dynamic shared memory on the current device
 void launch_euler(const EulerArgs& a, cudaStream_t s);
 void launch_euler_prepare();   // shared memory for H x D GAC terms (up to 256 x 64)
+// Chunk state from the noise (n = M D values), counters cleared; step 1's count (B robots) and modulation
+// rows (M tokens).
 void launch_begin(const float* noise, float* x, float* g, float* u, int n, int* nonfinite, int* evals,
-                  unsigned long long* stamps, cudaStream_t s);
+                  unsigned long long* stamps, int* cur_k, int B, int* cur_tau, const int* tau, int M, cudaStream_t s);
 // dst[(n * mult + off) * K + k] = src[k * N + n]: transpose [K][N] -> rows of K, convert dtype
 void launch_relayout(const float* src, int K, int N, void* dst, int dtype, int mult, long long off,
                      cudaStream_t s);
