@@ -57,20 +57,22 @@ __device__ __forceinline__ void load4(float* dst, const void* base, long long of
 }
 
 // ------------------------------------------------------------------------------------------
-// GEMM: out[m][n] = epi(sum_k A[m][k] * Wt[n][k]). A CTA of eight warps owns a BM x BN tile; WM x WN
+// GEMM: out[m][n] = epi(sum_k A[m][k] * Wt[n][k]). A CTA of eight warps (16 for the larger tiles, whose grids
+// leave an SM one CTA) owns a BM x BN tile; WM x WN
 // warps cover it and KS groups of them each own a share of every K chunk, so that a tile of 16
-// tokens still keeps eight warps busy; the groups' sums are added in group order (deterministic).
+// tokens still keeps them all busy; the groups' sums are added in group order (deterministic).
 // A lane owns BM / WM / 8 rows x BN / WN / 4 columns and reads four k at a time from rows that lie
 // K-contiguous in shared memory (pitch KC + 4: no bank conflicts), as the copies bring them. The
 // first chunks of the weights, which no kernel of the loop writes, are requested before the wait for
 // the kernel that writes A. Bound by the latency of its chain with few rows and by FFMA issue with
 // many. Against one 64 x 64 tile per CTA with K in series (4 CTAs for 16 rows x 256 outputs): tiny
-// fp32 expert, down projection (K = 1024) of 16 rows 75 -> 11 us, of 512 rows 93 -> 20 us.
+// fp32 expert, down projection (K = 1024) of 16 rows 75 -> 11 us, of 512 rows 93 -> 17 us (20 us with eight
+// warps: two a scheduler do not hide the shared-memory loads).
 // ------------------------------------------------------------------------------------------
-template <int BM_, int BN_, int WM_, int WN_, int KC_, int ST_>
+template <int THREADS_, int BM_, int BN_, int WM_, int WN_, int KC_, int ST_>
 struct FfTile {
-  static constexpr int BM = BM_, BN = BN_, WM = WM_, WN = WN_, KC = KC_, ST = ST_;
-  static constexpr int KS = 8 / (WM * WN), RM = BM / WM / 8, RN = BN / WN / 4, PITCH = KC + 4;
+  static constexpr int THREADS = THREADS_, BM = BM_, BN = BN_, WM = WM_, WN = WN_, KC = KC_, ST = ST_;
+  static constexpr int KS = THREADS / 32 / (WM * WN), RM = BM / WM / 8, RN = BN / WN / 4, PITCH = KC + 4;
   static constexpr int STAGE = (BM + BN) * PITCH;          // floats
   static constexpr int RPITCH = BN + 4;                    // reduction rows
   // shared memory of a K that takes `chunks` chunks: no more than it uses, so that the next kernel's
@@ -80,12 +82,12 @@ struct FfTile {
     return (pipe > red ? pipe : red) * sizeof(float);
   }
 };
-using FfSmall = FfTile<16, 16, 1, 1, 256, 4>;
-using FfMid = FfTile<32, 32, 1, 1, 256, 2>;
-using FfWide = FfTile<64, 64, 2, 2, 64, 3>;
+using FfSmall = FfTile<256, 16, 16, 1, 1, 256, 4>;
+using FfMid = FfTile<512, 32, 32, 1, 1, 256, 2>;
+using FfWide = FfTile<512, 64, 64, 2, 2, 64, 3>;
 
 template <int AD, int WD, class T>
-__global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
+__global__ void __launch_bounds__(T::THREADS) gemm_ffma_kernel(GemmArgs p) {
   extern __shared__ __align__(16) float fsm[];
   constexpr int KC = T::KC, PITCH = T::PITCH, ST = T::ST, RM = T::RM, RN = T::RN;
   const int m0 = blockIdx.y * T::BM, n0 = blockIdx.x * T::BN, K = p.K;
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
   const auto load_w = [&](int c) {
     float* dst = fsm + (c % ST) * T::STAGE + T::BM * PITCH;
 #pragma unroll 4
-    for (int e = tid; e < T::BN * (KC / 4); e += 256) {
+    for (int e = tid; e < T::BN * (KC / 4); e += T::THREADS) {
       const int r = e / (KC / 4), c4 = e % (KC / 4), n = n0 + r, k = c * KC + 4 * c4;
       if (n < p.N && k < K) load4<WD>(dst + r * PITCH + 4 * c4, p.W, (long long)n * K + k, K - k, vw);
       else *reinterpret_cast<float4*>(dst + r * PITCH + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
   const auto load_a = [&](int c) {
     float* dst = fsm + (c % ST) * T::STAGE;
 #pragma unroll 4
-    for (int e = tid; e < T::BM * (KC / 4); e += 256) {
+    for (int e = tid; e < T::BM * (KC / 4); e += T::THREADS) {
       const int r = e / (KC / 4), c4 = e % (KC / 4), m = m0 + r, k = c * KC + 4 * c4;
       if (m < p.M && k < K) load4<AD>(dst + r * PITCH + 4 * c4, p.A, (long long)m * p.lda + k, K - k, va);
       else *reinterpret_cast<float4*>(dst + r * PITCH + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -116,10 +118,10 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
   for (int c = 0; c < ST && c < nch; ++c) load_w(c);
   // residual update: this thread's first outputs' gates before the wait, their residual values right after
   // it, so that neither is fetched at the end
-  constexpr int EP = T::BM * T::BN / 256 < 4 ? T::BM * T::BN / 256 : 4;
+  constexpr int EP = T::BM * T::BN / T::THREADS < 4 ? (T::BM * T::BN + T::THREADS - 1) / T::THREADS : 4;
   float gate[EP], res[EP];
   const auto out_of = [&](int u, int& m, int& n) {
-    const int e = tid + 256 * u;
+    const int e = tid + T::THREADS * u;
     m = m0 + e / T::BN;
     n = n0 + e % T::BN;
     return m < p.M && n < p.N;
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
     return s;
   };
   if (p.epi == EPI_GEGLU) {
-    for (int e = tid; e < T::BM * T::BN / 2; e += 256) {
+    for (int e = tid; e < T::BM * T::BN / 2; e += T::THREADS) {
       const int ml = e / (T::BN / 2), nl = 2 * (e % (T::BN / 2)), m = m0 + ml, n = n0 + nl;
       if (m < p.M && n + 1 < p.N)
         store_as(p.out, (long long)m * p.ldo + n / 2, gelu_tanh_f(total(ml, nl)) * total(ml, nl + 1), p.out_dtype);
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
       if (out_of(u, m, n)) p.resid[(long long)m * p.ldr + n] = fmaf(gate[u], total(m - m0, n - n0) + (p.bias ? p.bias[n] : 0.f), res[u]);
     }
   }
-  for (int e = tid + (p.epi == EPI_RESID_GATE ? 256 * EP : 0); e < T::BM * T::BN; e += 256) {
+  for (int e = tid + (p.epi == EPI_RESID_GATE ? T::THREADS * EP : 0); e < T::BM * T::BN; e += T::THREADS) {
     const int ml = e / T::BN, nl = e % T::BN, m = m0 + ml, n = n0 + nl;
     if (m >= p.M || n >= p.N) continue;
     float r = total(ml, nl) + (p.bias ? p.bias[n] : 0.f);
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(GemmArgs p) {
 
 template <int AD, int WD, class T>
 void launch_tile(const GemmArgs& a, cudaStream_t s) {
-  launch_k(gemm_ffma_kernel<AD, WD, T>, dim3((a.N + T::BN - 1) / T::BN, (a.M + T::BM - 1) / T::BM), dim3(256),
+  launch_k(gemm_ffma_kernel<AD, WD, T>, dim3((a.N + T::BN - 1) / T::BN, (a.M + T::BM - 1) / T::BM), dim3(T::THREADS),
            T::smem((a.K + T::KC - 1) / T::KC), s, a);
 }
 
