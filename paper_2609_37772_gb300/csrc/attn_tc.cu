@@ -481,43 +481,49 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
 }
 
 // Merge the key chunks of every query row: o = sum_c w_c O_c / sum_c w_c l_c, w_c = 2^((m_c - M) c2).
-// One CTA per (query row, robot-group), one thread per two head dims (dh / 2 threads: the grid
-// fits the GPU in one wave, 8-byte loads); every partial is loaded before any arithmetic. Writes
-// o [(b*H + i)][(g*G + j)*dh + d] in bf16.
-__global__ void attn_combine_kernel(AttnTcArgs p, int n_chunks) {
+// A thread owns four head dims of one row, a CTA of 256 threads 1024 / DH rows, so that the whole grid starts
+// at once and the next kernel's CTAs can come in beside it (one row a CTA of 128 threads held them back);
+// every partial is loaded before any arithmetic. 18 layers, 400 rows of 256, 7 chunks: 717 -> 703 us per evaluation.
+// Writes o [(b*H + i)][(g*G + j)*dh + d] in bf16.
+__global__ void __launch_bounds__(256) attn_combine_kernel(AttnTcArgs p, int n_chunks) {
   constexpr int MAXC = kMaxKeyChunks;
   pdl_trigger();
-  pdl_wait();
-  const int r = blockIdx.x, bg = blockIdx.y, d = 2 * threadIdx.x, DH = 2 * blockDim.x;
+  const int DH = p.head_dim, tpr = DH / 4, r = blockIdx.x * (256 / tpr) + threadIdx.x / tpr, bg = blockIdx.y;
+  const int d = 4 * (threadIdx.x % tpr);
+  if (r >= p.rows) return;
   const int b = bg / p.n_kv_heads, g = bg % p.n_kv_heads;
+  pdl_wait();
   float m[MAXC], l[MAXC];
-  float2 o[MAXC];
+  float4 o[MAXC];
 #pragma unroll
   for (int c = 0; c < MAXC; ++c) {
     if (c < n_chunks) {
       const size_t idx = ((size_t)bg * n_chunks + c) * p.r_pad + r;
       m[c] = p.part_ml[idx * 2];
       l[c] = p.part_ml[idx * 2 + 1];
-      o[c] = *reinterpret_cast<const float2*>(p.part_o + idx * DH + d);
+      o[c] = *reinterpret_cast<const float4*>(p.part_o + idx * DH + d);
     }
   }
   float M = -INFINITY;
 #pragma unroll
   for (int c = 0; c < MAXC; ++c)
     if (c < n_chunks) M = fmaxf(M, m[c]);
-  float L = 0.f, ax = 0.f, ay = 0.f;
+  float L = 0.f;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
   for (int c = 0; c < MAXC; ++c) {
     if (c < n_chunks) {
       const float w = exp2f((m[c] - M) * p.scale_log2);
       L = fmaf(w, l[c], L);
-      ax = fmaf(w, o[c].x, ax);
-      ay = fmaf(w, o[c].y, ay);
+      a.x = fmaf(w, o[c].x, a.x);
+      a.y = fmaf(w, o[c].y, a.y);
+      a.z = fmaf(w, o[c].z, a.z);
+      a.w = fmaf(w, o[c].w, a.w);
     }
   }
   const int j = r / p.H, i = r % p.H;
-  *reinterpret_cast<__nv_bfloat162*>(p.out + ((size_t)b * p.H + i) * p.out_ld + (size_t)(g * p.group + j) * DH + d) =
-      __floats2bfloat162_rn(ax / L, ay / L);
+  *reinterpret_cast<uint2*>(p.out + ((size_t)b * p.H + i) * p.out_ld + (size_t)(g * p.group + j) * DH + d) =
+      make_uint2(pack_bf16(a.x / L, a.y / L), pack_bf16(a.z / L, a.w / L));
 }
 
 // Prefix K/V of one robot (fp32 or bf16 source [L][P][Hkv][dh], 16-byte aligned) into the K and Vt
@@ -704,8 +710,8 @@ void launch_attn_tc(const AttnTcMaps& maps, const AttnTcArgs& a, cudaStream_t s)
     else if (sp == 2) launch_k(attn_tc_kernel<256, 128>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
     else launch_k(attn_tc_kernel<256, 64>, grid, dim3(128), smem, s, maps.q, maps.k, vt, a);
   }
-  launch_k(attn_combine_kernel, dim3(a.rows, a.batch * a.n_kv_heads), dim3(a.head_dim / 2), 0, s, a,
-           attn_tc_chunks(a.n_keys));
+  const int rows = 1024 / a.head_dim;
+  launch_k(attn_combine_kernel, dim3((a.rows + rows - 1) / rows, bg), dim3(256), 0, s, a, kc);
 }
 
 void launch_kv_prefix(const void* k, const void* v, int src_dtype, const AttnTcArgs& a, int robot, cudaStream_t s) {
