@@ -450,7 +450,8 @@ void launch_norm(const NormArgs& a, cudaStream_t s) {
 // What bounds it is latency, half of it instruction fetch: a kernel whose code is not in the SM's
 // instruction cache runs at a dozen cycles an instruction. The prefix keys and values, which no
 // kernel of the loop writes, are loaded before the wait for the previous kernel, and a rehearsal pass
-// over them (its results dropped) brings the code in while the CTA would idle.
+// over them (its results dropped) brings the code in while the CTA would idle. A CTA with several tiles
+// loads the next one's keys and values into registers while it works on the current one.
 constexpr int kFewDh = 64, kFewQ = 16, kFewKT = 64, kFewCluster = 8;
 constexpr int kFewPitch = kFewDh + 8;     // bf16 rows of V and P: ldmatrix without bank conflicts
 constexpr int kFewSPitch = kFewKT + 4;    // fp32 rows of scores and partial outputs
@@ -463,9 +464,18 @@ struct FewSmem {
   float part[1];                          // [CTAs of the cluster][16][kFewSPitch]: O, then max and sum
 };
 static size_t few_smem_bytes(int c) { return sizeof(FewSmem) + (c > 1 ? (size_t)c * kFewQ * kFewSPitch * 4 : 0); }
-static int few_cluster(int n_keys) {
-  const int t = (n_keys + kFewKT - 1) / kFewKT;
-  return t < kFewCluster ? t : kFewCluster;
+// CTAs that share a query block: one a key tile while the whole grid is one CTA an SM. Past that a cluster
+// costs more than it gives (its CTAs start together, beside the previous kernel's, and meet twice), and the
+// CTAs walk their tiles alone. 24 heads, 16 queries, 264 keys, us per evaluation of the 16-layer expert:
+// 1 robot 795 with 5 CTAs a block (810 with 4); 4 robots 1200 with 5 or 3, 1163 with 2, 1112 with 1.
+static int few_cluster(int n_keys, long long blocks) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int c = (n_keys + kFewKT - 1) / kFewKT;
+  if (c > kFewCluster) c = kFewCluster;
+  while (c > 1 && c * blocks > sms) --c;
+  return c;
 }
 
 __device__ __forceinline__ void ldsm4(uint32_t* r, const void* p) {
@@ -502,27 +512,30 @@ __global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
     if (j < n_keys) return static_cast<const __nv_bfloat16*>(chunk) + (long long)(b * p.H + j - p.P) * p.kc_ld + g * kFewDh;
     return nullptr;
   };
-  uint32_t kf[8];
-  const auto load_tile = [&](int t) {
+  // a tile's keys and values wait in registers while the tile before it is worked on
+  uint32_t kn[8];
+  uint4 vn[2];
+  const int vj = tid >> 2, vcol = 16 * (tid & 3);   // a quarter of a value row each
+  const auto fetch = [&](int t) {
     const __nv_bfloat16* kr = row_of(p.kp, p.kc, t * kFewKT + 8 * warp + gr);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) kf[u] = kr ? __ldcg(reinterpret_cast<const unsigned*>(kr + 8 * u + tc)) : 0u;
-    const int j = tid >> 2, c = 16 * (tid & 3);   // a quarter of a value row each
-    const __nv_bfloat16* vr = row_of(p.vp, p.vc, t * kFewKT + j);
+    for (int u = 0; u < 8; ++u) kn[u] = kr ? __ldcg(reinterpret_cast<const unsigned*>(kr + 8 * u + tc)) : 0u;
+    const __nv_bfloat16* vr = row_of(p.vp, p.vc, t * kFewKT + vj);
     const uint4 zero = make_uint4(0, 0, 0, 0);
-    const uint4 v0 = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + c)) : zero;
-    const uint4 v1 = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + c + 8)) : zero;
-    *reinterpret_cast<uint4*>(sm.v + j * kFewPitch + c) = v0;
-    *reinterpret_cast<uint4*>(sm.v + j * kFewPitch + c + 8) = v1;
+    vn[0] = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + vcol)) : zero;
+    vn[1] = vr ? __ldcg(reinterpret_cast<const uint4*>(vr + vcol + 8)) : zero;
   };
   const bool early = (rank + 1) * kFewKT <= p.P;   // this CTA's first tile is prefix keys alone
-  if (early) load_tile(rank);
+  if (early) fetch(rank);
 
   float o[4];
   const int q = tid >> 4, kg = tid & 15;           // softmax: query q, keys 4 kg .. 4 kg + 3
 #pragma unroll 1
   for (int pass = early ? 0 : 1; pass < 2; ++pass) {
-    if (pass) pdl_wait();
+    if (pass) {
+      pdl_wait();
+      if (!early) fetch(rank);
+    }
     if (tid < kFewQ) {
       sm.m[tid] = -INFINITY;
       sm.l[tid] = 0.f;
@@ -537,7 +550,12 @@ __global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
         qf[ks][e] = (e & 1 ? q1 : q0) ? __ldcg(reinterpret_cast<const unsigned*>(qrow + (e & 1) * 8ll * p.q_ld + 16 * ks + 8 * (e >> 1))) : 0u;
 #pragma unroll 1
     for (int t = rank; t < nt; t += C) {
-      if (pass && (t != rank || !early)) load_tile(t);
+      uint32_t kf[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) kf[u] = kn[u];
+      *reinterpret_cast<uint4*>(sm.v + vj * kFewPitch + vcol) = vn[0];
+      *reinterpret_cast<uint4*>(sm.v + vj * kFewPitch + vcol + 8) = vn[1];
+      if (pass && t + C < nt) fetch(t + C);
       float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int ks = 0; ks < 4; ++ks) mma16816(c, qf[ks], kf + 2 * ks);
@@ -680,7 +698,7 @@ void launch_attention_prepare() {
 
 void launch_attention(const AttnArgs& a, cudaStream_t s) {
   if (attn_few_ok(a)) {
-    const int C = few_cluster(a.P + (a.kc ? a.H : 0));
+    const int C = few_cluster(a.P + (a.kc ? a.H : 0), (long long)((a.H + kFewQ - 1) / kFewQ) * a.n_heads * a.B);
     launch_cluster(attn_few_kernel, dim3((a.H + kFewQ - 1) / kFewQ * C, a.n_heads, a.B), dim3(256), few_smem_bytes(C), C, s, a, C);
     return;
   }

@@ -714,6 +714,21 @@ def test_dit_prefix_projection_lengths(prefix, robots):
         c.close()
 
 
+@pytest.mark.parametrize("chunk,prefix,robots", [(16, 600, 1), (24, 200, 1), (16, 130, 9), (17, 257, 10), (16, 1100, 13)])
+def test_dit_attention_tiles_and_clusters(chunk, prefix, robots):
+    """The few-query attention where a CTA walks several key tiles: more tiles than a cluster has
+    CTAs, two query blocks, and (with more robots) smaller clusters down to a CTA alone with all
+    tiles, the last of them partly filled."""
+    a = ARCHS["dit_small"].replace(name=f"dit_small_c{chunk}_p{prefix}", chunk_len=chunk, prefix_len=prefix)
+    c = Case(a, B=robots, seed=54)
+    try:
+        noise = make_noise(a, batch=robots, seed=54)
+        bud = np.stack([group_budgets(chunk, [(0, 3, 1), (4, chunk - 1, 2)])] * robots)
+        check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL["bf16"])
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("prefix", [1, 63, 64, 72, 129])
 def test_prefix_transposition_lengths(prefix):
     """Prefix keys and values into the attention caches at the edges of the 64-position tiles and of
