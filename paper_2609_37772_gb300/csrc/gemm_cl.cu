@@ -63,6 +63,11 @@ __host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits) {
   return splits > 1 ? (size_t)((rows + splits - 1) / splits) * splits * kBM * 4 : 0;
 }
 
+// E: the epilogue this instantiation is for, or, read from the arguments, kAny: any; kPlain: any but EPI_QKV_TC
+// and EPI_GEGLU. A kernel whose code is not in the SM's instruction cache runs at a dozen cycles an instruction,
+// so it matters which projections share code (TcGemmArgs::cl_code).
+constexpr int kAny = -2, kPlain = -1;
+template <int E>
 __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -125,7 +130,10 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       for (int i = issued - ring > 0 ? issued - ring : 0; i < issued; ++i) wait_bar(full + i % ring, (i / ring) & 1, p.err, 72);
     }
     __syncwarp();
-    if (S > 1) cluster_wait();
+    if (S > 1) {
+      cluster_wait();
+      cluster_arrive();
+    }
   } else if (warp == kConsWarps + 1) {
     // ---- MMA issuer ----
     if (lane == 0) {
@@ -143,14 +151,18 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       mma_commit(done);
     }
     __syncwarp();
-    if (S > 1) cluster_wait();
+    if (S > 1) {
+      cluster_wait();
+      cluster_arrive();
+    }
   } else {
     // ---- epilogue warps ----
     // residual update: this warp's first tokens' gates and residual rows are requested before the
     // MMAs are waited for
     constexpr int U = 4;
     const int n = nt * kBM + 4 * lane;   // this lane's four output features
-    const bool resid = p.epi == EPI_RESID_H;
+    const int epi = E >= 0 ? E : p.epi;
+    const bool resid = epi == EPI_RESID_H;
     const bool vec = reinterpret_cast<uintptr_t>(p.out) % 16 == 0 && p.ldo % 4 == 0;   // a caller's pointer may not be
     float4 hv[U], gv[U], bias = make_float4(0.f, 0.f, 0.f, 0.f);
     if (p.bias) {
@@ -177,7 +189,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       }
     };
     // RoPE: likewise the (cos, sin) of this warp's first tokens (constant), kept where the residual rows would be
-    const bool qk = p.epi == EPI_QKV_TC && p.qkv.rope && nt * kBM < p.qkv.qd + p.qkv.kvd;
+    const bool qkv = E == EPI_QKV_TC || (E == kAny && p.epi == EPI_QKV_TC);
+    const bool qk = qkv && p.qkv.rope && nt * kBM < p.qkv.qd + p.qkv.kvd;
     const auto load_cs = [&](int t) {
       const int sn = n < p.qkv.qd ? n : n - p.qkv.qd, r = sn % p.qkv.dh;
 #pragma unroll
@@ -213,6 +226,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       }
     }
     const bool all = S == 1 || cnt == 0 || wait_bar(got, 0, p.err, 75);
+    __syncwarp();
+    if (S > 1) cluster_arrive();   // this CTA's rows are here: once every CTA says so, none reads another's memory
     if (ok && all) {
       for (int t = warp; t < cnt; t += kConsWarps * U) {
         if (resid && t != warp) {
@@ -238,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
           v.y += bias.y;
           v.z += bias.z;
           v.w += bias.w;
-          switch (p.epi) {
+          switch (epi) {
             case EPI_RESID_H: {
               float4 h = hv[u];
               h.x = fmaf(gv[u].x, v.x, h.x);
@@ -248,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
               *reinterpret_cast<float4*>(p.resid + (size_t)m * p.N + n) = h;
               break;
             }
-            case EPI_GEGLU: {
+            case EPI_GEGLU: if constexpr (E == EPI_GEGLU || E == kAny) {
               // rows 2i (gate) and 2i + 1 (up) give output i
               const size_t off = (size_t)m * p.ldo + n / 2;
               const uint32_t pk = pack_bf16(gelu_tanh_approx(v.x) * v.y, gelu_tanh_approx(v.z) * v.w);
@@ -256,9 +271,9 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
                 *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(p.out) + off) = pk;
               else
                 *reinterpret_cast<float2*>(static_cast<float*>(p.out) + off) = make_float2(gelu_tanh_f(v.x) * v.y, gelu_tanh_f(v.z) * v.w);
-              break;
             }
-            case EPI_QKV_TC: {
+            break;
+            case EPI_QKV_TC: if constexpr (E == EPI_QKV_TC || E == kAny) {
               const QkvTcOut& o = p.qkv;
               const int b = m / o.H, i = m - b * o.H;
               if (nt * kBM < o.qd + o.kvd) {
@@ -278,15 +293,11 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
                   *reinterpret_cast<uint2*>(dst + r) = pack4(v.x, v.y, v.z, v.w);
                 }
               } else {
-                const int sn = n - o.qd - o.kvd, g = sn / o.dh, d = sn % o.dh;   // four dims of one head
-                __nv_bfloat16* dst = o.vtcache + ((((size_t)b * o.L + o.layer) * o.Hkv + g) * o.dh + d) * o.NKp + o.P + i;
-                dst[0] = __float2bfloat16_rn(v.x);
-                dst[o.NKp] = __float2bfloat16_rn(v.y);
-                dst[2 * (size_t)o.NKp] = __float2bfloat16_rn(v.z);
-                dst[3 * (size_t)o.NKp] = __float2bfloat16_rn(v.w);
+                // v: into this token's staged row (16-byte pieces swizzled by token), for the writes below
+                *reinterpret_cast<float4*>(T + (size_t)(t0 + tt) * kBM + 4 * (lane ^ (tt & 31))) = v;
               }
-              break;
             }
+            break;
             case EPI_PREFIX_KV: {
               const int w = p.pkv.width, part = nt * kBM / w;   // part = 2 layer + (0 k, 1 v)
               *reinterpret_cast<uint2*>(((part & 1) ? p.pkv.v : p.pkv.k) + ((size_t)(part >> 1) * p.M + m) * w + (n - part * w)) =
@@ -294,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
               break;
             }
             default: {
-              if (p.epi == EPI_BIAS_GELU) v = make_float4(gelu_tanh_f(v.x), gelu_tanh_f(v.y), gelu_tanh_f(v.z), gelu_tanh_f(v.w));
+              if (epi == EPI_BIAS_GELU) v = make_float4(gelu_tanh_f(v.x), gelu_tanh_f(v.y), gelu_tanh_f(v.z), gelu_tanh_f(v.w));
               const size_t off = (size_t)m * p.ldo + n;
               const int ns = p.n_store > 0 ? p.n_store : p.N;   // a narrow projection's padding rows are not stored
               if (!vec || n + 3 >= ns) {
@@ -314,14 +325,23 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         }
       }
     }
+    if (qkv && nt * kBM >= p.qkv.qd + p.qkv.kvd) {
+      // the CTA's v values, tokens fastest over the lanes: Vt holds a head dim's keys contiguously (a 2-byte
+      // store a key and dim straight from the sums: 897 us per evaluation of 18 layers at 200 tokens, so 870)
+      const QkvTcOut& o = p.qkv;
+      named_sync(1, kCons);   // reached by every epilogue warp, also by one whose wait ran out
+      for (int tt = lane; ok && all && tt < cnt; tt += 32) {
+        const int m = m0 + t0 + tt, b = m / o.H;
+        __nv_bfloat16* dst = o.vtcache + (((size_t)b * o.L + o.layer) * o.kvd + (nt * kBM - o.qd - o.kvd)) * o.NKp + o.P + (m - b * o.H);
+        for (int r = warp; r < kBM; r += kConsWarps)
+          dst[(size_t)r * o.NKp] = __float2bfloat16_rn(T[(size_t)(t0 + tt) * kBM + ((r & ~3) ^ (4 * (tt & 31))) + (r & 3)]);
+      }
+    }
   }
   tc_fence_before();
   __syncthreads();
   // a CTA leaves once every CTA has received its rows: until then its own are still being read
-  if (S > 1) {
-    cluster_arrive();
-    cluster_wait();
-  }
+  if (S > 1) cluster_wait();
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kBN));
@@ -358,14 +378,21 @@ static size_t gemm_cl_smem_bytes(int ring, int rows, int splits) {
 constexpr size_t kClSmem = 112 * 1024;   // two CTAs fit an SM
 
 void gemm_cl_prepare() {
-  cudaFuncSetAttribute(gemm_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+  for (const auto k : {gemm_cl_kernel<kAny>, gemm_cl_kernel<kPlain>, gemm_cl_kernel<EPI_QKV_TC>, gemm_cl_kernel<EPI_GEGLU>,
+                       gemm_cl_kernel<EPI_RESID_H>})
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
 }
 
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
   const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, rows = a.M < kBN ? a.M : kBN;
   int ring = per < kTcMaxStages ? per : kTcMaxStages;
   while (gemm_cl_smem_bytes(ring, rows, a.splits) > kClSmem) --ring;   // three slots at least
-  launch_cluster(gemm_cl_kernel, dim3(a.splits, a.N / kBM, (a.M + kBN - 1) / kBN), dim3(kThreads),
+  const bool own = a.cl_code == kClOwn, gated = a.epi == EPI_QKV_TC || a.epi == EPI_GEGLU;
+  const auto kernel = own && a.epi == EPI_QKV_TC ? gemm_cl_kernel<EPI_QKV_TC>
+                      : own && a.epi == EPI_GEGLU ? gemm_cl_kernel<EPI_GEGLU>
+                      : own && a.epi == EPI_RESID_H ? gemm_cl_kernel<EPI_RESID_H>
+                      : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain> : gemm_cl_kernel<kAny>;
+  launch_cluster(kernel, dim3(a.splits, a.N / kBM, (a.M + kBN - 1) / kBN), dim3(kThreads),
                  gemm_cl_smem_bytes(ring, rows, a.splits), a.splits, s, *tmx, a, ring);
 }
 

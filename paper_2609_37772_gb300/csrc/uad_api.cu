@@ -452,6 +452,14 @@ double gemm_bytes(const GemmArgs& g, int wes) {
   return b;
 }
 
+// Which kernels of the few-token form an expert's projections share (instruction cache; us per evaluation): the
+// 16-layer DiT expert, 16 tokens: all by kAny 795, by kPlain 773, residual updates by their own 793. The 18-layer
+// adaptive-RMS expert, 50 / 200 tokens: by kAny 707 / 1037, each by its own 691 / 1019. The two-layer
+// time-concatenating one, whose layers are a smaller part of its loop, 50 / 250 tokens: kAny 84 / 102, own 89 / 102.
+int cl_code(const uad_ctx* c) {
+  return c->a.kind == UAD_KIND_DIT ? kClPlain : c->a.kind == UAD_KIND_ADARMS ? kClOwn : kClAny;
+}
+
 // out = epi(A Wt^T): tensor cores when the weight is tiled, CUDA cores otherwise.
 void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   g.W = w.w;
@@ -464,7 +472,7 @@ void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   t.w_tiled = w.w; t.M = g.M; t.N = g.N; t.K = g.K;
   gemm_tc_plan(g.M, g.N, g.K, c->sms, g.epi, &t);
   t.epi = g.epi; t.out = g.out; t.ldo = g.ldo; t.out_dtype = g.out_dtype; t.bias = g.bias;
-  t.qkv = g.qkv; t.n_store = g.n_store; t.err = c->dev_err;
+  t.qkv = g.qkv; t.n_store = g.n_store; t.err = c->dev_err; t.cl_code = cl_code(c);
   launch_gemm_tc(&c->tmaps.at(g.A), t, s);
 }
 
@@ -491,7 +499,7 @@ void resid_gemm(uad_ctx* c, const Lin& w, GemmArgs g, int gate_off, const float*
     TcGemmArgs t;
     t.w_tiled = w.w; t.M = g.M; t.N = g.N; t.K = g.K; t.epi = EPI_RESID_H; t.ldo = g.N;
     gemm_tc_plan(g.M, g.N, g.K, c->sms, t.epi, &t);
-    t.bias = bias; t.resid = c->h; t.err = c->dev_err; t.tau_row = g.tau_row;
+    t.bias = bias; t.resid = c->h; t.err = c->dev_err; t.tau_row = g.tau_row; t.cl_code = cl_code(c);
     if (gate_off >= 0) { t.gate_tab = c->tab + gate_off; t.gate_stride = c->rowlen; }
     g.epi = EPI_RESID_GATE;
     Mark mk(c, s, name, gemm_bytes(g, c->es), flops);

@@ -216,6 +216,7 @@ struct TcGemmArgs {
   int wide = 0;                    // 1: the persistent wide form (one CTA per SM walking units of
                                    // tn tokens x 128 weight rows x a K range), 0: narrow split-K tiles
   int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)
+  int cl_code = 0;                 //    which projections share its code: kClAny, kClPlain or kClOwn
   int tn = 0;                      // persistent form: tokens per tile (256, 192 or 128)
 };
 // 2-D TMA descriptor of a bf16 activation matrix [rows][K] (64 x 64 boxes, 128-byte swizzle,
@@ -227,6 +228,7 @@ int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form s
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a);
 // gemm_cl.cu: the few-token form (K splits over a cluster), at most kClMaxSplits splits
 constexpr int kClMaxSplits = 8;
+constexpr int kClAny = 0, kClPlain = 1, kClOwn = 2;   // TcGemmArgs::cl_code
 int gemm_cl_splits(int M, int N, int K, int sms);
 bool gemm_cl_serves(int M, int N, int sms);
 void gemm_cl_prepare();
