@@ -1,6 +1,6 @@
 // Few-token tensor-core projection: the K range of an output tile split over a thread-block cluster.
 //
-// out[m][n] = epi(sum_k X[m][k] * Wt[n][k]) for tiles of 128 weight rows x up to 64 tokens. With few
+// out[m][n] = epi(sum_k X[m][k] * Wt[n][k]) for tiles of 128 or 64 weight rows x up to 64 tokens. With few
 // tokens a projection is a short chain of dependent steps (operands, MMAs, the sum over the K splits,
 // the epilogue), so the kernel keeps that sum out of global memory: the S CTAs of a cluster each
 // multiply their share of K into tensor memory, stage the fp32 tile in shared memory and send every
@@ -22,10 +22,9 @@ using namespace ptx;
 
 namespace {
 
-constexpr int kBM = 128, kBN = 64, kBK = 64;
-constexpr int kSlotA = kBM * kBK * 2;            // weights of a k-block: 16 KB
+constexpr int kTileM = 128, kBN = 64, kBK = 64;
+constexpr int kTileBytes = kTileM * kBK * 2;     // a k-block of the tiled weights: 16 KB, its rows 0-63 first
 constexpr int kSlotB = kBN * kBK * 2;            // activations: 8 KB
-constexpr int kSlot = kSlotA + kSlotB;
 constexpr int kConsWarps = 8, kCons = 32 * kConsWarps;
 constexpr int kThreads = kCons + 64;             // + producer warp, + MMA warp
 constexpr unsigned long long kWaitNs = 2000000000ull;
@@ -53,23 +52,26 @@ __device__ __forceinline__ float gelu_tanh_f(float x) {
 __device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) { return make_uint2(pack_bf16(a, b), pack_bf16(c, d)); }
 
 // Where a CTA's shared memory goes: the ring of k-block slots, reused after the MMAs as the staged tile
-// T[token][128]; then the partial rows received from the other CTAs, [rank][owned token][128], apart from
-// the ring, so that they may arrive while this CTA's MMAs still run. `rows`: tokens of the largest tile.
-__host__ __device__ __forceinline__ size_t cl_ring_bytes(int ring, int rows) {
-  const size_t pipe = (size_t)ring * kSlot, tile = (size_t)((rows + 15) / 16 * 16) * kBM * 4;
+// T[token][bm]; then the partial rows received from the other CTAs, [rank][owned token][bm], apart from
+// the ring, so that they may arrive while this CTA's MMAs still run. `rows`: tokens of the largest
+// tile, bm: weight rows of a tile.
+__host__ __device__ __forceinline__ size_t cl_ring_bytes(int ring, int rows, int bm) {
+  const size_t pipe = (size_t)ring * (bm * kBK * 2 + kSlotB), tile = (size_t)((rows + 15) / 16 * 16) * bm * 4;
   return pipe > tile ? pipe : tile;
 }
-__host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits) {
-  return splits > 1 ? (size_t)((rows + splits - 1) / splits) * splits * kBM * 4 : 0;
+__host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits, int bm) {
+  return splits > 1 ? (size_t)((rows + splits - 1) / splits) * splits * bm * 4 : 0;
 }
 
 // E: the epilogue this instantiation is for, or, read from the arguments, kAny: any; kPlain: any but EPI_QKV_TC
 // and EPI_GEGLU. A kernel whose code is not in the SM's instruction cache runs at a dozen cycles an instruction,
 // so it matters which projections share code (TcGemmArgs::cl_code).
 constexpr int kAny = -2, kPlain = -1;
-template <int E>
+template <int E, int kBM>
 __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
   extern __shared__ uint8_t smem_raw[];
+  constexpr int kSlotA = kBM * kBK * 2, kSlot = kSlotA + kSlotB;
+  constexpr int kLanes = kBM / 4, TP = 32 / kLanes;   // lanes that share a token row, rows a warp takes at once
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int S = p.splits, rank = blockIdx.x, nt = blockIdx.y, mt = blockIdx.z;
   const int KC = p.K / kBK, c0 = rank * KC / S, nkb = (rank + 1) * KC / S - c0;
@@ -78,8 +80,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   const int cnt = mcount - t0 < 0 ? 0 : mcount - t0 < per ? mcount - t0 : per;
   float* T = reinterpret_cast<float*>(smem);
   const int rows = p.M < kBN ? p.M : kBN;
-  float* recv = reinterpret_cast<float*>(smem + cl_ring_bytes(ring, rows));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + cl_ring_bytes(ring, rows) + cl_recv_bytes(rows, S));
+  float* recv = reinterpret_cast<float*>(smem + cl_ring_bytes(ring, rows, kBM));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + cl_ring_bytes(ring, rows, kBM) + cl_recv_bytes(rows, S, kBM));
   uint64_t* empty = full + ring;
   uint64_t* done = empty + ring;
   uint64_t* got = done + 1;
@@ -110,11 +112,11 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     // ---- producer ----
     if (lane == 0) {
       const uint64_t pol = policy_evict_first();
-      const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + ((size_t)nt * KC + c0) * kSlotA;
+      const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + ((size_t)(nt * kBM / kTileM) * KC + c0) * kTileBytes + nt * kBM % kTileM * kBK * 2;
       const int first = nkb < ring ? nkb : ring;
       for (int i = 0; i < first; ++i) {
         mbar_expect_tx(full + i, kSlot);
-        bulk_g2s(smem + (size_t)i * kSlot, wt + (size_t)i * kSlotA, kSlotA, full + i, pol);
+        bulk_g2s(smem + (size_t)i * kSlot, wt + (size_t)i * kTileBytes, kSlotA, full + i, pol);
       }
       pdl_wait();
       for (int i = 0; i < first; ++i) tma_2d(smem + (size_t)i * kSlot + kSlotA, &tmx, (c0 + i) * kBK, m0, full + i);
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         const int st = i % ring;
         if (!wait_bar(empty + st, (i / ring - 1) & 1, p.err, 71)) break;
         mbar_expect_tx(full + st, kSlot);
-        bulk_g2s(smem + (size_t)st * kSlot, wt + (size_t)i * kSlotA, kSlotA, full + st, pol);
+        bulk_g2s(smem + (size_t)st * kSlot, wt + (size_t)i * kTileBytes, kSlotA, full + st, pol);
         tma_2d(smem + (size_t)st * kSlot + kSlotA, &tmx, (c0 + i) * kBK, m0, full + st);
       }
       // no copies in flight into shared memory that is reused, or of a CTA that exits
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     // ---- MMA issuer ----
     if (lane == 0) {
       const uint32_t tmem = *tmem_slot;
-      const uint32_t idesc = idesc_m128((mcount + 15) / 16 * 16);
+      const uint32_t idesc = idesc_rows(kBM, (mcount + 15) / 16 * 16);
       const uint64_t ring0 = sw128_desc(su32(smem));
       for (int i = 0; i < nkb; ++i) {
         const int st = i % ring;
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     // residual update: this warp's first tokens' gates and residual rows are requested before the
     // MMAs are waited for
     constexpr int U = 4;
-    const int n = nt * kBM + 4 * lane;   // this lane's four output features
+    const int fl = lane % kLanes, sub = lane / kLanes, n = nt * kBM + 4 * fl;   // this lane's four output features
     const int epi = E >= 0 ? E : p.epi;
     const bool resid = epi == EPI_RESID_H;
     const bool vec = reinterpret_cast<uintptr_t>(p.out) % 16 == 0 && p.ldo % 4 == 0;   // a caller's pointer may not be
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     const auto load_gates = [&](int t) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int tt = t + kConsWarps * u;
+        const int tt = (t + kConsWarps * u) * TP + sub;
         gv[u] = make_float4(1.f, 1.f, 1.f, 1.f);
         if (tt < cnt && p.gate_tab)
           gv[u] = __ldg(reinterpret_cast<const float4*>(p.gate_tab + (size_t)__ldcg(p.tau_row + m0 + t0 + tt) * p.gate_stride + n));
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     const auto load_h = [&](int t) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int tt = t + kConsWarps * u;
+        const int tt = (t + kConsWarps * u) * TP + sub;
         if (tt < cnt) hv[u] = __ldcg(reinterpret_cast<const float4*>(p.resid + (size_t)(m0 + t0 + tt) * p.N + n));
       }
     };
@@ -195,13 +197,14 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       const int sn = n < p.qkv.qd ? n : n - p.qkv.qd, r = sn % p.qkv.dh;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int tt = t + kConsWarps * u;
+        const int tt = (t + kConsWarps * u) * TP + sub;
         if (tt < cnt) hv[u] = __ldg(reinterpret_cast<const float4*>(p.qkv.rope + (size_t)((m0 + t0 + tt) % p.qkv.H) * p.qkv.dh + r));
       }
     };
     if (resid) load_gates(warp);
     if (qk) load_cs(warp);
-    const int row = (warp & 3) * 32 + lane;
+    // 64 rows: 16 in each warp's quarter of tensor memory
+    const int row = kBM == 128 ? (warp & 3) * 32 + lane : (warp & 3) * 16 + (lane & 15);
     pdl_wait();
     if (resid) load_h(warp);
     const bool ok = wait_bar(done, 0, p.err, 74);
@@ -212,7 +215,8 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       float v[16];
       tmem_ld16(tm + q, v);
 #pragma unroll
-      for (int e = 0; e < 16; ++e) T[(q + e) * kBM + row] = v[e];
+      for (int e = 0; e < 16; ++e)
+        if (kBM == 128 || lane < 16) T[(q + e) * kBM + row] = v[e];
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     named_sync(1, kCons);
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     __syncwarp();
     if (S > 1) cluster_arrive();   // this CTA's rows are here: once every CTA says so, none reads another's memory
     if (ok && all) {
-      for (int t = warp; t < cnt; t += kConsWarps * U) {
+      for (int t = warp; t * TP < cnt; t += kConsWarps * U) {
         if (resid && t != warp) {
           load_gates(t);
           load_h(t);
@@ -237,12 +241,12 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         if (qk && t != warp) load_cs(t);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int tt = t + kConsWarps * u;
+          const int tt = (t + kConsWarps * u) * TP + sub;
           if (tt >= cnt) break;
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
           for (int r = 0; r < S; ++r) {
             const float* src = r == rank ? T + (size_t)(t0 + tt) * kBM : recv + ((size_t)r * per + tt) * kBM;
-            const float4 q = *reinterpret_cast<const float4*>(src + 4 * lane);
+            const float4 q = *reinterpret_cast<const float4*>(src + 4 * fl);
             v.x += q.x;
             v.y += q.y;
             v.z += q.z;
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
                 }
               } else {
                 // v: into this token's staged row (16-byte pieces swizzled by token), for the writes below
-                *reinterpret_cast<float4*>(T + (size_t)(t0 + tt) * kBM + 4 * (lane ^ (tt & 31))) = v;
+                *reinterpret_cast<float4*>(T + (size_t)(t0 + tt) * kBM + 4 * (fl ^ (tt & (kLanes - 1)))) = v;
               }
             }
             break;
@@ -334,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         const int m = m0 + t0 + tt, b = m / o.H;
         __nv_bfloat16* dst = o.vtcache + (((size_t)b * o.L + o.layer) * o.kvd + (nt * kBM - o.qd - o.kvd)) * o.NKp + o.P + (m - b * o.H);
         for (int r = warp; r < kBM; r += kConsWarps)
-          dst[(size_t)r * o.NKp] = __float2bfloat16_rn(T[(size_t)(t0 + tt) * kBM + ((r & ~3) ^ (4 * (tt & 31))) + (r & 3)]);
+          dst[(size_t)r * o.NKp] = __float2bfloat16_rn(T[(size_t)(t0 + tt) * kBM + ((r & ~3) ^ (4 * (tt & (kLanes - 1)))) + (r & 3)]);
       }
     }
   }
@@ -350,50 +354,75 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
 
 }  // namespace
 
-// K splits (= CTAs of a cluster), at most eight: as many as keep the grid near one and a half CTAs an SM, so
-// that the next kernel's CTAs find room beside them and fetch their first weights early; with up to 32 tokens,
-// where a CTA's work is shorter than its start, one CTA an SM unless a split would sum more than 768 products
-// (the tensor cores' accumulation truncates, so the error grows with the run). Per evaluation, 1 / 1.5 / 1.75
-// CTAs an SM: DiT head 805 / 838 / 887 us, its four robots 1227 / 1212 / 1321, pi0-like one robot 717 / 706 /
-// 706, four robots 957 / 900 / 897.
-int gemm_cl_splits(int M, int N, int K, int sms) {
-  const int tiles = (N / kBM) * ((M + kBN - 1) / kBN), KC = K / kBK;
-  const int one = (sms + tiles / 2) / tiles, half = (3 * sms + tiles) / (2 * tiles);
-  int s = M <= 32 ? one : half;
+// Rows of a tile and K splits (= CTAs of a cluster, at most eight).
+// Rows: 64 for one tile of more than 32 tokens of a narrow projection, where eight splits of 128 rows would leave
+// SMs idle: half as much to exchange, and most or all of a CTA's weights fit its ring, requested before the wait
+// (18-layer expert, 50 tokens, N = 1024 and 2560: 694 -> 675 us per evaluation; two-layer time-concatenating
+// one 84 -> 81). With 16 tokens the activation boxes weigh as much as the weights (16-layer DiT expert 772 with
+// 128 rows, 817 with 64), with a second token tile every weight is read twice (18 layers, 100 tokens: 770, 799).
+// Splits: up to 32 tokens, where a CTA's work is shorter than its start, one CTA an SM unless a split would
+// sum more than 768 products (the tensor cores' accumulation truncates, so the error grows with the run); else as
+// many as keep the grid near one and a half CTAs an SM, so that the next kernel's CTAs find room beside them
+// and fetch their first weights early. Per evaluation, 1 / 1.5 / 1.75 CTAs an SM: DiT expert 805 / 838 / 887 us,
+// its four robots 1227 / 1212 / 1321, 18-layer expert at one robot 717 / 706 / 706, four robots 957 / 900 / 897.
+// With so few tiles that one CTA an SM is five splits or more, further ones pay only until a CTA's share
+// fits four slots (DiT expert, N = 1536, K = 1536: six robots 1530 us with eight splits, 1312 with six; 18-layer
+// expert, N = 1024, K = 2048 and 4096, four robots: 863 with eight, 878 with six).
+void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
+  const int mt = (M + kBN - 1) / kBN, KC = K / kBK;
+  a->cl_bm = M > 32 && mt == 1 && 6 * (N / kTileM) <= sms ? 64 : 128;
+  const int tiles = (N / a->cl_bm) * mt;
+  const int one = (sms + tiles / 2) / tiles, half = (3 * sms + tiles) / (2 * tiles), fit = (KC + 3) / 4;
+  int s = M <= 32 ? one : one >= 5 ? (fit < one ? one : fit < half ? fit : half) : half;
   while (s < half && K > 768 * s) ++s;
   s = s < 1 ? 1 : s > kClMaxSplits ? kClMaxSplits : s;
-  return s < KC ? s : KC;
+  a->splits = s < KC ? s : KC;
 }
 
 // The cluster form serves every projection of one 64-token tile, and with more tokens those with so
 // few tiles that the SMs need K splits; a projection with more tiles takes one CTA a tile (narrow form,
 // gemm_tc.cu), whose epilogue it shares with nobody.
 bool gemm_cl_serves(int M, int N, int sms) {
-  return M <= kBN || 2 * (N / kBM) * ((M + kBN - 1) / kBN) <= sms;
+  return M <= kBN || 2 * (N / kTileM) * ((M + kBN - 1) / kBN) <= sms;
 }
 
-static size_t gemm_cl_smem_bytes(int ring, int rows, int splits) {
-  return 1024 + cl_ring_bytes(ring, rows) + cl_recv_bytes(rows, splits) + (2 * ring + 2) * 8 + 16;
+static size_t gemm_cl_smem_bytes(int ring, int rows, int splits, int bm) {
+  return 1024 + cl_ring_bytes(ring, rows, bm) + cl_recv_bytes(rows, splits, bm) + (2 * ring + 2) * 8 + 16;
 }
+constexpr int kClMaxStages = 8;
 constexpr size_t kClSmem = 112 * 1024;   // two CTAs fit an SM
 
-void gemm_cl_prepare() {
-  for (const auto k : {gemm_cl_kernel<kAny>, gemm_cl_kernel<kPlain>, gemm_cl_kernel<EPI_QKV_TC>, gemm_cl_kernel<EPI_GEGLU>,
-                       gemm_cl_kernel<EPI_RESID_H>})
+namespace {
+using ClKernel = void (*)(CUtensorMap, TcGemmArgs, int);
+
+// One CTA's rows of the output features: BM.
+template <int BM>
+ClKernel cl_kernel(const TcGemmArgs& a) {
+  const bool own = a.cl_code == kClOwn, gated = a.epi == EPI_QKV_TC || a.epi == EPI_GEGLU;
+  return own && a.epi == EPI_QKV_TC ? gemm_cl_kernel<EPI_QKV_TC, BM>
+         : own && a.epi == EPI_GEGLU ? gemm_cl_kernel<EPI_GEGLU, BM>
+         : own && a.epi == EPI_RESID_H ? gemm_cl_kernel<EPI_RESID_H, BM>
+         : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain, BM> : gemm_cl_kernel<kAny, BM>;
+}
+template <int BM>
+void cl_prepare() {
+  for (const auto k : {gemm_cl_kernel<kAny, BM>, gemm_cl_kernel<kPlain, BM>, gemm_cl_kernel<EPI_QKV_TC, BM>,
+                       gemm_cl_kernel<EPI_GEGLU, BM>, gemm_cl_kernel<EPI_RESID_H, BM>})
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+}
+}  // namespace
+
+void gemm_cl_prepare() {
+  cl_prepare<128>();
+  cl_prepare<64>();
 }
 
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
   const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, rows = a.M < kBN ? a.M : kBN;
-  int ring = per < kTcMaxStages ? per : kTcMaxStages;
-  while (gemm_cl_smem_bytes(ring, rows, a.splits) > kClSmem) --ring;   // three slots at least
-  const bool own = a.cl_code == kClOwn, gated = a.epi == EPI_QKV_TC || a.epi == EPI_GEGLU;
-  const auto kernel = own && a.epi == EPI_QKV_TC ? gemm_cl_kernel<EPI_QKV_TC>
-                      : own && a.epi == EPI_GEGLU ? gemm_cl_kernel<EPI_GEGLU>
-                      : own && a.epi == EPI_RESID_H ? gemm_cl_kernel<EPI_RESID_H>
-                      : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain> : gemm_cl_kernel<kAny>;
-  launch_cluster(kernel, dim3(a.splits, a.N / kBM, (a.M + kBN - 1) / kBN), dim3(kThreads),
-                 gemm_cl_smem_bytes(ring, rows, a.splits), a.splits, s, *tmx, a, ring);
+  int ring = per < kClMaxStages ? per : kClMaxStages;
+  while (gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm) > kClSmem) --ring;   // three slots at least
+  launch_cluster(a.cl_bm == 64 ? cl_kernel<64>(a) : cl_kernel<128>(a), dim3(a.splits, a.N / a.cl_bm, (a.M + kBN - 1) / kBN),
+                 dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring);
 }
 
 }  // namespace uad

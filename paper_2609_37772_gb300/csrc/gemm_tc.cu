@@ -688,7 +688,7 @@ void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
     a->splits = it->second.second;
   } else if (epi == EPI_RESID_H || alone || gemm_cl_serves(M, N, sms)) {
     a->cl = 1;
-    a->splits = gemm_cl_splits(M, N, K, sms);
+    gemm_cl_plan(M, N, K, sms, a);
   }
 }
 

@@ -216,6 +216,7 @@ struct TcGemmArgs {
   int wide = 0;                    // 1: the persistent wide form (one CTA per SM walking units of
                                    // tn tokens x 128 weight rows x a K range), 0: narrow split-K tiles
   int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)
+  int cl_bm = 128;                 //    weight rows of a tile: 128 or 64
   int cl_code = 0;                 //    which projections share its code: kClAny, kClPlain or kClOwn
   int tn = 0;                      // persistent form: tokens per tile (256, 192 or 128)
 };
@@ -229,7 +230,7 @@ void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a);
 // gemm_cl.cu: the few-token form (K splits over a cluster), at most kClMaxSplits splits
 constexpr int kClMaxSplits = 8;
 constexpr int kClAny = 0, kClPlain = 1, kClOwn = 2;   // TcGemmArgs::cl_code
-int gemm_cl_splits(int M, int N, int K, int sms);
+void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a);   // K splits and rows of a tile
 bool gemm_cl_serves(int M, int N, int sms);
 void gemm_cl_prepare();
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
