@@ -24,7 +24,9 @@ namespace {
 
 constexpr int kTileM = 128, kBN = 64, kBK = 64;
 constexpr int kTileBytes = kTileM * kBK * 2;     // a k-block of the tiled weights: 16 KB, its rows 0-63 first
-constexpr int kSlotB = kBN * kBK * 2;            // activations: 8 KB
+// A k-block's activations come in one box, of 64 token rows or, for up to 16 tokens, 16: 8 KB or 2 KB a slot, so
+// that a fifth slot of weights fits (16-layer DiT expert, 16 tokens: 772 -> 762 us per evaluation; two boxes of 16
+// for up to 32 tokens lost 1%).
 constexpr int kConsWarps = 8, kCons = 32 * kConsWarps;
 constexpr int kThreads = kCons + 64;             // + producer warp, + MMA warp
 constexpr unsigned long long kWaitNs = 2000000000ull;
@@ -56,7 +58,7 @@ __device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) { ret
 // the ring, so that they may arrive while this CTA's MMAs still run. `rows`: tokens of the largest
 // tile, bm: weight rows of a tile.
 __host__ __device__ __forceinline__ size_t cl_ring_bytes(int ring, int rows, int bm) {
-  const size_t pipe = (size_t)ring * (bm * kBK * 2 + kSlotB), tile = (size_t)((rows + 15) / 16 * 16) * bm * 4;
+  const size_t pipe = (size_t)ring * (bm + act_box_rows(rows)) * kBK * 2, tile = (size_t)((rows + 15) / 16 * 16) * bm * 4;
   return pipe > tile ? pipe : tile;
 }
 __host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits, int bm) {
@@ -67,10 +69,10 @@ __host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits, i
 // and EPI_GEGLU. A kernel whose code is not in the SM's instruction cache runs at a dozen cycles an instruction,
 // so it matters which projections share code (TcGemmArgs::cl_code).
 constexpr int kAny = -2, kPlain = -1;
-template <int E, int kBM>
+template <int E, int kBM, int kBox>
 __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
   extern __shared__ uint8_t smem_raw[];
-  constexpr int kSlotA = kBM * kBK * 2, kSlot = kSlotA + kSlotB;
+  constexpr int kSlotA = kBM * kBK * 2, kSlot = kSlotA + kBox * kBK * 2;
   constexpr int kLanes = kBM / 4, TP = 32 / kLanes;   // lanes that share a token row, rows a warp takes at once
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int S = p.splits, rank = blockIdx.x, nt = blockIdx.y, mt = blockIdx.z;
@@ -389,39 +391,40 @@ bool gemm_cl_serves(int M, int N, int sms) {
 static size_t gemm_cl_smem_bytes(int ring, int rows, int splits, int bm) {
   return 1024 + cl_ring_bytes(ring, rows, bm) + cl_recv_bytes(rows, splits, bm) + (2 * ring + 2) * 8 + 16;
 }
-constexpr int kClMaxStages = 8;
+constexpr int kClMaxStages = 12;
 constexpr size_t kClSmem = 112 * 1024;   // two CTAs fit an SM
 
 namespace {
 using ClKernel = void (*)(CUtensorMap, TcGemmArgs, int);
 
-// One CTA's rows of the output features: BM.
-template <int BM>
+// One CTA's rows of the output features: BM; token rows of an activation box: BOX.
+template <int BM, int BOX>
 ClKernel cl_kernel(const TcGemmArgs& a) {
   const bool own = a.cl_code == kClOwn, gated = a.epi == EPI_QKV_TC || a.epi == EPI_GEGLU;
-  return own && a.epi == EPI_QKV_TC ? gemm_cl_kernel<EPI_QKV_TC, BM>
-         : own && a.epi == EPI_GEGLU ? gemm_cl_kernel<EPI_GEGLU, BM>
-         : own && a.epi == EPI_RESID_H ? gemm_cl_kernel<EPI_RESID_H, BM>
-         : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain, BM> : gemm_cl_kernel<kAny, BM>;
+  return own && a.epi == EPI_QKV_TC ? gemm_cl_kernel<EPI_QKV_TC, BM, BOX>
+         : own && a.epi == EPI_GEGLU ? gemm_cl_kernel<EPI_GEGLU, BM, BOX>
+         : own && a.epi == EPI_RESID_H ? gemm_cl_kernel<EPI_RESID_H, BM, BOX>
+         : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain, BM, BOX> : gemm_cl_kernel<kAny, BM, BOX>;
 }
-template <int BM>
+template <int BM, int BOX>
 void cl_prepare() {
-  for (const auto k : {gemm_cl_kernel<kAny, BM>, gemm_cl_kernel<kPlain, BM>, gemm_cl_kernel<EPI_QKV_TC, BM>,
-                       gemm_cl_kernel<EPI_GEGLU, BM>, gemm_cl_kernel<EPI_RESID_H, BM>})
+  for (const auto k : {gemm_cl_kernel<kAny, BM, BOX>, gemm_cl_kernel<kPlain, BM, BOX>, gemm_cl_kernel<EPI_QKV_TC, BM, BOX>,
+                       gemm_cl_kernel<EPI_GEGLU, BM, BOX>, gemm_cl_kernel<EPI_RESID_H, BM, BOX>})
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
 }
 }  // namespace
 
 void gemm_cl_prepare() {
-  cl_prepare<128>();
-  cl_prepare<64>();
+  cl_prepare<128, 64>();
+  cl_prepare<128, 16>();
+  cl_prepare<64, 64>();
 }
 
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
   const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, rows = a.M < kBN ? a.M : kBN;
   int ring = per < kClMaxStages ? per : kClMaxStages;
   while (gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm) > kClSmem) --ring;   // three slots at least
-  launch_cluster(a.cl_bm == 64 ? cl_kernel<64>(a) : cl_kernel<128>(a), dim3(a.splits, a.N / a.cl_bm, (a.M + kBN - 1) / kBN),
+  launch_cluster(a.cl_bm == 64 ? cl_kernel<64, 64>(a) : act_box_rows(a.M) == 16 ? cl_kernel<128, 16>(a) : cl_kernel<128, 64>(a), dim3(a.splits, a.N / a.cl_bm, (a.M + kBN - 1) / kBN),
                  dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring);
 }
 

@@ -42,7 +42,7 @@ int launch_linear(const void* x, const void* w_tiled, const float* bias, float* 
   if (cudaGetDevice(&dev) != cudaSuccess) return UAD_ECUDA;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   CUtensorMap tm;
-  if (encode_act_tmap(&tm, x, K, M)) return UAD_ECUDA;
+  if (encode_act_tmap(&tm, x, K, M, act_box_rows(M))) return UAD_ECUDA;
   TcGemmArgs a;
   a.w_tiled = w_tiled; a.M = M; a.N = N; a.K = K;
   gemm_tc_plan(M, N, K, sms, EPI_STORE, &a);   // the tile selection of the velocity network's projections

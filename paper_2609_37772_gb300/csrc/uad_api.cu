@@ -64,7 +64,7 @@ struct uad_ctx {
   bool force_simt = false;     // UAD_GEMM=simt: CUDA-core GEMMs only (debugging)
 
   // tensor-core GEMM: TMA descriptors of the activation buffers
-  std::map<const void*, CUtensorMap> tmaps;
+  std::map<const void*, CUtensorMap> tmaps, tmaps16;   // by buffer: boxes of 64 rows, of 16
   // tensor-core attention (bf16 joint-attention experts): query matrix, K and Vt caches
   bool attn_tc = false;
   AttnTcArgs at0;                 // shapes and buffers; batch / layer set per launch
@@ -460,6 +460,10 @@ int cl_code(const uad_ctx* c) {
   return c->a.kind == UAD_KIND_DIT ? kClPlain : c->a.kind == UAD_KIND_ADARMS ? kClOwn : kClAny;
 }
 
+const CUtensorMap* act_map(const uad_ctx* c, const void* buf, int M) {
+  return &(act_box_rows(M) == 16 ? c->tmaps16 : c->tmaps).at(buf);
+}
+
 // out = epi(A Wt^T): tensor cores when the weight is tiled, CUDA cores otherwise.
 void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   g.W = w.w;
@@ -473,7 +477,7 @@ void gemm(uad_ctx* c, const Lin& w, GemmArgs g, cudaStream_t s) {
   gemm_tc_plan(g.M, g.N, g.K, c->sms, g.epi, &t);
   t.epi = g.epi; t.out = g.out; t.ldo = g.ldo; t.out_dtype = g.out_dtype; t.bias = g.bias;
   t.qkv = g.qkv; t.n_store = g.n_store; t.err = c->dev_err; t.cl_code = cl_code(c);
-  launch_gemm_tc(&c->tmaps.at(g.A), t, s);
+  launch_gemm_tc(act_map(c, g.A, t.M), t, s);
 }
 
 void gemm(uad_ctx* c, const void* w, GemmArgs g, cudaStream_t s) {
@@ -503,7 +507,7 @@ void resid_gemm(uad_ctx* c, const Lin& w, GemmArgs g, int gate_off, const float*
     if (gate_off >= 0) { t.gate_tab = c->tab + gate_off; t.gate_stride = c->rowlen; }
     g.epi = EPI_RESID_GATE;
     Mark mk(c, s, name, gemm_bytes(g, c->es), flops);
-    launch_gemm_tc(&c->tmaps.at(g.A), t, s);
+    launch_gemm_tc(act_map(c, g.A, t.M), t, s);
     return;
   }
   if (w.tiled) {
@@ -536,13 +540,15 @@ void norm_after(uad_ctx* c, NormArgs n, PendingResid* pend, cudaStream_t s) {
   launch_norm(n, s);
 }
 
-// 2-D TMA descriptor of a bf16 activation buffer [rows][K]: 64 x 64 boxes, 128-byte swizzle,
-// zero fill outside the buffer.
+// 2-D TMA descriptors of a bf16 activation buffer [rows][K]: boxes of 64 and of 16 rows x 64, 128-byte
+// swizzle, zero fill outside the buffer.
 int make_tmap(uad_ctx* c, const void* base, int K, int rows) {
-  CUtensorMap m;
-  const int r = encode_act_tmap(&m, base, K, rows);
+  CUtensorMap m, few;
+  int r = encode_act_tmap(&m, base, K, rows, 64);
+  if (!r) r = encode_act_tmap(&few, base, K, rows, 16);
   if (r) return fail(c, UAD_ECUDA, "TMA descriptor encoding failed (%d)", r);
   c->tmaps[base] = m;
+  c->tmaps16[base] = few;
   return UAD_OK;
 }
 
@@ -1256,7 +1262,7 @@ int uad_set_prefix_kv(uad_ctx* c, int32_t robot, const void* k, const void* v, i
       t.epi = EPI_PREFIX_KV; t.out_dtype = BF16; t.err = c->dev_err;
       const size_t base = (size_t)robot * a.n_layers * per_layer;
       t.pkv = {static_cast<__nv_bfloat16*>(c->kpre) + base, static_cast<__nv_bfloat16*>(c->vpre) + base, c->qd};
-      launch_gemm_tc(&c->tmaps.at(c->pre_tok), t, s);
+      launch_gemm_tc(act_map(c, c->pre_tok, t.M), t, s);
     }
     for (int l = 0; l < a.n_layers && !c->pre_tok; ++l) {
       for (int which = 0; which < 2; ++which) {

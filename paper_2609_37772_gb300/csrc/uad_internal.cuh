@@ -220,9 +220,11 @@ struct TcGemmArgs {
   int cl_code = 0;                 //    which projections share its code: kClAny, kClPlain or kClOwn
   int tn = 0;                      // persistent form: tokens per tile (256, 192 or 128)
 };
-// 2-D TMA descriptor of a bf16 activation matrix [rows][K] (64 x 64 boxes, 128-byte swizzle,
+// 2-D TMA descriptor of a bf16 activation matrix [rows][K] (boxes of box_rows x 64, 128-byte swizzle,
 // zero fill past the last row). 0 on success.
-int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows);
+int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows, int box_rows);
+// rows of the boxes that a projection of M tokens is read in
+__host__ __device__ constexpr int act_box_rows(int M) { return M <= 16 ? 16 : 64; }
 void gemm_tc_prepare();
 int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form serves this projection
 // The tile plan of one projection (wide form, tokens per tile, K splits) into a.

@@ -66,9 +66,11 @@ def test_linear_wide_tiles_match_reference(M, N, K):
 #   (63, 128, 4096): seven CTAs with eight rows, one with seven; (65, 256, 1024): a second tile of one row;
 #   (637, 1024, 2048), (1200, 512, 2112): two and three splits of ragged last tiles
 # and tiles of 64 weight rows (33 to 64 tokens): (33, 128, 64): one k-block, no splits; (47, 384, 1600): an odd
-# number of tokens, more k-blocks than slots; (64, 3200, 320): the widest N that they serve
+# number of tokens, more k-blocks than slots; (64, 3200, 320): the widest N that they serve;
+# boxes of 16 token rows, five slots walked more than once, and the first size past them: (16, 6400, 1088), (17, 128, 128)
 @pytest.mark.parametrize("M,N,K", [(1, 128, 512), (9, 256, 640), (63, 128, 4096), (65, 256, 1024), (637, 1024, 2048),
-                                   (1200, 512, 2112), (33, 128, 64), (47, 384, 1600), (64, 3200, 320)])
+                                   (1200, 512, 2112), (33, 128, 64), (47, 384, 1600), (64, 3200, 320),
+                                   (16, 6400, 1088), (17, 128, 128)])
 def test_linear_cluster_shares_match_reference(M, N, K):
     rng = np.random.default_rng(M + N + K)
     x = rng.normal(size=(M, K)).astype(np.float32)
