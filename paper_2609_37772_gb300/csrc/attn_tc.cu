@@ -110,47 +110,57 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   }
   __syncwarp();
 
-  // ---- softmax over this key chunk: one query row per thread ----
-  pdl_wait();
-  const bool ok_s = mbar_wait(bar_s, 0, p.err, 22);
-  tc_fence_after();
+  // ---- softmax over this key chunk: one query row per thread. Warps 2 and 3, which have nothing to do until
+  //      the scores are there, first go through it once (on whatever tensor memory holds, storing nothing): that
+  //      brings its code, run once a CTA, into the SM's instruction cache. 18 layers, 180 tokens: 862 -> 854 us per
+  //      evaluation ----
   const int row = warp * 32 + lane;
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
   const float c2 = p.scale_log2;             // log2(e) / sqrt(dh)
   const int key0 = kc * kKT;
   const int nv = p.n_keys - key0;            // valid keys of the chunk (all of them but in the last)
-  float sv[kKT];                             // the chunk's scores of this row, one wait for all
-  __syncwarp();
-  tmem_ld128(tS + lane_base, sv);
-  if (nv < kKT) {   // keys past the end (last chunk): excluded from the maximum, P = 2^-inf = 0
-#pragma unroll
-    for (int i = 0; i < kKT; ++i)
-      if (i >= nv) sv[i] = -INFINITY;
-  }
-  float mx = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < kKT; ++i) mx = fmaxf(mx, sv[i]);
-  const float ms = mx * c2;
-  float l = 0.f;
   const int r8 = row & 7;
-#pragma unroll
-  for (int cc = 0; cc < kKT / 32; ++cc) {
-    uint32_t pk[16];
-#pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-      const int k = cc * 32 + i;
-      const float e0 = ex2_fast(fmaf(sv[k], c2, -ms)), e1 = ex2_fast(fmaf(sv[k + 1], c2, -ms));
-      const __nv_bfloat162 h = __floats2bfloat162_rn(e0, e1);
-      const float2 hf = __bfloat1622float2(h);
-      l += hf.x + hf.y;   // normalise by what the MMA actually sums
-      pk[i / 2] = *reinterpret_cast<const uint32_t*>(&h);
+  float sv[kKT];                             // the chunk's scores of this row, one wait for all
+  float mx, l;
+  bool ok_s = false;
+#pragma unroll 1
+  for (int pass = warp >= 2 ? 0 : 1; pass < 2; ++pass) {
+    if (pass) {
+      pdl_wait();
+      ok_s = mbar_wait(bar_s, 0, p.err, 22);
+      tc_fence_after();
     }
-    // 32 keys = four 16-byte granules of row `row` in P block (cc / 2), granules (cc % 2) * 4 + q
-    uint8_t* prow = sP + (cc / 2) * (kQT * 128) + row * 128;
+    __syncwarp();
+    tmem_ld128(tS + lane_base, sv);
+    if (nv < kKT) {   // keys past the end (last chunk): excluded from the maximum, P = 2^-inf = 0
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int gidx = (cc % 2) * 4 + q;
-      *reinterpret_cast<uint4*>(prow + ((gidx ^ r8) * 16)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      for (int i = 0; i < kKT; ++i)
+        if (i >= nv) sv[i] = -INFINITY;
+    }
+    mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < kKT; ++i) mx = fmaxf(mx, sv[i]);
+    const float ms = mx * c2;
+    l = 0.f;
+#pragma unroll
+    for (int cc = 0; cc < kKT / 32; ++cc) {
+      uint32_t pk[16];
+#pragma unroll
+      for (int i = 0; i < 32; i += 2) {
+        const int k = cc * 32 + i;
+        const float e0 = ex2_fast(fmaf(sv[k], c2, -ms)), e1 = ex2_fast(fmaf(sv[k + 1], c2, -ms));
+        const __nv_bfloat162 h = __floats2bfloat162_rn(e0, e1);
+        const float2 hf = __bfloat1622float2(h);
+        l += hf.x + hf.y;   // normalise by what the MMA actually sums
+        pk[i / 2] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      // 32 keys = four 16-byte granules of row `row` in P block (cc / 2), granules (cc % 2) * 4 + q
+      uint8_t* prow = sP + (cc / 2) * (kQT * 128) + row * 128;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int gidx = (cc % 2) * 4 + q;
+        if (pass) *reinterpret_cast<uint4*>(prow + ((gidx ^ r8) * 16)) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      }
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -179,7 +189,7 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
   constexpr uint32_t pitch = DV * 4 + 16;
   uint8_t* srow = smem + (size_t)row * pitch;
   __syncwarp();
-#pragma unroll
+#pragma unroll 1
   for (int cc = 0; cc < DV / 32; ++cc) {
     tmem_ld32(tO + lane_base + cc * 32, sv);
 #pragma unroll
