@@ -729,6 +729,27 @@ def test_dit_attention_tiles_and_clusters(chunk, prefix, robots):
         c.close()
 
 
+@pytest.mark.parametrize("name,robots", [("dit_small", 2), ("tiny", 1), ("pi0_small", 3)])
+def test_step_graphs_of_changing_step_counts(name, robots):
+    """Chunks of different step counts one after the other on one context, whose graphs hold a divisor
+    of the steps each (one step at 7, 11 and 13): each chunk bit for bit what a fresh context gives."""
+    a = ARCHS[name]
+    noise = make_noise(a, batch=robots, seed=55)
+    blob = make_weights(a, seed=55)
+    c = Case(a, B=robots, seed=55, blob=blob)
+    try:
+        for n in (7, 2, 13, 12, 1, 7, 11):
+            bud = np.stack([group_budgets(a.chunk_len, [(0, 2, (n + 1) // 2), (3, a.chunk_len - 1, n)])] * robots)
+            res = c.gpu(noise, bud)
+            fresh = Case(a, B=robots, seed=55, blob=blob)
+            ref = fresh.gpu(noise, bud)
+            fresh.close()
+            assert res["evals"] == ref["evals"] == n
+            assert np.array_equal(res["final"], ref["final"]) and np.array_equal(res["ghost"], ref["ghost"])
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("prefix", [1, 63, 64, 72, 129])
 def test_prefix_transposition_lengths(prefix):
     """Prefix keys and values into the attention caches at the edges of the 64-position tiles and of
