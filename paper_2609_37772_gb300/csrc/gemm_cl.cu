@@ -369,13 +369,16 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
 // its four robots 1227 / 1212 / 1321, 18-layer expert at one robot 717 / 706 / 706, four robots 957 / 900 / 897.
 // With so few tiles that one CTA an SM is five splits or more, further ones pay only until a CTA's share
 // fits four slots (DiT expert, N = 1536, K = 1536: six robots 1530 us with eight splits, 1312 with six; 18-layer
-// expert, N = 1024, K = 2048 and 4096, four robots: 863 with eight, 878 with six).
+// expert, N = 1024, K = 2048 and 4096, four robots: 863 with eight, 878 with six); with four, none do (DiT
+// expert, N = 4608, K = 1536, 64 tokens: 1089 us with six splits, 1073 with four; 144 tokens: 1770 and 1498).
 void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
   const int mt = (M + kBN - 1) / kBN, KC = K / kBK;
   a->cl_bm = M > 32 && mt == 1 && 6 * (N / kTileM) <= sms ? 64 : 128;
   const int tiles = (N / a->cl_bm) * mt;
   const int one = (sms + tiles / 2) / tiles, half = (3 * sms + tiles) / (2 * tiles), fit = (KC + 3) / 4;
-  int s = M <= 32 ? one : one >= 5 ? (fit < one ? one : fit < half ? fit : half) : half;
+  int s = half;
+  if (M <= 32 || (one == 4 && a->cl_bm == 128)) s = one;
+  else if (one >= 5) s = fit < one ? one : fit < half ? fit : half;
   while (s < half && K > 768 * s) ++s;
   s = s < 1 ? 1 : s > kClMaxSplits ? kClMaxSplits : s;
   a->splits = s < KC ? s : KC;

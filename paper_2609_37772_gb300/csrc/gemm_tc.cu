@@ -624,6 +624,15 @@ int gemm_tc_use_wide(int M, int N, int sms) {
   return M >= 512 || t256 * 5 >= sms * 3 || t128 * 2 >= sms ? 1 : 0;
 }
 
+// A residual projection may also split K into planes that the next norm sums, so the persistent form fills
+// the SMs from a third 64-token tile on, where the cluster form's exchange costs more than writing the planes.
+// Per evaluation, N = 1024, 18 layers: 180 tokens 852 -> 842 us, 250 tokens 1053 -> 968, 400 tokens 1288 -> 1183;
+// N = 1536, 16 layers: 128 tokens 1368 -> 1378, 192 tokens 1820 -> 1795, 256 tokens 1850 -> 1761, 320 tokens
+// 1886 -> 2005, 480 tokens 2556 -> 2450. Narrower ones stay: N = 512, 250 tokens 102 -> 109.
+int gemm_tc_resid_wide(int M, int N, int sms) {
+  return gemm_tc_use_wide(M, N, sms) || (M > 128 && N >= 1024 && N <= 2048);
+}
+
 // The persistent form's plan: tokens per tile (256, 192 or 128) and, for partial-plane
 // epilogues, K splits. Units go to the CTAs round robin; the plan minimises the busiest CTA's
 // work, counted in k-blocks of a 256-token tile: a k-block of nb 64-token boxes costs half by
@@ -666,7 +675,7 @@ void gemm_tc_pers_plan(int M, int N, int K, int sms, int epi, int* tn, int* spli
 }
 
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
-  a->wide = gemm_tc_use_wide(M, N, sms);
+  a->wide = epi == EPI_PARTIAL ? gemm_tc_resid_wide(M, N, sms) : gemm_tc_use_wide(M, N, sms);
   a->tn = 0;
   a->splits = 1;
   a->cl = 0;

@@ -435,7 +435,7 @@ struct Mark {
 // Partial planes a residual projection [M][W] x [W][K]^T writes on the tensor cores (none with few
 // tokens, where it updates the residual stream itself).
 size_t residual_planes(const uad_ctx* c, int M, int K) {
-  if (!gemm_tc_use_wide(M, c->a.width, c->sms)) return 0;
+  if (!gemm_tc_resid_wide(M, c->a.width, c->sms)) return 0;
   TcGemmArgs t;
   gemm_tc_plan(M, c->a.width, K, c->sms, EPI_PARTIAL, &t);
   return (size_t)t.splits;
@@ -499,7 +499,7 @@ struct PendingResid {
 void resid_gemm(uad_ctx* c, const Lin& w, GemmArgs g, int gate_off, const float* bias, PendingResid* pend,
                 const char* name, cudaStream_t s) {
   const double flops = 2.0 * g.M * g.N * g.K;
-  if (w.tiled && !gemm_tc_use_wide(g.M, g.N, c->sms)) {
+  if (w.tiled && !gemm_tc_resid_wide(g.M, g.N, c->sms)) {
     TcGemmArgs t;
     t.w_tiled = w.w; t.M = g.M; t.N = g.N; t.K = g.K; t.epi = EPI_RESID_H; t.ldo = g.N;
     gemm_tc_plan(g.M, g.N, g.K, c->sms, t.epi, &t);

@@ -227,6 +227,7 @@ int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows, int box_r
 __host__ __device__ constexpr int act_box_rows(int M) { return M <= 16 ? 16 : 64; }
 void gemm_tc_prepare();
 int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form serves this projection
+int gemm_tc_resid_wide(int M, int N, int sms);  // the same for a residual projection, which may split K into planes
 // The tile plan of one projection (wide form, tokens per tile, K splits) into a.
 void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a);
 // gemm_cl.cu: the few-token form (K splits over a cluster), at most kClMaxSplits splits

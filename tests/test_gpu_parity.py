@@ -750,6 +750,20 @@ def test_step_graphs_of_changing_step_counts(name, robots):
         c.close()
 
 
+@pytest.mark.parametrize("name,chunk,robots", [("pi0", 32, 4), ("pi0", 43, 3), ("pi0", 50, 5), ("dit", 16, 9), ("dit", 13, 20)])
+def test_residual_projections_around_the_wide_form(name, chunk, robots):
+    """Residual projections of a layer from 128 tokens (the last size of the cluster form) and 129 (the
+    first of the persistent form with planes of K splits) on, with ragged last token tiles."""
+    a = ARCHS[name].replace(name=f"{name}_c{chunk}", n_layers=1, chunk_len=chunk, prefix_len=70)
+    c = Case(a, B=robots, seed=56)
+    try:
+        noise = make_noise(a, batch=robots, seed=56)
+        bud = np.stack([group_budgets(chunk, [(0, 3, 1), (4, chunk - 1, 2)])] * robots)
+        check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL["bf16"])
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("prefix", [1, 63, 64, 72, 129])
 def test_prefix_transposition_lengths(prefix):
     """Prefix keys and values into the attention caches at the edges of the 64-position tiles and of
