@@ -1411,6 +1411,7 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
     if (it == c->graphs.end()) {
       cudaGraph_t g = nullptr;
       CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+      if (per == steps) enqueue_begin(c, B, steps, s);   // the chunk's only graph: begin joins it
       enqueue_steps(c, B, steps, per, use_step, s);
       cudaError_t e = cudaStreamEndCapture(s, &g);
       if (e != cudaSuccess) return fail(c, UAD_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
@@ -1420,7 +1421,7 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
       if (e != cudaSuccess) return fail(c, UAD_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
       it = c->graphs.emplace(key, ex).first;
     }
-    enqueue_begin(c, B, steps, s);
+    if (per != steps) enqueue_begin(c, B, steps, s);
     for (int k = 0; k < steps; k += per) CK(cudaGraphLaunch(it->second, s));
   } else if (profile) {
     // capture with an event-record node around every kernel, so that the event times are
