@@ -486,10 +486,10 @@ void gemm(uad_ctx* c, const void* w, GemmArgs g, cudaStream_t s) {
   gemm(c, l, g, s);
 }
 
-// Residual update h += gate(tau) * (A W^T + bias) (gate 1 without a table). Tensor-core
-// weights: the K splits write fp32 partial planes and the update is left pending in `pend`
-// for the next norm, which sums the planes in a fixed order, applies it and normalises in one
-// pass over the row. CUDA-core weights: applied in the GEMM epilogue.
+// Residual update h += gate(tau) * (A W^T + bias) (gate 1 without a table). Tensor-core weights with few tokens
+// and CUDA-core weights: applied in the GEMM epilogue. Tensor-core weights with more: the K splits of the
+// persistent form write fp32 partial planes and the update is left pending in `pend` for the next norm, which
+// sums the planes in a fixed order, applies it and normalises in one pass over the row.
 struct PendingResid {
   const float* part = nullptr; int n_part = 0;
   const float* gate_tab = nullptr; int gate_off = 0;
