@@ -33,6 +33,9 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
+__device__ __forceinline__ float lo_word(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi_word(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+
 // Four consecutive values of a row into shared memory as fp32; `vec`: rows are 16-byte (fp32) or
 // 8-byte (bf16) aligned and a multiple of 4 long. fp32 vectors are asynchronous copies.
 template <int DT>
@@ -69,8 +72,9 @@ __device__ __forceinline__ void load4(float* dst, const void* base, long long of
 // fp32 expert, down projection (K = 1024) of 16 rows 75 -> 11 us, of 512 rows 93 -> 17 us (20 us with eight
 // warps: two a scheduler do not hide the shared-memory loads).
 // ------------------------------------------------------------------------------------------
-template <int THREADS_, int BM_, int BN_, int WM_, int WN_, int KC_, int ST_>
+template <int THREADS_, int BM_, int BN_, int WM_, int WN_, int KC_, int ST_, bool SERIAL_ = false>
 struct FfTile {
+  static constexpr bool SERIAL = SERIAL_;   // every output one fp32 sum over ascending k
   static constexpr int THREADS = THREADS_, BM = BM_, BN = BN_, WM = WM_, WN = WN_, KC = KC_, ST = ST_;
   static constexpr int KS = THREADS / 32 / (WM * WN), RM = BM / WM / 8, RN = BN / WN / 4, PITCH = KC + 4;
   static constexpr int STAGE = (BM + BN) * PITCH;          // floats
@@ -85,6 +89,12 @@ struct FfTile {
 using FfSmall = FfTile<256, 16, 16, 1, 1, 256, 4>;
 using FfMid = FfTile<512, 32, 32, 1, 1, 256, 2>;
 using FfWide = FfTile<512, 64, 64, 2, 2, 64, 3>;
+// The time table's: one sum per output over ascending k, so that a row has the same bits whichever tile made it
+// and however many rows are filled at once. Every modulation of every step goes through these rows: a
+// last bit of theirs moves bf16 roundings of every layer (18-layer expert, 16 and 64 robots: with sums
+// in groups the actions differed by 6.9e-4, at the same distance from 64 bits, 5.2e-4).
+using FfTabSmall = FfTile<64, 16, 16, 1, 2, 256, 4, true>;
+using FfTabWide = FfTile<256, 64, 64, 4, 2, 64, 3, true>;
 
 template <int AD, int WD, class T>
 __global__ void __launch_bounds__(T::THREADS) gemm_ffma_kernel(GemmArgs p) {
@@ -150,7 +160,8 @@ __global__ void __launch_bounds__(T::THREADS) gemm_ffma_kernel(GemmArgs p) {
   constexpr int WT = T::WM * T::WN, KW = KC / T::KS;   // warps over the tile; k of a chunk per group
   const int ks = warp / WT, wm = (warp % WT) / T::WN, wn = warp % T::WN;
   const int lr = lane >> 2, lc = lane & 3;
-  unsigned long long acc[RM][RN];
+  static_assert(!T::SERIAL || T::KS == 1, "one group of warps walks the whole K");
+  unsigned long long acc[RM][RN];   // the sums of even and odd k; SERIAL: one sum, in the low word
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
@@ -171,8 +182,17 @@ __global__ void __launch_bounds__(T::THREADS) gemm_ffma_kernel(GemmArgs p) {
       for (int i = 0; i < RM; ++i)
 #pragma unroll
         for (int j = 0; j < RN; ++j) {
-          fma2(acc[i][j], av[i].x, wv[j].x);
-          fma2(acc[i][j], av[i].y, wv[j].y);
+          if constexpr (T::SERIAL) {
+            float r = lo_word(acc[i][j]);
+            r = fmaf(lo_word(av[i].x), lo_word(wv[j].x), r);
+            r = fmaf(hi_word(av[i].x), hi_word(wv[j].x), r);
+            r = fmaf(lo_word(av[i].y), lo_word(wv[j].y), r);
+            r = fmaf(hi_word(av[i].y), hi_word(wv[j].y), r);
+            acc[i][j] = __float_as_uint(r);
+          } else {
+            fma2(acc[i][j], av[i].x, wv[j].x);
+            fma2(acc[i][j], av[i].y, wv[j].y);
+          }
         }
     }
     __syncthreads();
@@ -189,8 +209,8 @@ __global__ void __launch_bounds__(T::THREADS) gemm_ffma_kernel(GemmArgs p) {
   for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < RN; ++j) {
-      const float lo = __uint_as_float((unsigned)acc[i][j]), hi = __uint_as_float((unsigned)(acc[i][j] >> 32));
-      red[((size_t)ks * T::BM + wm * (T::BM / T::WM) + lr + 8 * i) * T::RPITCH + wn * (T::BN / T::WN) + lc + 4 * j] = lo + hi;
+      const float lo = lo_word(acc[i][j]), hi = hi_word(acc[i][j]);
+      red[((size_t)ks * T::BM + wm * (T::BM / T::WM) + lr + 8 * i) * T::RPITCH + wn * (T::BN / T::WN) + lc + 4 * j] = T::SERIAL ? lo : lo + hi;
     }
   __syncthreads();
   const auto total = [&](int m, int n) {
@@ -451,6 +471,12 @@ void prepare_tiles() {
   cudaFuncSetAttribute(gemm_ffma_kernel<AD, WD, FfMid>, at, (int)FfMid::smem(FfMid::ST));
   cudaFuncSetAttribute(gemm_ffma_kernel<AD, WD, FfWide>, at, (int)FfWide::smem(FfWide::ST));
 }
+template <int WD>
+void prepare_table_tiles() {
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaFuncSetAttribute(gemm_ffma_kernel<F32, WD, FfTabSmall>, at, (int)FfTabSmall::smem(FfTabSmall::ST));
+  cudaFuncSetAttribute(gemm_ffma_kernel<F32, WD, FfTabWide>, at, (int)FfTabWide::smem(FfTabWide::ST));
+}
 
 int device_sms() {
   int dev = 0, sms = 0;
@@ -469,7 +495,21 @@ void launch_gemm_ffma(const GemmArgs& a, cudaStream_t s) {
   else launch_types<BF16, F32>(a, sms, s);
 }
 
+// The time table's projections (fp32 activations): the wide tile once its grid covers the SMs.
+void launch_gemm_table(const GemmArgs& a, cudaStream_t s) {
+  const bool wide = (long long)((a.M + 63) / 64) * ((a.N + 63) / 64) >= device_sms();
+  if (a.w_dtype == F32) {
+    if (wide) launch_tile<F32, F32, FfTabWide>(a, s);
+    else launch_tile<F32, F32, FfTabSmall>(a, s);
+  } else {
+    if (wide) launch_tile<F32, BF16, FfTabWide>(a, s);
+    else launch_tile<F32, BF16, FfTabSmall>(a, s);
+  }
+}
+
 void ffma_prepare(int dh) {
+  prepare_table_tiles<F32>();
+  prepare_table_tiles<BF16>();
   prepare_tiles<F32, F32>();
   prepare_tiles<F32, BF16>();
   prepare_tiles<BF16, BF16>();

@@ -341,19 +341,19 @@ int fill_times(uad_ctx* c, const std::vector<std::pair<int, int>>& fr, cudaStrea
   GemmArgs g;
   g.A = c->temb; g.lda = W; g.a_dtype = F32; g.W = c->t_w1; g.w_dtype = c->a.dtype;
   g.M = n; g.N = W; g.K = W; g.epi = EPI_BIAS_SILU; g.out = c->tc1; g.ldo = W; g.bias = c->t_b1;
-  launch_gemm_ffma(g, s);
+  launch_gemm_table(g, s);
   g.A = c->tc1; g.W = c->t_w2; g.out = c->tc2; g.bias = c->t_b2;
-  launch_gemm_ffma(g, s);
+  launch_gemm_table(g, s);
   g.A = c->tc2; g.W = c->w_mod; g.N = c->rowlen; g.epi = EPI_STORE; g.bias = c->b_mod;
   g.out = c->tab + (size_t)c->tab_rows * c->rowlen; g.ldo = c->rowlen;
-  launch_gemm_ffma(g, s);
+  launch_gemm_table(g, s);
   if (c->a.kind == UAD_KIND_CONCAT) {
     // the time half of the input MLP: e(tau) W_it + b_it after the (constant) modulation
     GemmArgs t;
     t.A = c->temb; t.lda = W; t.a_dtype = F32; t.W = c->w_it; t.w_dtype = c->a.dtype;
     t.M = n; t.N = W; t.K = W; t.epi = EPI_STORE; t.bias = c->b_it;
     t.out = c->tab + (size_t)c->tab_rows * c->rowlen + concat_off(c); t.ldo = c->rowlen;
-    launch_gemm_ffma(t, s);
+    launch_gemm_table(t, s);
   }
   CK(cudaGetLastError());
   for (int r = 0; r < n; ++r) c->tau_row[fr[r]] = c->tab_rows + r;

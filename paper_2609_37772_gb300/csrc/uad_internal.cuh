@@ -195,6 +195,7 @@ void launch_add_tau_silu(const float* x, const float* tab, int stride, int off, 
 
 // ffma.cu: CUDA-core GEMM and attention
 void launch_gemm_ffma(const GemmArgs& a, cudaStream_t s);
+void launch_gemm_table(const GemmArgs& a, cudaStream_t s);   // fp32 activations, every output summed over ascending k
 void launch_attn_rows(const AttnArgs& a, cudaStream_t s);
 void ffma_prepare(int head_dim);   // opt in to > 48 KB dynamic shared memory on the current device
 

@@ -819,3 +819,24 @@ def test_cuda_core_gemm_and_attention_edges(dtype, dh, heads, kv, width, mlp, ch
         check(c, c.gpu(noise, bud), c.oracle(noise, bud), bud, TOL[dtype])
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("name,robots", [("tiny", 2), ("pi0_small", 3), ("dit_small", 2), ("concat_small", 2)])
+def test_flow_times_filled_early_or_late_give_the_same_bits(name, robots):
+    """A time-table row does not depend on how many rows are filled with it: a chunk has the same bits
+    whether its flow times come one chunk at a time or hundreds at once from prepare_times."""
+    a = ARCHS[name]
+    blob = make_weights(a, seed=57)
+    noise = make_noise(a, batch=robots, seed=57)
+    bud = np.stack([group_budgets(a.chunk_len, [(0, 2, 3), (3, a.chunk_len - 1, 5)])] * robots)
+    got = []
+    for prepared in (0, 5, 12, 28):
+        c = Case(a, B=robots, seed=57, blob=blob)
+        try:
+            if prepared:
+                c.ex.prepare_times(prepared)
+            got.append(c.gpu(noise, bud))
+        finally:
+            c.close()
+    for g in got[1:]:
+        assert np.array_equal(g["final"], got[0]["final"]) and np.array_equal(g["ghost"], got[0]["ghost"])
