@@ -18,6 +18,7 @@
 #include <cudaTypedefs.h>
 
 #include "uad_internal.cuh"
+#include "attn_ring.cuh"
 #include "ptx.cuh"
 
 namespace uad {
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
 // rescaled in place (after the previous P V has completed). Otherwise the stale M stays: every P
 // is at most 2^8, and O and the row sum share the same reference, so O / sum is unchanged. O / l
 // is written in bf16.
-constexpr int kKC2 = 128;                       // keys per chunk
+constexpr int kKC2 = kRingChunk;                // keys per chunk
 constexpr uint32_t kTmem2 = 512;                // S buffers at columns [0,128) and [128,256), O at [256, 256 + DV)
 constexpr float kRescaleLog2 = 8.f;             // raise M only past this many powers of two
 constexpr int kSlots2 = 5;                      // operand ring slots
@@ -251,7 +252,6 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   constexpr int NC = DH / 64;
   constexpr int KP = attn2_kpieces(DH);          // K pieces per chunk
   constexpr int NCP = NC / KP;                   // 64-dim blocks of 128 keys per piece
-  constexpr int PPC = KP + 2;                    // ring entries per chunk: K pieces, two Vt halves
   constexpr uint32_t QB = DH * kQT * 2;          // Q: NC blocks of 128 rows x 64
   constexpr uint32_t PB = NCP * kKC2 * 128;      // one K piece
   constexpr uint32_t VBLK = DV * 128;            // one Vt half: DV rows x 64 keys
@@ -301,35 +301,30 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
   const uint32_t tO = tmem + 2 * kKC2;
   pdl_trigger();
 
-  // Ring entries in the order the MMAs read them: K of chunk 0, then per chunk c the K of chunk
-  // c + 1 (S runs a chunk ahead of P V) and the Vt of chunk c.
-  const auto k_entry = [&](int c, int j) { return c == 0 ? j : KP + (c - 1) * PPC + j; };
-  const auto v_entry = [&](int c, int h) { return KP + c * PPC + (c + 1 < nck ? KP : 0) + h; };
+  const AttnRing ring{KP, nck};   // its entries, in the order the MMAs read them
 
   if (threadIdx.x == 128) {
     // producer: ring entry e into slot e % kSlots2 once entry e - kSlots2 has been read. The first entries that
     // hold prefix keys alone, which no kernel of the step loop writes, are requested before the wait for the
-    // kernel that writes Q and the chunk's keys
+    // kernel that writes Q and the chunk's keys (not always the whole ring: with one K piece a chunk, head
+    // dim 64, its fifth entry is K of chunk 2)
     const uint64_t pol = policy_evict_last();
-    const int total = KP + (nck - 1) * PPC + 2;
+    const int total = ring.total();
     const auto load = [&](int e) {
-      const int t = e % kSlots2, f = e - KP, c = e < KP ? -1 : f / PPC < nck - 1 ? f / PPC : nck - 1;
-      const int r = e < KP ? e : f - c * PPC;                        // place in the group of chunk c
-      const bool k = e < KP || (c + 1 < nck && r < KP);
-      if (k) {
+      const int t = e % kSlots2;
+      const AttnRing::Entry x = ring.at(e);
+      if (x.k) {
         mbar_expect_tx(r_full + t, PB);
 #pragma unroll
         for (int cc = 0; cc < NCP; ++cc)
-          tma_3d(sR + t * SLOT + cc * (kKC2 * 128), &tk, (r * NCP + cc) * 64, (c + 1) * kKC2, kvz, r_full + t, pol);
+          tma_3d(sR + t * SLOT + cc * (kKC2 * 128), &tk, (x.part * NCP + cc) * 64, x.chunk * kKC2, kvz, r_full + t, pol);
       } else {
-        const int h = c + 1 < nck ? r - KP : r;
         mbar_expect_tx(r_full + t, VBLK);
-        tma_3d(sR + t * SLOT, &tv, c * kKC2 + h * 64, d0, kvz, r_full + t, pol);
+        tma_3d(sR + t * SLOT, &tv, x.chunk * kKC2 + x.part * 64, d0, kvz, r_full + t, pol);
       }
     };
     int e = 0;
-    if (2 * kKC2 <= p.prefix)   // the ring's first entries: K of chunks 0 and 1, Vt of chunk 0
-      for (; e < kSlots2 && e < total; ++e) load(e);
+    for (const int n = ring.early(kSlots2, p.prefix); e < n; ++e) load(e);
     pdl_wait();
     mbar_expect_tx(q_full, QB);
 #pragma unroll
@@ -346,7 +341,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
       const int sb = c & 1;
       if (c >= 2) ok = mbar_wait(s_empty + sb, ((c >> 1) - 1) & 1, p.err, 44);
       for (int j = 0; j < KP && ok; ++j) {
-        const int e = k_entry(c, j), t = e % kSlots2;
+        const int e = ring.k_entry(c, j), t = e % kSlots2;
         ok = mbar_wait(r_full + t, (e / kSlots2) & 1, p.err, 43);
         if (!ok) break;
         tc_fence_after();
@@ -364,7 +359,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
       if (ch + 1 < nck) issue_s(ch + 1);
       ok = ok && mbar_wait(p_full + sb, (ch >> 1) & 1, p.err, 45);
       for (int h = 0; h < 2 && ok; ++h) {
-        const int e = v_entry(ch, h), t = e % kSlots2;
+        const int e = ring.v_entry(ch, h), t = e % kSlots2;
         ok = mbar_wait(r_full + t, (e / kSlots2) & 1, p.err, 46);
         if (!ok) break;
         tc_fence_after();

@@ -840,3 +840,27 @@ def test_flow_times_filled_early_or_late_give_the_same_bits(name, robots):
             c.close()
     for g in got[1:]:
         assert np.array_equal(g["final"], got[0]["final"]) and np.array_equal(g["ghost"], got[0]["ghost"])
+
+
+@pytest.mark.parametrize("name,robots,prefix", [("concat_small", 16, p) for p in (127, 128, 255, 256, 300, 383, 384)] +
+                         [("concat_small", 20, 300), ("pi0_small", 40, 256), ("pi0_small", 40, 300)])
+def test_one_pass_attention_prefix_lengths(name, robots, prefix):
+    """The one-pass attention where its first loads are prefix keys alone, end just before the chunk's own
+    keys or would reach into them (head dims 64 and 128): against the oracle, the same bits over repeated
+    chunks whose keys change in every evaluation."""
+    a = ARCHS[name].replace(name=f"{name}_p{prefix}", prefix_len=prefix)
+    c = Case(a, B=robots, seed=58)
+    try:
+        noise = make_noise(a, batch=robots, seed=58)
+        bud = np.stack([group_budgets(a.chunk_len, [(0, 3, 2), (4, a.chunk_len - 1, 3)])] * robots)
+        res = c.gpu(noise, bud)
+        for b in (0, robots // 2, robots - 1):
+            ref = denoise(build_model(a, c.blob, c.pre[b]).velocity, noise[b], bud[b])
+            assert rel_err(res["final"][b], ref["final"]) <= TOL["bf16"], b
+            assert rel_err(res["ghost"][b], ref["ghost"]) <= TOL["bf16"], b
+        for _ in range(3):
+            again = c.gpu(noise[::-1].copy(), bud)   # other keys in between
+            again = c.gpu(noise, bud)
+            assert np.array_equal(again["final"], res["final"])
+    finally:
+        c.close()
