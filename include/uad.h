@@ -250,7 +250,8 @@ int uad_tile_weight(const float* w, int32_t K, int32_t N, uint16_t* out);
  * or NULL; out: device fp32 [M][N]. Needs N % 128 == 0, K % 64 == 0, M >= 1.
  * An error word is allocated by the library with cudaMalloc on the first call on each device and kept
  * until exit; K splits are combined on the chip, so calls on different streams may overlap.
- * Asynchronous on `stream` (a cudaStream_t, NULL = legacy stream). Returns UAD_OK, UAD_EINVAL,
+ * Asynchronous on `stream` (a cudaStream_t, NULL = legacy stream) and in its order: x, w_tiled and bias may
+ * be written by work queued on it before the call. Returns UAD_OK, UAD_EINVAL,
  * UAD_ENOMEM or UAD_ECUDA. */
 int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out, int32_t M,
                int32_t N, int32_t K, void* stream);

@@ -8,8 +8,8 @@
 // the S partial rows of its tokens in rank order (the result does not depend on timing) and applies
 // the epilogue to them. The receive area lies apart from the operand ring, so that rows arrive while other
 // CTAs' MMAs still run (aliased on the ring: DiT head 916 us per evaluation, apart 840; four robots 1246 and
-// 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. Weights are requested before the wait for the kernel that produces the
-// activations. Every wait is bounded; the cluster barriers are reached on every path.
+// 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. An expert's weights are requested before the wait for the
+// kernel that produces the activations (a caller's after it: TcGemmArgs::ordered). Every wait is bounded; the cluster barriers are reached on every path.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       const uint64_t pol = policy_evict_first();
       const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + ((size_t)(nt * kBM / kTileM) * KC + c0) * kTileBytes + nt * kBM % kTileM * kBK * 2;
       const int first = nkb < ring ? nkb : ring;
+      if (p.ordered) pdl_wait();
       for (int i = 0; i < first; ++i) {
         mbar_expect_tx(full + i, kSlot);
         bulk_g2s(smem + (size_t)i * kSlot, wt + (size_t)i * kTileBytes, kSlotA, full + i, pol);
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     const bool resid = epi == EPI_RESID_H;
     const bool vec = reinterpret_cast<uintptr_t>(p.out) % 16 == 0 && p.ldo % 4 == 0;   // a caller's pointer may not be
     float4 hv[U], gv[U], bias = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.ordered) pdl_wait();
     if (p.bias) {
       const int nb = p.n_store > 0 ? p.n_store : p.N;
       if (n < nb) bias.x = __ldg(p.bias + n);

@@ -307,9 +307,10 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   pdl_trigger();
   if (threadIdx.x == 0) {
     // ---- producer: weight block (bulk copy) + activation tile (tensor map) per K chunk.
-    //      Weights are constant: the first ring's worth is requested before waiting for the
-    //      kernel that produces the activations. ----
+    //      An expert's weights are constant: the first ring's worth is requested before waiting
+    //      for the kernel that produces the activations. ----
     const uint64_t pol = policy_evict_first();
+    if (p.ordered) pdl_wait();
     const uint8_t* wt = static_cast<const uint8_t*>(p.w_tiled) + (size_t)t * nch * kStageA;
     const int first = nch < stages ? nch : stages;
     for (int i = 0; i < first; ++i) {

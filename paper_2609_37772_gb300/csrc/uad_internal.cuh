@@ -214,8 +214,11 @@ struct TcGemmArgs {
   const int* tau_row = nullptr;
   int n_store = 0;                 // EPI_STORE: > 0: rows n >= n_store are padding (not stored, no bias)
   int* err = nullptr;              // set to a nonzero code if a bounded wait gave up
+  int ordered = 0;                 // 1: weights and bias are a caller's tensors, which work before this kernel on its
+                                   // stream may write: nothing is read before the dependent-launch wait.
+                                   // 0: an expert's own, constant, requested before it
   int wide = 0;                    // 1: the persistent wide form (one CTA per SM walking units of
-                                   // tn tokens x 128 weight rows x a K range), 0: narrow split-K tiles
+                                   // tn tokens x 128 weight rows x a K range), 0: narrow tiles, no K splits
   int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)
   int cl_bm = 128;                 //    weight rows of a tile: 128 or 64
   int cl_code = 0;                 //    which projections share its code: kClAny, kClPlain or kClOwn

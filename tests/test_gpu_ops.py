@@ -105,3 +105,33 @@ def test_linear_rejects_bad_shapes():
     assert uad.uad_linear(1, 1, None, 1, 50, 100, 64, None) == uad.UAD_EINVAL
     assert uad.uad_linear(1, 1, None, 1, 0, 128, 64, None) == uad.UAD_EINVAL
     assert uad.uad_linear(None, 1, None, 1, 50, 128, 64, None) == uad.UAD_EINVAL
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 512, 1536), (50, 1024, 512), (160, 8192, 128), (637, 1024, 2048)])
+def test_linear_reads_weights_and_bias_in_stream_order(M, N, K):
+    """A call's bias is the output of the call just before it on the stream, its weights are copied there in
+    between: on the cluster form (16 and 50 rows, long K) and the narrow form, each sees them complete."""
+    rng = np.random.default_rng(M + N + K)
+    st = torch.cuda.Stream()
+    big = 3072   # rows of the call that computes the bias: long enough that the next call's CTAs could start beside it
+    xb = torch.from_numpy(rng.normal(size=(big, K)).astype(np.float32)).to(torch.bfloat16).cuda()
+    x = torch.from_numpy(rng.normal(size=(M, K)).astype(np.float32)).to(torch.bfloat16).cuda()
+    ws = [(rng.normal(size=(K, N)) * 0.02).astype(np.float32) for _ in range(3)]
+    tiled = [torch.from_numpy(uad.tile_weight(w).view(np.int16)).cuda() for w in ws]
+    refs = [x.float().cpu().numpy().astype(np.float64) @ round_to_bf16(w).astype(np.float64) for w in ws]
+    lasts = [xb[-1].float().cpu().numpy().astype(np.float64) @ round_to_bf16(w).astype(np.float64) for w in ws]
+    wt = torch.zeros_like(tiled[0])
+    outb = torch.zeros(big, N, device="cuda")
+    outs = [torch.zeros(M, N, device="cuda") for _ in range(12)]
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        assert uad.uad_linear(xb.data_ptr(), tiled[i % 3].data_ptr(), None, outb.data_ptr(), big, N, K, st.cuda_stream) == 0
+        if i % 2:   # with the weights' copy between the two calls, and without
+            with torch.cuda.stream(st):
+                wt.copy_(tiled[(i + 1) % 3])
+        w = wt if i % 2 else tiled[(i + 1) % 3]
+        assert uad.uad_linear(x.data_ptr(), w.data_ptr(), outb[-1].data_ptr(), out.data_ptr(), M, N, K, st.cuda_stream) == 0
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        want = refs[(i + 1) % 3] + lasts[i % 3]
+        assert np.abs(out.cpu().numpy() - want).max() <= 1e-5 * np.abs(want).max(), i
