@@ -301,7 +301,9 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
                   *reinterpret_cast<uint2*>(dst + r) = pack4(v.x, v.y, v.z, v.w);
                 }
               } else {
-                // v: into this token's staged row (16-byte pieces swizzled by token), for the writes below
+                // v: into this token's staged row (16-byte pieces swizzled by token), for the writes below, once every
+                // lane of the row has read its own piece of it
+                __syncwarp(kLanes == 32 ? 0xffffffffu : 0xffffu << (16 * sub));
                 *reinterpret_cast<float4*>(T + (size_t)(t0 + tt) * kBM + 4 * (fl ^ (tt & (kLanes - 1)))) = v;
               }
             }
