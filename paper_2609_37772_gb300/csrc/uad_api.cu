@@ -146,8 +146,9 @@ struct uad_ctx {
   cudaStream_t worker = nullptr;
   cudaEvent_t ev_in = nullptr, ev_done = nullptr;
   // (robots, N*, persistent kernel): the whole chunk on the persistent kernel, else as many steps as
-  // graph_steps allows, launched until N* are done
-  std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
+  // graph_steps allowed when it was captured, launched until N* are done
+  struct StepGraph { cudaGraphExec_t exec = nullptr; int steps = 0; };
+  std::map<std::tuple<int, int, int>, StepGraph> graphs;
 
   // in-flight chunk
   bool in_flight = false;
@@ -851,9 +852,10 @@ void enqueue_steps(uad_ctx* c, int B, int n_steps, int count, bool step, cudaStr
   }
 }
 
-int launches_per_step(const uad_ctx* c, int B) {
+// step: on the persistent evaluation kernel (with the step epilogue at its end), else on the per-operation kernels.
+int launches_per_step(const uad_ctx* c, int B, bool step) {
   const uad_arch& a = c->a;
-  if (step_path(c, B)) return 1;   // persistent evaluation kernel with the step epilogue at its end
+  if (step) return 1;
   if (a.kind == UAD_KIND_DIT) return 11 * a.n_layers + 4;
   // per layer: norm, qkv, attention (split-KV + combine, or the one-pass kernel), o, norm,
   // gate/up, down
@@ -873,7 +875,7 @@ int launches_per_step(const uad_ctx* c, int B) {
 int graph_steps(const uad_ctx* c, int B, int n_steps) {
   int g = 1;
   for (int d = 1; d <= n_steps; ++d)
-    if (n_steps % d == 0 && d * launches_per_step(c, B) <= 256) g = d;
+    if (n_steps % d == 0 && d * launches_per_step(c, B, false) <= 256) g = d;
   return g;
 }
 
@@ -1406,9 +1408,9 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
   CK(cudaMemcpyAsync(c->noise, noise, (size_t)M * D * 4, cudaMemcpyDefault, s));
   if (c->use_graphs && !profile) {
     const auto key = std::make_tuple(B, steps, use_step ? 1 : 0);
-    const int per = use_step ? steps : graph_steps(c, B, steps);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
+      const int per = use_step ? steps : graph_steps(c, B, steps);
       cudaGraph_t g = nullptr;
       CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
       if (per == steps) enqueue_begin(c, B, steps, s);   // the chunk's only graph: begin joins it
@@ -1419,10 +1421,11 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
       e = cudaGraphInstantiate(&ex, g, 0);
       cudaGraphDestroy(g);
       if (e != cudaSuccess) return fail(c, UAD_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
-      it = c->graphs.emplace(key, ex).first;
+      it = c->graphs.emplace(key, uad_ctx::StepGraph{ex, per}).first;
     }
-    if (per != steps) enqueue_begin(c, B, steps, s);
-    for (int k = 0; k < steps; k += per) CK(cudaGraphLaunch(it->second, s));
+    const uad_ctx::StepGraph& sg = it->second;
+    if (sg.steps != steps) enqueue_begin(c, B, steps, s);
+    for (int k = 0; k < steps; k += sg.steps) CK(cudaGraphLaunch(sg.exec, s));
   } else if (profile) {
     // capture with an event-record node around every kernel, so that the event times are
     // GPU timestamps between graph nodes (no host launch gaps)
@@ -1431,7 +1434,7 @@ static int denoise_impl(uad_ctx* c, const float* noise, const uad_schedule* sc, 
     c->prof_next = 0;
     // create the events before capture
     {
-      int need = 2 * (1 + steps * launches_per_step(c, B)) + 8;
+      int need = 2 * (1 + steps * launches_per_step(c, B, use_step)) + 8;
       while ((int)c->prof_ev.size() < need) {
         cudaEvent_t e;
         CK(cudaEventCreate(&e));
@@ -1600,7 +1603,7 @@ int uad_step_times(const uad_ctx* c, double* ms, int32_t max_entries) {
 
 int uad_launches_per_chunk(const uad_ctx* c, int32_t batch, int32_t n_star) {
   if (!c || batch < 1 || n_star < 1) return UAD_EINVAL;
-  return 1 + n_star * launches_per_step(c, batch);
+  return 1 + n_star * launches_per_step(c, batch, step_path(c, batch));
 }
 
 int uad_so3_check(const float* w, int32_t n, float* log_exp, float* log_comp) {
@@ -1628,7 +1631,7 @@ int uad_set_wait_limit(uad_ctx* c, int64_t wait_ns, int32_t unreachable) {
   c->test_unreachable = unreachable;
   c->step_failed = false;   // the persistent kernel is tried again
   // the launch arguments are baked into the cached graphs
-  for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.exec);
   c->graphs.clear();
   return UAD_OK;
 }
@@ -1647,7 +1650,7 @@ void uad_destroy(uad_ctx* c) {
       return;
     }
   }
-  for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.exec);
   for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
   if (c->worker) cudaStreamDestroy(c->worker);
   if (c->ev_in) cudaEventDestroy(c->ev_in);

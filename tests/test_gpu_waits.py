@@ -4,6 +4,7 @@ ever makes, with a 1 ms limit. Every wait gives up, records its code and lets th
 down; uad_finish reports the error; the same context then runs a correct chunk."""
 import numpy as np
 import pytest
+import torch
 
 import paper_2609_37772_gb300 as uad
 from oracle.model import build_model
@@ -75,5 +76,47 @@ def test_expired_wait_falls_back_to_per_operation_kernels():
         ex.set_wait_limit()
         names = {r["name"] for r in ex.profile(noise, bud[None])}
         assert names == {"begin", "step_kernel"}, names
+    finally:
+        ex.close()
+
+
+def test_a_cached_chunk_runs_once_after_a_wait_ran_out():
+    """Four robots of 16 tokens leave the persistent kernel no room for their flow times, so their chunks run on
+    the per-operation kernels beside one-robot chunks on the persistent one. Their cached graph keeps its
+    own number of steps when a wait of the persistent kernel runs out later: the chunk takes as long as
+    before (not twice) and gives the same bits."""
+    a = ARCHS["pi0_small"].replace(name="pi0_small_h16", chunk_len=16)
+    ex = uad.Expert(a, make_weights(a, seed=23), max_batch=4)
+    noise = make_noise(a, batch=4, seed=23)
+    bud = np.stack([group_budgets(16, [(0, 3, 4 + b), (4, 15, 16)]) for b in range(4)])
+    dev = torch.from_numpy(noise).cuda()
+    stream = torch.cuda.Stream()
+
+    def chunk():
+        ms = []
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record(stream)
+            ex.denoise(dev, bud, stream=stream)
+            t1.record(stream)
+            r = ex.finish(timeout_us=60_000_000)
+            torch.cuda.synchronize()
+            ms.append(t0.elapsed_time(t1))
+        return r, min(ms)
+
+    try:
+        for b in range(4):
+            ex.set_prefix(b, *make_prefix_kv(a, robot=b, seed=23))
+        names = {r["name"] for r in ex.profile(noise, bud)}
+        assert "step_kernel" not in names, names
+        ex.set_wait_limit(wait_ns=1_000_000, unreachable=1)
+        first, t_first = chunk()
+        ex.denoise(noise[:1], bud[:1])
+        r = ex.finish(timeout_us=60_000_000, check=False)
+        assert r["rc"] == uad.UAD_ECUDA and "per-operation kernels" in uad.uad_last_error(ex.h).decode()
+        again, t_again = chunk()
+        print(f"16 steps of four robots: {t_first:.3f} ms, after the expired wait {t_again:.3f} ms")
+        assert np.array_equal(again["final"], first["final"]) and again["evals"] == first["evals"] == 16
+        assert t_again <= 1.4 * t_first
     finally:
         ex.close()
