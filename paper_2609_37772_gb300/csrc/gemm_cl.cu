@@ -414,18 +414,15 @@ ClKernel cl_kernel(const TcGemmArgs& a) {
          : a.cl_code == kClPlain && !gated ? gemm_cl_kernel<kPlain, BM, BOX> : gemm_cl_kernel<kAny, BM, BOX>;
 }
 template <int BM, int BOX>
-void cl_prepare() {
+int cl_prepare() {
   for (const auto k : {gemm_cl_kernel<kAny, BM, BOX>, gemm_cl_kernel<kPlain, BM, BOX>, gemm_cl_kernel<EPI_QKV_TC, BM, BOX>,
                        gemm_cl_kernel<EPI_GEGLU, BM, BOX>, gemm_cl_kernel<EPI_RESID_H, BM, BOX>})
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem) != cudaSuccess) return -1;
+  return 0;
 }
 }  // namespace
 
-void gemm_cl_prepare() {
-  cl_prepare<128, 64>();
-  cl_prepare<128, 16>();
-  cl_prepare<64, 64>();
-}
+int gemm_cl_prepare() { return cl_prepare<128, 64>() || cl_prepare<128, 16>() || cl_prepare<64, 64>() ? -1 : 0; }
 
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
   const int KC = a.K / kBK, per = (KC + a.splits - 1) / a.splits, rows = a.M < kBN ? a.M : kBN;

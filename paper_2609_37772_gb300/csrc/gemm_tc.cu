@@ -22,6 +22,7 @@
 
 #include "uad_internal.cuh"
 #include "ptx.cuh"
+#include "once_per_device.h"
 
 namespace uad {
 
@@ -600,17 +601,19 @@ static size_t gemm_tc_pers_smem_bytes(int tn) {
          (2 * st + 5) * 8 + 16;
 }
 
-void gemm_tc_prepare() {
-  static bool done = false;
-  if (done) return;
-  done = true;
-  gemm_cl_prepare();
-  cudaFuncSetAttribute(gemm_tc_pers_kernel<256, kPersStages256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)gemm_tc_pers_smem_bytes(256));
-  cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)gemm_tc_pers_smem_bytes(128));
-  cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)gemm_tc_smem_bytes(kTcMaxStages));
+int gemm_tc_prepare() {
+  static OncePerDevice once;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+  return once.run(dev, [] {
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (gemm_cl_prepare() ||
+        cudaFuncSetAttribute(gemm_tc_pers_kernel<256, kPersStages256>, at, (int)gemm_tc_pers_smem_bytes(256)) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128>, at, (int)gemm_tc_pers_smem_bytes(128)) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_tc_kernel, at, (int)gemm_tc_smem_bytes(kTcMaxStages)) != cudaSuccess)
+      return -1;
+    return 0;
+  });
 }
 
 // Wide tiles (MMA N up to 256 tokens) run the tensor cores near their rate (N = 64 runs at a

@@ -48,7 +48,7 @@ int launch_linear(const void* x, const void* w_tiled, const float* bias, float* 
   gemm_tc_plan(M, N, K, sms, EPI_STORE, &a);   // the tile selection of the velocity network's projections
   a.epi = EPI_STORE; a.out = out; a.ldo = N; a.out_dtype = F32; a.bias = bias;
   a.err = err; a.ordered = 1;
-  gemm_tc_prepare();
+  if (gemm_tc_prepare()) return UAD_ECUDA;
   launch_gemm_tc(&tm, a, s);
   return cudaGetLastError() == cudaSuccess ? UAD_OK : UAD_ECUDA;
 }

@@ -1165,7 +1165,10 @@ int uad_init(const uad_arch* arch, const float* weights, size_t n_floats, uad_ct
       part = std::max({part, residual_planes(c, b * H, c->qd) * (size_t)b * H * W,
                        residual_planes(c, b * H, F) * (size_t)b * H * W});
     TRY(dalloc_t(c, &c->part, part));
-    gemm_tc_prepare();
+    if (gemm_tc_prepare()) {
+      fail(c, UAD_ECUDA, "projection kernels: shared memory opt-in failed");
+      TRY(UAD_ECUDA);
+    }
   }
   TRY(step_setup(c));
   TRY(dalloc_t(c, &c->E, (size_t)a.max_batch * D));

@@ -229,7 +229,7 @@ struct TcGemmArgs {
 int encode_act_tmap(CUtensorMap* m, const void* base, int K, int rows, int box_rows);
 // rows of the boxes that a projection of M tokens is read in
 __host__ __device__ constexpr int act_box_rows(int M) { return M <= 16 ? 16 : 64; }
-void gemm_tc_prepare();
+int gemm_tc_prepare();   // opts its kernels in to their shared memory on the current device, once on each; 0 on success
 int gemm_tc_use_wide(int M, int N, int sms);    // 1: the persistent wide form serves this projection
 int gemm_tc_resid_wide(int M, int N, int sms);  // the same for a residual projection, which may split K into planes
 // The tile plan of one projection (wide form, tokens per tile, K splits) into a.
@@ -239,7 +239,7 @@ constexpr int kClMaxSplits = 8;
 constexpr int kClAny = 0, kClPlain = 1, kClOwn = 2;   // TcGemmArgs::cl_code
 void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a);   // K splits and rows of a tile
 bool gemm_cl_serves(int M, int N, int sms);
-void gemm_cl_prepare();
+int gemm_cl_prepare();   // part of gemm_tc_prepare
 void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
 void gemm_tc_prefix_plan(int M, int N, int K, int sms, TcGemmArgs* a);   // EPI_PREFIX_KV: no K splits
 void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s);
