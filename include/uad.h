@@ -248,13 +248,25 @@ int uad_tile_weight(const float* w, int32_t K, int32_t N, uint16_t* out);
  * the projection kernel of every velocity-network layer (Sec. 3, Eq. 1).
  * x: device bf16 [M][K]; w_tiled: device, the layout of uad_tile_weight; bias: device fp32 [N]
  * or NULL; out: device fp32 [M][N]. Needs N % 128 == 0, K % 64 == 0, M >= 1.
- * An error word is allocated by the library with cudaMalloc on the first call on each device and kept
- * until exit; K splits are combined on the chip, so calls on different streams may overlap.
+ * 4 KiB of error words are allocated by the library with cudaMalloc on the first call on each device and
+ * kept until exit; K splits are combined on the chip, so calls on different streams may overlap.
  * Asynchronous on `stream` (a cudaStream_t, NULL = legacy stream) and in its order: x, w_tiled and bias may
  * be written by work queued on it before the call. Returns UAD_OK, UAD_EINVAL,
  * UAD_ENOMEM or UAD_ECUDA. */
 int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out, int32_t M,
                int32_t N, int32_t K, void* stream);
+
+/* Whether the finished projections of the current device (uad_linear, uad_linear_static_scratch) are complete.
+ * Every wait inside their kernels is bounded (2 s). One that runs out ends its call, whose output is then
+ * incomplete, and no other call, before, after or beside it. Returns UAD_ECUDA if one ran out in the last
+ * 1024 calls of the process since the last query (and forgets it), UAD_OK otherwise. Synchronous on the
+ * legacy stream: synchronise the calls' streams first; not while a stream is being captured. */
+int uad_linear_status(void);
+
+/* Testing aid for those waits (not part of the method): uad_linear as if one of its waits had just run out, so that
+ * every other that is not over within microseconds gives up and its part of the output is not computed. */
+int uad_linear_check(const void* x, const void* w_tiled, const float* bias, float* out, int32_t M,
+                     int32_t N, int32_t K, void* stream);
 
 /* ---- The same projection op for callers that cannot allocate device memory ---------------
  * The paper has no counterpart: this serves deployments rather than the method. A real-time
@@ -262,16 +274,15 @@ int uad_linear(const void* x, const void* w_tiled, const float* bias, float* out
  * time and synchronize the device, stalling the control loop), and a host framework whose
  * caching allocator already holds the GPU's memory cannot take a stray allocation. This entry
  * point computes exactly what uad_linear computes but allocates nothing: no cudaMalloc,
- * cudaFree or allocating library call. It needs no scratch beyond an error word inside the
+ * cudaFree or allocating library call. It needs no scratch beyond error words (4 KiB) inside the
  * library's device image.
  *   - Limits: M * N <= UAD_LINEAR_STATIC_MAX_ELEMS and (N / 128) * ceil(M / 64) <=
  *     UAD_LINEAR_STATIC_MAX_TILES; larger calls return UAD_ETOOBIG and launch nothing.
- *   - The first call on a device looks up that word's device address (cudaGetSymbolAddress,
+ *   - The first call on a device looks up their device address (cudaGetSymbolAddress,
  *     which may load the library's device code: with lazy module loading, the CUDA default,
  *     the driver reserves its memory only then). Make one warm-up call per device during
  *     start-up, before any stream capture begins and before the control loop runs, so that
  *     the device code is resident when "allocates nothing" matters.
- *   - Every call clears the error word (asynchronously, on `stream`) before its kernel.
  * Arguments, layout and other errors are those of uad_linear. */
 #define UAD_ETOOBIG (-7)
 #define UAD_LINEAR_STATIC_MAX_ELEMS (1 << 20)

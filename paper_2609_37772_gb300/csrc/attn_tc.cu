@@ -106,6 +106,8 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
 #pragma unroll
       for (int c = 0; c < NC; ++c)
         mma_kblock(tS, qd + c * (kQT * 128 >> 4), kd + c * (kKT * 128 >> 4), idesc_m128(kKT), c ? 1u : 0u);
+    } else {
+      mbar_drain_issued(bar_qk, 0);   // no copies in flight into shared memory of an exiting CTA
     }
     mma_commit(bar_s);
   }
@@ -175,11 +177,14 @@ __global__ void __launch_bounds__(128, 1) attn_tc_kernel(const __grid_constant__
 #pragma unroll
       for (int u = 0; u < kKT / 64; ++u)
         mma_kblock(tO, pd + u * (kQT * 128 >> 4), vd + u * (VBLK >> 4), idesc_m128(DV), u ? 1u : 0u);
+    } else {
+      mbar_drain_issued(bar_v, 0);
     }
     mma_commit(bar_o);
   }
   __syncwarp();
   const bool ok_o = mbar_wait(bar_o, 0, p.err, 24);
+  if (!ok_o) mbar_drain_issued(bar_o, 0);   // nor MMAs, once tensor memory is given back
   tc_fence_after();
 
   // ---- partial output row (unnormalised) + (max, sum): the row is staged in shared memory (all
@@ -333,6 +338,9 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
       if (e >= kSlots2 && !mbar_wait(r_empty + e % kSlots2, (e / kSlots2 - 1) & 1, p.err, 41)) break;
       load(e);
     }
+    // do not leave copies in flight into shared memory of an exiting CTA
+    mbar_drain_issued(q_full, 0);
+    for (int i = e - kSlots2 > 0 ? e - kSlots2 : 0; i < e; ++i) mbar_drain_issued(r_full + i % kSlots2, (i / kSlots2) & 1);
   } else if (threadIdx.x == 160) {
     // issuer: S(0); per chunk c: S(c + 1), then P V(c) once the softmax warps have written P(c)
     bool ok = mbar_wait(q_full, 0, p.err, 42);
@@ -374,6 +382,7 @@ __global__ void __launch_bounds__(192, 1) attn_tc2_kernel(const __grid_constant_
       mma_commit(s_empty + sb);
     }
     mma_commit(o_done);
+    mbar_drain_issued(o_done, 0);   // before tensor memory is given back
   }
   if (warp >= 4) {
     // producer / issuer warps: done issuing; wait for the output stage before releasing TMEM

@@ -9,7 +9,8 @@
 // the epilogue to them. The receive area lies apart from the operand ring, so that rows arrive while other
 // CTAs' MMAs still run (aliased on the ring: DiT head 916 us per evaluation, apart 840; four robots 1246 and
 // 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. An expert's weights are requested before the wait for the
-// kernel that produces the activations (a caller's after it: TcGemmArgs::ordered). Every wait is bounded; the cluster barriers are reached on every path.
+// kernel that produces the activations (a caller's after it: TcGemmArgs::ordered). Every wait is bounded; the cluster barriers are reached on every path, and no CTA
+// leaves with copies in flight into its shared memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
         tma_2d(smem + (size_t)st * kSlot + kSlotA, &tmx, (c0 + i) * kBK, m0, full + st);
       }
       // no copies in flight into shared memory that is reused, or of a CTA that exits
-      for (int i = issued - ring > 0 ? issued - ring : 0; i < issued; ++i) wait_bar(full + i % ring, (i / ring) & 1, p.err, 72);
+      for (int i = issued - ring > 0 ? issued - ring : 0; i < issued; ++i) mbar_drain_issued(full + i % ring, (i / ring) & 1);
     }
     __syncwarp();
     if (S > 1) {
@@ -142,6 +143,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   } else if (warp == kConsWarps + 1) {
     // ---- MMA issuer ----
     if (lane == 0) {
+      if (p.own_err && rank + nt + mt == 0) *reinterpret_cast<volatile int*>(p.err) = 0;
       const uint32_t tmem = *tmem_slot;
       const uint32_t idesc = idesc_rows(kBM, (mcount + 15) / 16 * 16);
       const uint64_t ring0 = sw128_desc(su32(smem));
@@ -212,6 +214,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     pdl_wait();
     if (resid) load_h(warp);
     const bool ok = wait_bar(done, 0, p.err, 74);
+    if (!ok) mbar_drain_issued(done, 0);   // the MMAs, before tensor memory is given back
     tc_fence_after();
     const uint32_t tm = tmem_base_after_wait(tmem_slot) + ((uint32_t)((warp & 3) * 32) << 16);
     __syncwarp();
@@ -234,6 +237,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
       }
     }
     const bool all = S == 1 || cnt == 0 || wait_bar(got, 0, p.err, 75);
+    if (!all) mbar_drain(got, 0, 2 * kWaitNs);   // the others' rows, which they send also if a wait of theirs gave up
     __syncwarp();
     if (S > 1) cluster_arrive();   // this CTA's rows are here: once every CTA says so, none reads another's memory
     if (ok && all) {

@@ -331,9 +331,10 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
     }
     // do not leave copies in flight into shared memory of an exiting CTA
     for (int i = issued - stages > 0 ? issued - stages : 0; i < issued; ++i)
-      mbar_wait(full + i % stages, (i / stages) & 1, p.err, 12);
+      mbar_drain_issued(full + i % stages, (i / stages) & 1);
   } else if (threadIdx.x == 32) {
     // ---- MMA issuer ----
+    if (p.own_err && t + mt == 0) *reinterpret_cast<volatile int*>(p.err) = 0;
     const uint64_t adesc = sw128_desc(su32(sA)), bdesc = sw128_desc(su32(sB));
     bool ok = true;
     for (int i = 0; i < nch && ok; ++i) {
@@ -352,6 +353,7 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
   // ---- epilogue: TMEM -> registers, one weight row (output feature) per thread ----
   pdl_wait();
   const bool ok = mbar_wait(done, 0, p.err, 14);
+  if (!ok) mbar_drain_issued(done, 0);   // the MMAs, before tensor memory is given back
   tc_fence_after();
   const int row = warp * 32 + lane;
   const int n = t * kBM + row;
@@ -447,11 +449,12 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
       }
       // do not leave copies in flight into shared memory of an exiting CTA
       for (int i = it - STAGES > 0 ? it - STAGES : 0; i < it; ++i)
-        mbar_wait(full + i % STAGES, (i / STAGES) & 1, p.err, 62);
+        mbar_drain_issued(full + i % STAGES, (i / STAGES) & 1);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // ---- MMA issuer ----
+      if (p.own_err && blockIdx.x == 0) *reinterpret_cast<volatile int*>(p.err) = 0;
       const uint32_t tmem = *tmem_slot;
       const uint64_t adesc = sw128_desc(su32(sA)), bdesc = sw128_desc(su32(sB));
       int it = 0, j = 0;
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
         if (ok) mma_commit(tfull + b);
       }
       mma_commit(done);
-      mbar_wait(done, 0, p.err, 65);
+      mbar_drain_issued(done, 0);   // before tensor memory is given back
     }
   } else {
     // ---- epilogue: group g = warps 2 + 4g .. 5 + 4g takes slices g, g + 4, ...; warp w reads

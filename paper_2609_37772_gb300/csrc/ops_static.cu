@@ -5,7 +5,7 @@
 // time and synchronize the device, stalling the control loop), and a host framework whose
 // caching allocator has already reserved the GPU's memory would see a stray allocation fail
 // or fragment its pool. uad_linear_static_scratch serves them: the projection combines its K splits
-// on the chip, and the kernel's error word is in the library's device image.
+// on the chip, and the kernels' error words are in the library's device image.
 #include <cstdio>
 #include <mutex>
 
@@ -14,27 +14,32 @@
 
 namespace uad {
 int launch_linear(const void* x, const void* w_tiled, const float* bias, float* out, int M, int N, int K, int* err,
-                  cudaStream_t s);
+                  bool stopped, cudaStream_t s);
+constexpr int kErrWords = 1024;
 int linear_tiles(int M, int N);
+int static_err_words(int** err, bool look_up);
 }  // namespace uad
 
 namespace {
 
-// The kernel's error word, part of the library's device image.
-static __device__ int g_linear_err;
+// The error words of the last calls, part of the library's device image.
+static __device__ int g_linear_err[uad::kErrWords];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 int* g_err_addr[kMaxDevices] = {};
 
+}  // namespace
+
 // Device address of g_linear_err on the current device. In host code the name only stands in for the
-// symbol, so the address is looked up once per device, with that device current.
-int err_on_current_device(int** err) {
+// symbol, so the address is looked up once per device, with that device current (look_up: now, if it has not
+// been; else null until it has been).
+int uad::static_err_words(int** err, bool look_up) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return UAD_ECUDA;
   if (dev < 0 || dev >= kMaxDevices) return UAD_EINVAL;
   std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_err_addr[dev]) {
+  if (!g_err_addr[dev] && look_up) {
     void* p = nullptr;
     const cudaError_t e = cudaGetSymbolAddress(&p, g_linear_err);
     if (e != cudaSuccess) {
@@ -47,8 +52,6 @@ int err_on_current_device(int** err) {
   return UAD_OK;
 }
 
-}  // namespace
-
 extern "C" int uad_linear_static_scratch(const void* x, const void* w_tiled, const float* bias, float* out,
                                          int32_t M, int32_t N, int32_t K, void* stream) {
   if (!x || !w_tiled || !out || M < 1 || N < 128 || N % 128 || K < 64 || K % 64) return UAD_EINVAL;
@@ -59,10 +62,7 @@ extern "C" int uad_linear_static_scratch(const void* x, const void* w_tiled, con
     return UAD_ETOOBIG;
   }
   int* err = nullptr;
-  const int rc = err_on_current_device(&err);
+  const int rc = uad::static_err_words(&err, true);
   if (rc) return rc;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // what an earlier call left must not end this one's waits
-  if (cudaMemsetAsync(err, 0, 4, s) != cudaSuccess) return UAD_ECUDA;
-  return uad::launch_linear(x, w_tiled, bias, out, M, N, K, err, s);
+  return uad::launch_linear(x, w_tiled, bias, out, M, N, K, err, false, static_cast<cudaStream_t>(stream));
 }

@@ -44,8 +44,8 @@ __device__ __forceinline__ bool mbar_peek(uint64_t* b, uint32_t parity) {
       : "=r"(ok) : "r"(su32(b)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Wait for the phase with the given parity; false at once if an error is already recorded in
-// *err, false with *err = code once `limit_ns` has passed.
+// Wait for the phase with the given parity; false with *err = code once `limit_ns` has passed, or, from the 64th
+// poll on, if an error is already recorded in *err.
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err, int code,
                                           unsigned long long limit_ns) {
   unsigned long long t0 = 0;
@@ -63,11 +63,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err
     }
   }
 }
-// Wait for own asynchronous work before a CTA exits: bounded by time only.
+// Wait for own asynchronous work before a CTA exits: bounded by time only, whatever has been recorded.
 __device__ __forceinline__ void mbar_drain(uint64_t* b, uint32_t parity, unsigned long long limit_ns) {
   const unsigned long long t0 = gtime();
   while (!mbar_test(b, parity))
     if (gtime() - t0 > limit_ns) return;
+}
+// The same for copies and MMAs that have been issued, which land within microseconds, in few instructions: bounded
+// by the number of polls.
+__device__ __forceinline__ void mbar_drain_issued(uint64_t* b, uint32_t parity) {
+  for (uint32_t it = 0; it < (1u << 22) && !mbar_test(b, parity); ++it) {
+  }
 }
 
 // ---- copies --------------------------------------------------------------------------------

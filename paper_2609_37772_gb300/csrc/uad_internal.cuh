@@ -217,6 +217,8 @@ struct TcGemmArgs {
   int ordered = 0;                 // 1: weights and bias are a caller's tensors, which work before this kernel on its
                                    // stream may write: nothing is read before the dependent-launch wait.
                                    // 0: an expert's own, constant, requested before it
+  int own_err = 0;                 // 1: err is this call's alone; cleared when the kernel starts (no wait looks at it for
+                                   // microseconds), so that nothing left there ends the call's waits
   int wide = 0;                    // 1: the persistent wide form (one CTA per SM walking units of
                                    // tn tokens x 128 weight rows x a K range), 0: narrow tiles, no K splits
   int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)

@@ -120,3 +120,38 @@ def test_a_cached_chunk_runs_once_after_a_wait_ran_out():
         assert t_again <= 1.4 * t_first
     finally:
         ex.close()
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 512, 6144), (50, 1024, 4096), (160, 8192, 512), (600, 4096, 1024), (2, 1536, 6144)])
+def test_a_stopped_projection_harms_no_other_call(M, N, K):
+    """A projection that runs as if one of its waits had run out (cluster form with 128 and 64 weight rows, narrow
+    and persistent form): it ends at once, uad_linear_status reports it once, and the calls after it on
+    its stream and beside it on another give what they always give, 1500 of them, so that each error word
+    is used again."""
+    rng = np.random.default_rng(M + N + K)
+    x = torch.from_numpy(rng.normal(size=(M, K)).astype(np.float32)).to(torch.bfloat16).cuda()
+    w = torch.from_numpy(uad.tile_weight((rng.normal(size=(K, N)) * 0.02).astype(np.float32)).view(np.int16)).cuda()
+    s0, s1 = torch.cuda.Stream(), torch.cuda.Stream()
+    outs = [torch.full((M, N), float("nan"), device="cuda") for _ in range(12)]
+    torch.cuda.synchronize()
+
+    def call(entry, out, s):
+        assert entry(x.data_ptr(), w.data_ptr(), None, out.data_ptr(), M, N, K, s.cuda_stream) == 0
+
+    uad.uad_linear_status()
+    call(uad.uad_linear, outs[0], s0)
+    torch.cuda.synchronize()
+    assert uad.uad_linear_status() == uad.UAD_OK
+    for _ in range(5):
+        call(uad.uad_linear_check, outs[1], s0)
+        call(uad.uad_linear, outs[2], s1)
+        call(uad.uad_linear, outs[3], s0)
+    torch.cuda.synchronize()
+    assert uad.uad_linear_status() == uad.UAD_ECUDA
+    assert uad.uad_linear_status() == uad.UAD_OK
+    call(uad.uad_linear_check, outs[1], s0)
+    for i in range(1500):
+        call(uad.uad_linear, outs[4 + i % 8], s0 if i % 3 else s1)
+    torch.cuda.synchronize()
+    assert torch.isfinite(outs[0]).all()
+    assert all(torch.equal(o, outs[0]) for o in outs[2:])
