@@ -29,6 +29,11 @@ constexpr int kTileBytes = kTileM * kBK * 2;     // a k-block of the tiled weigh
 // that a fifth slot of weights fits (16-layer DiT expert, 16 tokens: 772 -> 762 us per evaluation; two boxes of 16
 // for up to 32 tokens lost 1%).
 constexpr int kConsWarps = 8, kCons = 32 * kConsWarps;
+// The tensor cores' accumulation truncates, so its error grows with the run of products: a CTA's k-blocks take turns
+// over one, two or four accumulators, which are added in fp32, rounded to nearest, when the tile is read out.
+// Products of positive numbers, mean error of 16 x 6144 x 1536 1.5e-6 with one accumulator, 2.7e-7 with four; DiT
+// expert, one / four robots 755 / 1070 -> 759 / 1084 us per evaluation, 18-layer expert at one robot 672 -> 677.
+constexpr int kTmCols = 256;                     // tensor memory of a CTA, half an SM's: four accumulators of 64 tokens
 constexpr int kThreads = kCons + 64;             // + producer warp, + MMA warp
 constexpr unsigned long long kWaitNs = 2000000000ull;
 
@@ -71,7 +76,9 @@ __host__ __device__ __forceinline__ size_t cl_recv_bytes(int rows, int splits, i
 // so it matters which projections share code (TcGemmArgs::cl_code).
 constexpr int kAny = -2, kPlain = -1;
 template <int E, int kBM, int kBox>
-__global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring) {
+__global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_constant__ CUtensorMap tmx, TcGemmArgs p, int ring_sets) {
+  // in one word: a field of its own, further on in the arguments, cost 1% (a cold line of constant memory)
+  const int ring = ring_sets & 255, sets = ring_sets >> 8;   // ring slots, accumulators
   extern __shared__ uint8_t smem_raw[];
   constexpr int kSlotA = kBM * kBK * 2, kSlot = kSlotA + kBox * kBK * 2;
   constexpr int kLanes = kBM / 4, TP = 32 / kLanes;   // lanes that share a token row, rows a warp takes at once
@@ -81,6 +88,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   const int m0 = mt * kBN, mcount = p.M - m0 < kBN ? p.M - m0 : kBN;
   const int per = (mcount + S - 1) / S, t0 = rank * per;            // token rows this CTA finishes
   const int cnt = mcount - t0 < 0 ? 0 : mcount - t0 < per ? mcount - t0 : per;
+  const int width = (mcount + 15) / 16 * 16;   // columns of an accumulator
   float* T = reinterpret_cast<float*>(smem);
   const int rows = p.M < kBN ? p.M : kBN;
   float* recv = reinterpret_cast<float*>(smem + cl_ring_bytes(ring, rows, kBM));
@@ -102,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     if (S > 1 && cnt > 0) mbar_expect_tx(got, (uint32_t)((S - 1) * cnt * kBM * 4));
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(kBN));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(kTmCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
@@ -145,14 +153,16 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     if (lane == 0) {
       if (p.own_err && rank + nt + mt == 0) *reinterpret_cast<volatile int*>(p.err) = 0;
       const uint32_t tmem = *tmem_slot;
-      const uint32_t idesc = idesc_rows(kBM, (mcount + 15) / 16 * 16);
+      const uint32_t idesc = idesc_rows(kBM, width), last = tmem + (sets - 1) * width;
+      uint32_t d = tmem;
       const uint64_t ring0 = sw128_desc(su32(smem));
       for (int i = 0; i < nkb; ++i) {
         const int st = i % ring;
         if (!wait_bar(full + st, (i / ring) & 1, p.err, 73)) break;
         tc_fence_after();
         const uint64_t a = ring0 + (uint64_t)(st * (kSlot >> 4));
-        mma_kblock(tmem, a, a + (kSlotA >> 4), idesc, i ? 1u : 0u);
+        mma_kblock(d, a, a + (kSlotA >> 4), idesc, i >= sets ? 1u : 0u);
+        d = d == last ? tmem : d + width;
         if (i + ring < nkb) mma_commit(empty + st);
       }
       mma_commit(done);
@@ -218,12 +228,23 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
     tc_fence_after();
     const uint32_t tm = tmem_base_after_wait(tmem_slot) + ((uint32_t)((warp & 3) * 32) << 16);
     __syncwarp();
-    for (int q = 16 * (warp >> 2); q < mcount; q += 32) {   // warps 4-7 take the odd 16-token slices
-      float v[16];
-      tmem_ld16(tm + q, v);
+    if (sets <= 2) {
+      for (int q = 16 * (warp >> 2); q < mcount; q += 32) {   // warps 4-7 take the odd 16-token slices
+        float v[16];
+        if (sets == 2) tmem_sum16(tm + q, tm + width + q, v);
+        else tmem_ld16(tm + q, v);
 #pragma unroll
-      for (int e = 0; e < 16; ++e)
-        if (kBM == 128 || lane < 16) T[(q + e) * kBM + row] = v[e];
+        for (int e = 0; e < 16; ++e)
+          if (kBM == 128 || lane < 16) T[(q + e) * kBM + row] = v[e];
+      }
+    } else {
+      for (int q = 8 * (warp >> 2); q < width; q += 16) {
+        float v[8];
+        tmem_sum8x4(tm + q, width, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (kBM == 128 || lane < 16) T[(q + e) * kBM + row] = v[e];
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     named_sync(1, kCons);
@@ -358,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 2) gemm_cl_kernel(const __grid_const
   if (S > 1) cluster_wait();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kBN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kTmCols));
   }
 }
 
@@ -390,6 +411,12 @@ void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
   while (s < half && K > 768 * s) ++s;
   s = s < 1 ? 1 : s > kClMaxSplits ? kClMaxSplits : s;
   a->splits = s < KC ? s : KC;
+  // Accumulators: as many as keep a run to the k-blocks that a CTA would sum if K were cut until the grid had one CTA
+  // an SM (two, where that is more than four k-blocks), however few splits a cluster can have
+  const int t64 = N / kTileM * mt, nkb = KC / a->splits, most = (KC + a->splits - 1) / a->splits;
+  const auto run_of = [&](int ctas) { return (KC * t64 + ctas / 2) / ctas > 1 ? (KC * t64 + ctas / 2) / ctas : 1; };
+  const int run = run_of(sms) <= 4 ? run_of(sms) : run_of(2 * sms) > 4 ? run_of(2 * sms) : 4;
+  a->cl_sets = most <= run || nkb < 2 ? 1 : most <= 2 * run || nkb < 4 ? 2 : 4;
 }
 
 // The cluster form serves every projection of one 64-token tile, and with more tokens those with so
@@ -433,7 +460,7 @@ void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s)
   int ring = per < kClMaxStages ? per : kClMaxStages;
   while (gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm) > kClSmem) --ring;   // three slots at least
   launch_cluster(a.cl_bm == 64 ? cl_kernel<64, 64>(a) : act_box_rows(a.M) == 16 ? cl_kernel<128, 16>(a) : cl_kernel<128, 64>(a), dim3(a.splits, a.N / a.cl_bm, (a.M + kBN - 1) / kBN),
-                 dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring);
+                 dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring | a.cl_sets << 8);
 }
 
 }  // namespace uad

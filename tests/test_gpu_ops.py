@@ -135,3 +135,22 @@ def test_linear_reads_weights_and_bias_in_stream_order(M, N, K):
     for i, out in enumerate(outs):
         want = refs[(i + 1) % 3] + lasts[i % 3]
         assert np.abs(out.cpu().numpy() - want).max() <= 1e-5 * np.abs(want).max(), i
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 4608, 1536), (16, 6144, 1536), (16, 1536, 6144), (1, 1024, 6144), (32, 1536, 6144),
+                                   (50, 1024, 4096), (64, 512, 4096), (64, 1536, 6144), (100, 1024, 4096), (13, 384, 8192)])
+def test_linear_sums_few_rows_in_short_runs(M, N, K):
+    """The tensor cores' accumulation truncates: each step of 16 products loses up to an ulp of the sum so far, half
+    of one on average. Over positive products, where the sum grows evenly, a run of 256 so loses at most
+    16 / 2 steps x 2^-24 = 4.8e-7 of it on average, and a longer run more."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + K)
+    x = torch.randn((M, K), generator=g, device="cuda").abs().bfloat16()
+    w = torch.randn((K, N), generator=g, device="cuda").mul_(0.02).abs().bfloat16()
+    tiled = torch.from_numpy(uad.tile_weight(w.float().cpu().numpy()).view(np.int16)).cuda()
+    out = torch.empty((M, N), device="cuda")
+    assert uad.uad_linear(x.data_ptr(), tiled.data_ptr(), None, out.data_ptr(), M, N, K, torch.cuda.current_stream().cuda_stream) == 0
+    ref = x.double() @ w.double()
+    mean = ((out.double() - ref) / ref).mean().abs().item()
+    print(f"{M} x {K} x {N}: mean relative error {mean:.2e}")
+    assert mean <= 8 * 2.0 ** -24
