@@ -416,7 +416,7 @@ void gemm_cl_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
   const int t64 = N / kTileM * mt, nkb = KC / a->splits, most = (KC + a->splits - 1) / a->splits;
   const auto run_of = [&](int ctas) { return (KC * t64 + ctas / 2) / ctas > 1 ? (KC * t64 + ctas / 2) / ctas : 1; };
   const int run = run_of(sms) <= 4 ? run_of(sms) : run_of(2 * sms) > 4 ? run_of(2 * sms) : 4;
-  a->cl_sets = most <= run || nkb < 2 ? 1 : most <= 2 * run || nkb < 4 ? 2 : 4;
+  a->sets = most <= run || nkb < 2 ? 1 : most <= 2 * run || nkb < 4 ? 2 : 4;
 }
 
 // The cluster form serves every projection of one 64-token tile, and with more tokens those with so
@@ -460,7 +460,7 @@ void launch_gemm_cl(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s)
   int ring = per < kClMaxStages ? per : kClMaxStages;
   while (gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm) > kClSmem) --ring;   // three slots at least
   launch_cluster(a.cl_bm == 64 ? cl_kernel<64, 64>(a) : act_box_rows(a.M) == 16 ? cl_kernel<128, 16>(a) : cl_kernel<128, 64>(a), dim3(a.splits, a.N / a.cl_bm, (a.M + kBN - 1) / kBN),
-                 dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring | a.cl_sets << 8);
+                 dim3(kThreads), gemm_cl_smem_bytes(ring, rows, a.splits, a.cl_bm), a.splits, s, *tmx, a, ring | a.sets << 8);
 }
 
 }  // namespace uad

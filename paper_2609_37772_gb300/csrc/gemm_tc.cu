@@ -383,8 +383,10 @@ __global__ void __launch_bounds__(128, 1) gemm_tc_kernel(const __grid_constant__
 // slice q to group q % 4, each group through a staging slice of its own, so a unit's epilogue
 // overlaps the next unit's main loop. A ragged last token tile loads and multiplies only its
 // 64-token boxes. K splits (residual projections only) write planes of their own, summed by the
-// norm that follows.
-template <int TN, int STAGES>
+// norm that follows. SETS = 2: a unit's k-blocks take turns over two accumulators (all 512 columns of tensor
+// memory with the double buffering), added in fp32 when they are read out, so that the tensor cores'
+// truncating accumulation runs over half as many products.
+template <int TN, int STAGES, int SETS>
 __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                        TcGemmArgs p) {
   constexpr int kStageBw = TN * kBK * 2;
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(2 * TN));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)), "r"(2 * TN * SETS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
@@ -468,13 +470,14 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
         const int b = j & 1;
         if (j >= 2 && !mbar_wait(tempty + b, ((j >> 1) - 1) & 1, p.err, 63)) break;
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(b * TN);
+        const uint32_t d = tmem + (uint32_t)(b * TN * SETS);
         for (int kb = k0; kb < k1; ++kb, ++it) {
           const int st = it % STAGES, round = it / STAGES;
           if (!mbar_wait(full + st, round & 1, p.err, 64)) { ok = false; break; }
           tc_fence_after();
-          mma_kblock(d, adesc + (uint64_t)(st * (kStageA >> 4)), bdesc + (uint64_t)(st * (kStageBw >> 4)), idesc,
-                     kb > k0 ? 1u : 0u);
+          const uint32_t set = SETS == 1 ? 0 : (uint32_t)((kb - k0) % SETS * TN);
+          mma_kblock(d + set, adesc + (uint64_t)(st * (kStageA >> 4)), bdesc + (uint64_t)(st * (kStageBw >> 4)), idesc,
+                     kb > k0 + SETS - 1 ? 1u : 0u);
           mma_commit(empty + st);
         }
         if (ok) mma_commit(tfull + b);
@@ -504,13 +507,16 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
         tc_fence_before();
         mbar_arrive(tempty + b);
       }
-      const uint32_t tb = tmem_base_after_wait(tmem_slot) + (uint32_t)(b * TN) + ((uint32_t)(q4 * 32) << 16);
+      const uint32_t tb = tmem_base_after_wait(tmem_slot) + (uint32_t)(b * TN * SETS) + ((uint32_t)(q4 * 32) << 16);
       const int n = nt * kBM + row;
       for (int q = g; q < nsl; q += kPersGroups) {
         const int m0 = mt * tn + q * kPersSlice;
         const int mcount = p.M - m0 < kPersSlice ? p.M - m0 : kPersSlice;
         float v[kPersSlice];
-        tmem_ld16(tb + q * kPersSlice, v);
+        bool sum = false;
+        if constexpr (SETS == 2) sum = (sp + 1 < S ? per : KC - sp * per) > 1;   // k-blocks for both accumulators
+        if (sum) tmem_sum16(tb + q * kPersSlice, tb + TN + q * kPersSlice, v);
+        else tmem_ld16(tb + q * kPersSlice, v);
         if (q == mylast) {
           // the group's share of the accumulator is in registers: hand it back
           tc_fence_before();
@@ -534,7 +540,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) gemm_tc_pers_kernel(const __g
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(2 * TN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(2 * TN * SETS));
   }
 }
 
@@ -611,8 +617,9 @@ int gemm_tc_prepare() {
   return once.run(dev, [] {
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (gemm_cl_prepare() ||
-        cudaFuncSetAttribute(gemm_tc_pers_kernel<256, kPersStages256>, at, (int)gemm_tc_pers_smem_bytes(256)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128>, at, (int)gemm_tc_pers_smem_bytes(128)) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_tc_pers_kernel<256, kPersStages256, 1>, at, (int)gemm_tc_pers_smem_bytes(256)) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128, 1>, at, (int)gemm_tc_pers_smem_bytes(128)) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_tc_pers_kernel<128, kPersStages128, 2>, at, (int)gemm_tc_pers_smem_bytes(128)) != cudaSuccess ||
         cudaFuncSetAttribute(gemm_tc_kernel, at, (int)gemm_tc_smem_bytes(kTcMaxStages)) != cudaSuccess)
       return -1;
     return 0;
@@ -636,21 +643,24 @@ int gemm_tc_use_wide(int M, int N, int sms) {
 // Per evaluation, N = 1024, 18 layers: 180 tokens 852 -> 842 us, 250 tokens 1053 -> 968, 400 tokens 1288 -> 1183;
 // N = 1536, 16 layers: 128 tokens 1368 -> 1378, 192 tokens 1820 -> 1795, 256 tokens 1850 -> 1761, 320 tokens
 // 1886 -> 2005, 480 tokens 2556 -> 2450. Narrower ones stay: N = 512, 250 tokens 102 -> 109.
+// They have fewer splits than the narrow form's planes had, so a tile of 128 tokens sums its k-blocks in two
+// accumulators (SETS): the longest run is no longer than there (180 tokens, N = 1024, K = 2048 and 4096: error 4.7e-7 ->
+// 2.3e-7, positive products 8.4e-7 -> 3.6e-7; 6.4 -> 6.5 and 6.5 -> 6.6 us).
 int gemm_tc_resid_wide(int M, int N, int sms) {
   return gemm_tc_use_wide(M, N, sms) || (M > 128 && N >= 1024 && N <= 2048);
 }
 
-// The persistent form's plan: tokens per tile (256, 192 or 128) and, for partial-plane
+// The persistent form's plan: tokens per tile (256, 192 or 128, at most most_tn) and, for partial-plane
 // epilogues, K splits. Units go to the CTAs round robin; the plan minimises the busiest CTA's
 // work, counted in k-blocks of a 256-token tile: a k-block of nb 64-token boxes costs half by
 // its MMA time (nb / 4) and half by its bytes ((2 + nb) / 6, weights 16 KB + 8 KB a box), plus
 // half a k-block per unit and, per extra plane, the cost of writing and reading it once more.
-void gemm_tc_pers_plan(int M, int N, int K, int sms, int epi, int* tn, int* splits) {
+void gemm_tc_pers_plan(int M, int N, int K, int sms, int epi, int most_tn, int* tn, int* splits) {
   const int KC = K / kBK, n_nt = N / kBM;
   double best = 1e30;
-  *tn = 256;
+  *tn = most_tn;
   *splits = 1;
-  for (int t = 256; t >= 128; t -= 64) {
+  for (int t = most_tn; t >= 128; t -= 64) {
     const int n_mt = (M + t - 1) / t;
     const int smax = epi == EPI_PARTIAL ? 8 : 1;
     for (int sp = 1; sp <= smax && sp <= KC; ++sp) {
@@ -686,18 +696,19 @@ void gemm_tc_plan(int M, int N, int K, int sms, int epi, TcGemmArgs* a) {
   a->tn = 0;
   a->splits = 1;
   a->cl = 0;
+  a->sets = a->wide && !gemm_tc_use_wide(M, N, sms) ? 2 : 1;
   // a long K over so few tiles that each would walk it alone: the cluster form's K splits (637 rows, N = 1024,
   // K = 4096: 21.2 -> 14.9 us; K = 2048, 800 rows: 13.0 -> 12.5). The residual projections split K anyway.
   const bool alone = a->wide && epi != EPI_PARTIAL && K >= 2048 && (N / kBM) * ((M + kBN - 1) / kBN) <= sms;
   if (alone) a->wide = 0;
   if (a->wide) {
     // the plan search walks every unit: remember its answers
-    thread_local std::map<std::array<int, 5>, std::pair<int, int>> memo;
-    const std::array<int, 5> key{M, N, K, sms, epi == EPI_PARTIAL};
+    thread_local std::map<std::array<int, 6>, std::pair<int, int>> memo;
+    const std::array<int, 6> key{M, N, K, sms, epi == EPI_PARTIAL, a->sets};
     auto it = memo.find(key);
     if (it == memo.end()) {
       std::pair<int, int> v;
-      gemm_tc_pers_plan(M, N, K, sms, epi, &v.first, &v.second);
+      gemm_tc_pers_plan(M, N, K, sms, epi, a->sets == 2 ? 128 : 256, &v.first, &v.second);
       it = memo.emplace(key, v).first;
     }
     a->tn = it->second.first;
@@ -717,7 +728,7 @@ void gemm_tc_prefix_plan(int M, int N, int K, int sms, TcGemmArgs* a) {
   a->cl = !a->wide;
   a->splits = 1;
   a->tn = 0;
-  if (a->wide) gemm_tc_pers_plan(M, N, K, sms, EPI_PREFIX_KV, &a->tn, &a->splits);
+  if (a->wide) gemm_tc_pers_plan(M, N, K, sms, EPI_PREFIX_KV, 256, &a->tn, &a->splits);
 }
 
 void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s) {
@@ -728,10 +739,13 @@ void launch_gemm_tc(const CUtensorMap* tmx, const TcGemmArgs& a, cudaStream_t s)
     const int units = (a.N / kBM) * ((a.M + a.tn - 1) / a.tn) * a.splits;
     const dim3 grid(units < sms ? units : sms);
     if (a.tn > 128)
-      launch_k(gemm_tc_pers_kernel<256, kPersStages256>, grid, dim3(kPersThreads), gemm_tc_pers_smem_bytes(256), s,
+      launch_k(gemm_tc_pers_kernel<256, kPersStages256, 1>, grid, dim3(kPersThreads), gemm_tc_pers_smem_bytes(256), s,
+               *tmx, a);
+    else if (a.sets == 2)
+      launch_k(gemm_tc_pers_kernel<128, kPersStages128, 2>, grid, dim3(kPersThreads), gemm_tc_pers_smem_bytes(128), s,
                *tmx, a);
     else
-      launch_k(gemm_tc_pers_kernel<128, kPersStages128>, grid, dim3(kPersThreads), gemm_tc_pers_smem_bytes(128), s,
+      launch_k(gemm_tc_pers_kernel<128, kPersStages128, 1>, grid, dim3(kPersThreads), gemm_tc_pers_smem_bytes(128), s,
                *tmx, a);
     return;
   }

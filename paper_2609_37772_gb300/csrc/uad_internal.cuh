@@ -223,7 +223,8 @@ struct TcGemmArgs {
                                    // tn tokens x 128 weight rows x a K range), 0: narrow tiles, no K splits
   int cl = 0;                      // 1: the few-token form, K splits over a cluster (gemm_cl.cu)
   int cl_bm = 128;                 //    weight rows of a tile: 128 or 64
-  int cl_sets = 1;                 //    accumulators that a CTA's k-blocks take turns over: 1, 2 or 4
+  int sets = 1;                    // accumulators that a tile's k-blocks take turns over: 1, 2 or 4 (few-token form), 1
+                                   // or 2 (persistent form, with tiles of 128 tokens)
   int cl_code = 0;                 //    which projections share its code: kClAny, kClPlain or kClOwn
   int tn = 0;                      // persistent form: tokens per tile (256, 192 or 128)
 };
