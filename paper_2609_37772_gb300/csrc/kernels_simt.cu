@@ -440,7 +440,10 @@ void launch_norm(const NormArgs& a, cudaStream_t s) {
 // partial rows by log-sum-exp, received through distributed shared memory. Per tile: Q K^T on the tensor
 // cores (m16n8k16: the products of bf16 operands are exact, sums in fp32), warp = 8 keys, operands
 // straight from global memory; softmax in fp32; P V on the tensor cores with every fp32 probability
-// as the sum of three bf16 terms (24 bits: nothing is rounded away), warp = 8 head dims.
+// as the sum of three bf16 terms (24 bits: nothing is rounded away), warp = 8 head dims. The tensor cores'
+// accumulation truncates, so none runs long: a score is two sums of 32 products, a tile's P V one of the leading
+// terms and one of the others, added to O in fp32 (error against 64 bits, 320 keys: 8.4e-8, scores 4.7e-8; fp32
+// FMA chains 3.2e-7 and 5.1e-8; one accumulator over all tiles 1.1e-6, one a score 6.5e-8).
 // What bounds it is latency, half of it instruction fetch: a kernel whose code is not in the SM's
 // instruction cache runs at a dozen cycles an instruction. The prefix keys and values, which no
 // kernel of the loop writes, are loaded before the wait for the previous kernel, and a rehearsal pass
@@ -551,9 +554,11 @@ __global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
       *reinterpret_cast<uint4*>(sm.v + vj * kFewPitch + vcol) = vn[0];
       *reinterpret_cast<uint4*>(sm.v + vj * kFewPitch + vcol + 8) = vn[1];
       if (pass && t + C < nt) fetch(t + C);
-      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      float c[4] = {0.f, 0.f, 0.f, 0.f}, d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) mma16816(c, qf[ks], kf + 2 * ks);
+      for (int ks = 0; ks < 4; ++ks) mma16816(ks & 1 ? d : c, qf[ks], kf + 2 * ks);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) c[e] += d[e];
       float* sr = sm.s + gr * kFewSPitch + 8 * warp + tc;
       *reinterpret_cast<float2*>(sr) = make_float2(c[0] * p.scale, c[1] * p.scale);
       *reinterpret_cast<float2*>(sr + 8 * kFewSPitch) = make_float2(c[2] * p.scale, c[3] * p.scale);
@@ -597,10 +602,7 @@ __global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
       }
       __syncthreads();
       const float a0 = sm.alpha[gr], a1 = sm.alpha[gr + 8];
-      o[0] *= a0;
-      o[1] *= a0;
-      o[2] *= a1;
-      o[3] *= a1;
+      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};   // of the leading terms, of the others
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         uint32_t vf[4];
@@ -611,9 +613,13 @@ __global__ void __launch_bounds__(256) attn_few_kernel(AttnArgs p, int C) {
           for (int k = 0; k < 3; ++k) {
             uint32_t pf[4];
             ldsm4(pf, sm.p[k] + (lane & 15) * kFewPitch + 32 * half + 16 * k2 + 8 * (lane >> 4));
-            mma16816(o, pf, vf + 2 * k2);
+            mma16816(k ? lo : hi, pf, vf + 2 * k2);
           }
       }
+      o[0] = fmaf(o[0], a0, hi[0] + lo[0]);
+      o[1] = fmaf(o[1], a0, hi[1] + lo[1]);
+      o[2] = fmaf(o[2], a1, hi[2] + lo[2]);
+      o[3] = fmaf(o[3], a1, hi[3] + lo[3]);
       if (!pass) break;
       __syncthreads();   // the next tile's values, scores and probabilities overwrite this one's
     }
