@@ -62,13 +62,13 @@ __global__ void __launch_bounds__(256) gemv_rows_kernel(GemmArgs p) {
   }
 }
 
-// Short K (at most 64): a thread keeps the weights of one output in registers, read before the wait for
+// Short K (at most kShortK): a thread keeps the weights of one output in registers, read before the wait for
 // the kernel that writes A, and a CTA of 256 outputs walks `rows` token rows staged in shared memory.
 // Bound by the bytes out; one CTA a row re-read every weight for each row (3200 rows of 1024 outputs, K = 32, with
 // the launch around it: 22 us as CUDA-core tiles of 64 x 64, 41 as their successor's, 19 here).
 template <int AD, int WD>
 __global__ void __launch_bounds__(256) short_k_kernel(GemmArgs p, int rows) {
-  constexpr int KM = 64, RM = 16;
+  constexpr int KM = kShortK, RM = 16;
   __shared__ float a_s[RM * KM];
   const int n = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * rows, K = p.K;
   const int cnt = p.M - m0 < rows ? p.M - m0 : rows;
@@ -124,12 +124,12 @@ __global__ void __launch_bounds__(256) short_k_kernel(GemmArgs p, int rows) {
 }
 
 bool gemv_rows_ok(const GemmArgs& a) {
-  return a.epi == EPI_STORE && a.out_dtype == F32 && a.K <= kGemvMaxK && (a.N <= 64 || a.K <= 64);
+  return a.epi == EPI_STORE && a.out_dtype == F32 && a.K <= kGemvMaxK && (a.N <= 64 || a.K <= kShortK);
 }
 
 template <int AD, int WD>
 static void launch_gemv(const GemmArgs& a, cudaStream_t s) {
-  if (a.K > 64) {
+  if (a.K > kShortK) {
     launch_k(gemv_rows_kernel<AD, WD>, dim3(a.M), dim3(256), 0, s, a);
     return;
   }

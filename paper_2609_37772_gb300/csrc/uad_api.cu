@@ -301,7 +301,9 @@ int validate_arch(const uad_arch& a, std::string& why) {
   if (a.n_heads < 1 || a.n_kv_heads < 1 || a.n_heads % a.n_kv_heads) return bad("heads");
   if (a.head_dim != 64 && a.head_dim != 128 && a.head_dim != 256) return bad("head_dim in {64,128,256}");
   if (a.mlp_dim < 1 || a.mlp_dim > 65536) return bad("mlp_dim");
-  if (a.action_dim < 1 || a.action_dim > 64) return bad("action_dim in 1..64");
+  // no more: the action-in projection has to be the kernel that starts a step (kShortK)
+  static_assert(kShortK == 64, "action_dim in 1..64");
+  if (a.action_dim < 1 || a.action_dim > kShortK) return bad("action_dim in 1..64");
   if (a.chunk_len < 1 || a.chunk_len > 256) return bad("chunk_len in 1..256");
   if (a.prefix_len < 0 || a.prefix_len > 16384) return bad("prefix_len");
   if (a.max_batch < 1 || a.max_batch > 1024) return bad("max_batch");

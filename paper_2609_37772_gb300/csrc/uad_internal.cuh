@@ -12,10 +12,16 @@ constexpr int kFlagStride = kMaxSteps + 1;  // host flag slots per robot (steps 
 
 enum DType { F32 = 0, BF16 = 1 };
 
-// Programmatic dependent launch. Kernels of the step loop are launched so that the next kernel's
-// CTAs may start while the previous kernel drains; every kernel calls pdl_trigger() once it has
-// started and pdl_wait() before it reads anything a predecessor wrote or writes anything a
-// predecessor reads (pdl_wait returns at once for a kernel launched without the attribute).
+// Programmatic dependent launch. Kernels of the step loop are launched so that the next kernel's CTAs may start
+// while the previous kernel drains. Every kernel calls pdl_trigger() once it has started, and pdl_wait() before
+// it reads anything a predecessor wrote or writes anything a predecessor reads (pdl_wait returns at once for a
+// kernel launched without the attribute). Two exceptions, which hold each other up:
+//  - What does not change while a chunk runs (an expert's weights and biases, the time table, RoPE, prefix keys and
+//    values) and the step's modulation rows (EulerArgs::cur_tau, through L2) are read before the wait.
+//  - The step's first kernel, the action-in projection, triggers only after its wait for the step epilogue (the
+//    chunk's first kernel) that wrote those rows, so that no kernel after it starts before they are there. That
+//    kernel is short_k_kernel, which serves up to kShortK action dims: the most that uad_init takes.
+constexpr int kShortK = 64;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 bool pdl_enabled();   // UAD_PDL=0 turns it off (debugging)
@@ -172,7 +178,7 @@ struct EulerArgs {
 
 // kernels_simt.cu
 constexpr int kGemvMaxK = 8192;
-bool gemv_rows_ok(const GemmArgs& a);                     // tiny-side projection (N or K <= 64)
+bool gemv_rows_ok(const GemmArgs& a);                     // tiny-side projection (N <= 64 or K <= kShortK)
 void launch_gemv_rows(const GemmArgs& a, cudaStream_t s);
 void launch_norm(const NormArgs& a, cudaStream_t s);   // applies the pending residual if part != null
 void launch_attention(const AttnArgs& a, cudaStream_t s);
