@@ -730,24 +730,30 @@ def test_dit_attention_tiles_and_clusters(chunk, prefix, robots):
 
 
 @pytest.mark.parametrize("name,robots", [("dit_small", 2), ("tiny", 1), ("pi0_small", 3)])
-def test_step_graphs_of_changing_step_counts(name, robots):
-    """Chunks of different step counts one after the other on one context, whose graphs hold a divisor
-    of the steps each (one step at 7, 11 and 13): each chunk bit for bit what a fresh context gives."""
+def test_step_graphs_of_changing_step_counts(name, robots, monkeypatch):
+    """Chunks of different step counts one after the other on one context. A graph holds the most steps that divide
+    the chunk's and stay within 256 launches: with 18 to 26 launches a step, one at 17, five at 15, eight or four at
+    16, the whole chunk at 7 and less, where the first kernel joins it. Each chunk bit for bit what the same
+    kernels give without graphs, the split ones also against the oracle."""
     a = ARCHS[name]
     noise = make_noise(a, batch=robots, seed=55)
     blob = make_weights(a, seed=55)
     c = Case(a, B=robots, seed=55, blob=blob)
+    monkeypatch.setenv("UAD_GRAPHS", "0")
+    plain = Case(a, B=robots, seed=55, blob=blob)
     try:
-        for n in (7, 2, 13, 12, 1, 7, 11):
+        per_step = (c.ex.launches_per_chunk(robots, 10) - 1) // 10
+        assert 17 * per_step > 256 and 7 * per_step <= 256, per_step
+        for n in (7, 2, 17, 16, 1, 15, 7, 17):
             bud = np.stack([group_budgets(a.chunk_len, [(0, 2, (n + 1) // 2), (3, a.chunk_len - 1, n)])] * robots)
-            res = c.gpu(noise, bud)
-            fresh = Case(a, B=robots, seed=55, blob=blob)
-            ref = fresh.gpu(noise, bud)
-            fresh.close()
+            res, ref = c.gpu(noise, bud), plain.gpu(noise, bud)
             assert res["evals"] == ref["evals"] == n
             assert np.array_equal(res["final"], ref["final"]) and np.array_equal(res["ghost"], ref["ghost"])
+            if n > 7:
+                check(c, res, c.oracle(noise, bud), bud, TOL[a.dtype])
     finally:
         c.close()
+        plain.close()
 
 
 @pytest.mark.parametrize("name,chunk,robots", [("pi0", 32, 4), ("pi0", 43, 3), ("pi0", 50, 5), ("dit", 16, 9), ("dit", 13, 20)])
