@@ -171,6 +171,23 @@ __device__ __forceinline__ void tile_epilogue(const TcGemmArgs& p, const float* 
       }
       break;
     }
+    case EPI_PREFIX_KV: {
+      // Not reached as things are (the persistent form writes these rows from registers, few tokens take the cluster
+      // form), but without this case the compiler lays the others out so that the 18-layer expert is slower: 16 / 64
+      // robots 1392 / 2901 us per evaluation with it, 1409 / 2922 without, 1408 / 2910 with the QKV case first or last.
+      // one layer's k or v rows: tokens over the warps, lane owns 4 consecutive features, so that a
+      // warp writes a token's 128 features as one contiguous run
+      const int n0 = n - row, w = p.pkv.width, part = n0 / w;   // part = 2 layer + (0 k, 1 v)
+      __nv_bfloat16* dst = ((part & 1) ? p.pkv.v : p.pkv.k) + (size_t)(part >> 1) * p.M * w + (n0 - part * w) + 4 * lane;
+      for (int j = row >> 5; j < mcount; j += kBM / 32) {
+        const float4 v = *reinterpret_cast<const float4*>(T + j * pitch + 4 * lane);
+        uint2 pk;
+        pk.x = ptx::pack_bf16(v.x, v.y);
+        pk.y = ptx::pack_bf16(v.z, v.w);
+        *reinterpret_cast<uint2*>(dst + (size_t)(m0 + j) * w) = pk;
+      }
+      break;
+    }
     default:
       if (p.n_store > 0 && n >= p.n_store) break;   // padding rows of a narrow projection
 #pragma unroll 4
