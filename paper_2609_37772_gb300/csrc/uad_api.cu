@@ -574,8 +574,8 @@ const char* step_unfit(uad_ctx* c, int* ring) {
   for (auto& sh : shapes)
     if (sh[0] % 128 || sh[1] % 64) return "projection shape";
   // Large experts run faster as per-operation kernels (pi0-like, one robot, per evaluation: 706 us against 762;
-  // with 2 of its 18 layers 90 against 105). So do small ones (2 layers of width 512: 73 against 86), but those
-  // keep the one launch per evaluation that uad_launches_per_chunk promises them.
+  // with 2 of its 18 layers 90 against 105). So do small ones (2 layers of width 512: 73 against 86), which stay on
+  // this kernel all the same: callers count on its one launch per evaluation (uad_launches_per_chunk).
   const double layer = 2.0 * ((double)c->qkvd * W + (double)W * c->qd + 3.0 * F * W);
   if (a.n_layers * layer > 32e6) return "large expert";
   const int most = step_max_tiles(c->sms, shapes, 4);
