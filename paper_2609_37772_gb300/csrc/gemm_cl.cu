@@ -8,9 +8,10 @@
 // the S partial rows of its tokens in rank order (the result does not depend on timing) and applies
 // the epilogue to them. The receive area lies apart from the operand ring, so that rows arrive while other
 // CTAs' MMAs still run (aliased on the ring: DiT head 916 us per evaluation, apart 840; four robots 1246 and
-// 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. An expert's weights are requested before the wait for the
-// kernel that produces the activations (a caller's after it: TcGemmArgs::ordered). Every wait is bounded; the cluster barriers are reached on every path, and no CTA
-// leaves with copies in flight into its shared memory.
+// 1214). The exchange is slow (10-13 B a cycle and SM): it pays while a CTA's share is a few KB. An expert's
+// weights are requested before the wait for the kernel that produces the activations (a caller's after it:
+// TcGemmArgs::ordered). Every wait is bounded; the cluster barriers are reached on every path, and no CTA leaves with
+// copies in flight into its shared memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

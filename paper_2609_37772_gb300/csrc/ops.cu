@@ -38,7 +38,6 @@ int check_linear_args(const void* x, const void* w, const float* out, int32_t M,
 
 namespace uad {
 
-constexpr int kErrWords = 1024;
 int static_err_words(int** err, bool look_up);   // ops_static.cu
 
 // Shared by uad_linear and its static variant: launch the projection kernel with
@@ -120,13 +119,13 @@ int uad_linear_status(void) {
     if (dev < (int)g_err.size()) words[0] = g_err[dev];
   }
   static_err_words(&words[1], false);
-  std::vector<int> codes(kErrWords);
   bool ran_out = false;
   for (int* w : words) {
     if (!w) continue;
-    if (cudaMemcpy(codes.data(), w, kErrWords * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return UAD_ECUDA;
-    const bool any = std::any_of(codes.begin(), codes.end(), [](int c) { return c != 0; });
-    if (any && cudaMemset(w, 0, kErrWords * 4) != cudaSuccess) return UAD_ECUDA;
+    int codes[kErrWords];
+    if (cudaMemcpy(codes, w, sizeof(codes), cudaMemcpyDeviceToHost) != cudaSuccess) return UAD_ECUDA;
+    const bool any = std::any_of(codes, codes + kErrWords, [](int c) { return c != 0; });
+    if (any && cudaMemset(w, 0, sizeof(codes)) != cudaSuccess) return UAD_ECUDA;
     ran_out |= any;
   }
   return ran_out ? UAD_ECUDA : UAD_OK;

@@ -15,7 +15,6 @@
 namespace uad {
 int launch_linear(const void* x, const void* w_tiled, const float* bias, float* out, int M, int N, int K, int* err,
                   bool stopped, cudaStream_t s);
-constexpr int kErrWords = 1024;
 int linear_tiles(int M, int N);
 int static_err_words(int** err, bool look_up);
 }  // namespace uad

@@ -205,6 +205,7 @@ void launch_gemm_table(const GemmArgs& a, cudaStream_t s);   // fp32 activations
 void launch_attn_rows(const AttnArgs& a, cudaStream_t s);
 void ffma_prepare(int head_dim);   // opt in to > 48 KB dynamic shared memory on the current device
 
+constexpr int kErrWords = 1024;        // error words of the projection op, one a call in turn (ops.cu, ops_static.cu)
 // gemm_tc.cu: tcgen05 projection GEMM (bf16 operands, fp32 accumulation in TMEM)
 constexpr int kTcMaxStages = 4;        // <= ~97 KB of shared memory: two CTAs fit one SM
 struct TcGemmArgs {
